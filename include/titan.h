@@ -261,7 +261,7 @@ titan_status titan_read_state_dev(titan_sim *sim, float *pos_dev, float *vel_dev
  * Group g is the masses with caller indices first_dev[g] .. first_dev[g+1] - 1
  * (first_dev: DEVICE uint32 array of n_groups + 1 non-decreasing offsets, the
  * last at most n_masses).  out_dev[g][0..2] (DEVICE float) = the mean
- * position of the group, summed in FP64 mass by mass, minus origin_dev[g][..]
+ * position of the group, summed in FP64 in a fixed order, minus origin_dev[g][..]
  * when origin_dev (DEVICE float [n_groups][3]) is non-NULL; an empty group
  * gives 0.  Enqueued on the simulation stream.  Offsets are not read on the
  * host: out-of-range ones are clamped to n_masses.  Errors: TITAN_E_INVALID

@@ -30,6 +30,7 @@
 #include <string>
 #include <vector>
 
+#include "group_mean.cuh"
 #include "layout.h"
 #include "physics.cuh"
 #include "ptx.cuh"
@@ -232,20 +233,14 @@ k_batch_rollout(const BatchCta *__restrict__ ctas, const MassState *__restrict__
         }
 }
 
-// Per-robot centroid x, y, z (fixed summation order: mass by mass).
-__global__ void k_batch_centroid(const uint32_t *__restrict__ mass_off, const uint32_t *__restrict__ mass_cnt,
-                                 const MassState *__restrict__ state, uint32_t n_robots, float *__restrict__ out) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_robots) return;
-    double sx = 0, sy = 0, sz = 0;
-    const uint32_t o = mass_off[r], n = mass_cnt[r];
-    for (uint32_t m = 0; m < n; ++m) {
-        const float4 p = state[o + m].p;
-        sx += p.x; sy += p.y; sz += p.z;
-    }
-    out[3 * r] = (float)(sx / n);
-    out[3 * r + 1] = (float)(sy / n);
-    out[3 * r + 2] = (float)(sz / n);
+// Per-robot centroid x, y, z.  A block per robot; see group_mean.
+__global__ void __launch_bounds__(titan::kMeanThreads)
+k_batch_centroid(const uint32_t *__restrict__ mass_off, const uint32_t *__restrict__ mass_cnt,
+                 const MassState *__restrict__ state, float *__restrict__ out) {
+    const uint32_t r = blockIdx.x, o = mass_off[r];
+    double m[3];
+    titan::group_mean(mass_cnt[r], [&](uint32_t i) { return state[o + i].p; }, m);
+    if (threadIdx.x < 3) out[3 * (size_t)r + threadIdx.x] = (float)m[threadIdx.x];
 }
 
 struct Group {
@@ -623,8 +618,8 @@ titan_status titan_batch_read(titan_batch *b, uint32_t system, float *pos, float
 titan_status titan_batch_centroids(titan_batch *b, float *out) {
     if (!b || !out) return bfail(b, TITAN_E_INVALID, "batch or out is null");
     if (!b->n_robots) return TITAN_OK;
-    k_batch_centroid<<<(b->n_robots + 127) / 128, 128, 0, b->stream>>>(b->d_moff, b->d_mcnt, b->d_state[b->cur],
-                                                                       b->n_robots, b->d_centroid);
+    k_batch_centroid<<<b->n_robots, titan::kMeanThreads, 0, b->stream>>>(b->d_moff, b->d_mcnt, b->d_state[b->cur],
+                                                                          b->d_centroid);
     BATCH_CK(b, cudaGetLastError());
     titan_status st = titan_batch_sync(b);
     if (st != TITAN_OK) return st;

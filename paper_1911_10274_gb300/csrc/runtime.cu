@@ -18,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "group_mean.cuh"
 #include "layout.h"
 #include "sim_internal.h"
 #include "titan.h"
@@ -290,25 +291,19 @@ bool uses_cube(const titan_sim *sim) { return sim->csr_kernel == 8; }
 
 // Uploads the per-entry actuation arrays of the current layout.
 // Mean position of each group of masses (caller indices first[g] ..
-// first[g+1] - 1, clamped to n), summed in FP64 in caller order, minus the
-// group's origin if given (an empty group: 0); one thread per group.
-__global__ void k_group_centroid(const MassState *__restrict__ state, const uint32_t *__restrict__ dev_of_caller,
-                                 uint32_t n, const uint32_t *__restrict__ first, uint32_t n_groups,
-                                 const float *__restrict__ origin, float *__restrict__ out) {
-    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_groups) return;
+// first[g+1] - 1, clamped to n), minus the group's origin if given (an empty
+// group: 0).  A block per group; see group_mean.
+__global__ void __launch_bounds__(titan::kMeanThreads)
+k_group_centroid(const MassState *__restrict__ state, const uint32_t *__restrict__ dev_of_caller, uint32_t n,
+                 const uint32_t *__restrict__ first, const float *__restrict__ origin, float *__restrict__ out) {
+    const uint32_t g = blockIdx.x;
     const uint32_t i0 = min(first[g], n), i1 = max(i0, min(first[g + 1], n));
-    double sx = 0, sy = 0, sz = 0;
-    for (uint32_t i = i0; i < i1; ++i) {
-        const float4 p = state[dev_of_caller[i]].p;
-        sx += p.x; sy += p.y; sz += p.z;
+    double m[3];
+    titan::group_mean(i1 - i0, [&](uint32_t i) { return state[dev_of_caller[i0 + i]].p; }, m);
+    if (threadIdx.x < 3) {
+        const float o = origin && i1 > i0 ? origin[3 * (size_t)g + threadIdx.x] : 0.f;
+        out[3 * (size_t)g + threadIdx.x] = (float)(m[threadIdx.x] - (double)o);
     }
-    const double c = i1 > i0 ? 1.0 / (double)(i1 - i0) : 0.0;
-    float o[3] = {0.f, 0.f, 0.f};
-    if (origin && i1 > i0) { o[0] = origin[3 * g]; o[1] = origin[3 * g + 1]; o[2] = origin[3 * g + 2]; }
-    out[3 * g] = (float)(sx * c - (double)o[0]);
-    out[3 * g + 1] = (float)(sy * c - (double)o[1]);
-    out[3 * g + 2] = (float)(sz * c - (double)o[2]);
 }
 
 // seed[i][axis] = w[g] / |group g| for the masses of group g; a warp per group.
@@ -1223,9 +1218,8 @@ titan_status titan_group_centroids(titan_sim *sim, uint32_t n_groups, const uint
         titan_status es_ = titan::ensure_layout(sim);
         if (es_ != TITAN_OK) return es_;
     }
-    k_group_centroid<<<(n_groups + 127) / 128, 128, 0, sim->stream>>>(sim->state[sim->cur], sim->d_dev_of_caller,
-                                                                       sim->n, first_dev, n_groups, origin_dev,
-                                                                       out_dev);
+    k_group_centroid<<<n_groups, titan::kMeanThreads, 0, sim->stream>>>(sim->state[sim->cur], sim->d_dev_of_caller,
+                                                                         sim->n, first_dev, origin_dev, out_dev);
     TITAN_CK(sim, cudaGetLastError());
     return TITAN_OK;
 }
