@@ -187,8 +187,61 @@ __device__ __forceinline__ void prefetch_slice(const uint32_t *slice_off, uint32
     if (HAS_ACT) ptx::bulk_prefetch_l2(act + e0, ne * 8);
 }
 
-template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP>
-__global__ void __launch_bounds__(kHaloThreads, kHaloMinBlocks)
+// Deep form of the row loop, for grids that leave the SMs mostly empty (see
+// deep_grid): COLS columns of the half-edge stream per group, two groups in
+// flight, so that a warp has up to 2 COLS columns of loads outstanding instead
+// of two, and a group's springs are evaluated side by side.  Same entries, same
+// order of the sums: the same bits.
+constexpr int kDeepMinBlocks = 2;      // resident CTAs per SM the deep form's registers are sized for
+
+template <int COLS, bool HAS_C, bool HAS_ACT>
+struct Cols {
+    uint32_t j[COLS];                  // table slot (halo) or slot offset (box) of the neighbour
+    float2 a[COLS];                    // {k, L0}
+    float c[HAS_C ? COLS : 1];
+    float2 s[HAS_ACT ? COLS : 1];
+};
+
+// Adds the first `left` (at least one) columns of group g to the force.
+template <int COLS, bool HAS_C, bool HAS_ACT>
+__device__ __forceinline__ void row_group(const Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t left, const float4 &p,
+                                          const float4 &v, const StepConst &c, float ph, const float4 *tA,
+                                          const float2 *tB, float &fx, float &fy, float &fz) {
+    auto term = [&](int u, float &f, float &ux, float &uy, float &uz) {
+        const float4 qa = tA[g.j[u]];
+        const float2 qb = tB[g.j[u]];
+        const float L = HAS_ACT ? actuated_length(c, g.a[u].y, g.s[HAS_ACT ? u : 0], ph) : g.a[u].y;
+        spring_terms(p, v, qa, make_float4(qa.w, qb.x, qb.y, 0.f), g.a[u].x, L, HAS_C ? g.c[HAS_C ? u : 0] : c.c_uniform,
+                     f, ux, uy, uz);
+    };
+    if (left >= COLS) {
+        float f[COLS], ux[COLS], uy[COLS], uz[COLS];
+#pragma unroll
+        for (int u = 0; u < COLS; ++u) term(u, f[u], ux[u], uy[u], uz[u]);
+#pragma unroll
+        for (int u = 0; u < COLS; ++u) {
+            fx = __fmaf_rn(f[u], ux[u], fx);
+            fy = __fmaf_rn(f[u], uy[u], fy);
+            fz = __fmaf_rn(f[u], uz[u], fz);
+        }
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < COLS; u += 2) {        // row widths are even
+        if ((uint32_t)u >= left) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float f, ux, uy, uz;
+            term(u + h, f, ux, uy, uz);
+            fx = __fmaf_rn(f, ux, fx);
+            fy = __fmaf_rn(f, uy, fy);
+            fz = __fmaf_rn(f, uz, fz);
+        }
+    }
+}
+
+template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP, int COLS>
+__global__ void __launch_bounds__(kHaloThreads, COLS > 2 ? kDeepMinBlocks : kHaloMinBlocks)
 k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n,
             const uint32_t *__restrict__ slice_off, const uint16_t *__restrict__ nslot,
             const float2 *__restrict__ kl, const float *__restrict__ cc,
@@ -206,7 +259,7 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
     if (OVERLAP) ptx::grid_dep_launch();    // the next step's CTAs may take SM slots this tail frees
     const bool valid = i < n;
 
-    if (lane == 0) {
+    if (COLS == 2 && lane == 0) {
         if (b < ahead || ahead == 0) {
             if (sl < n_slices) prefetch_slice<HAS_C, HAS_ACT>(slice_off, sl, nslot, kl, cc, act);
         }
@@ -218,6 +271,22 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
     if (valid) {
         e0 = __ldg(slice_off + sl);
         width = (__ldg(slice_off + sl + 1) - e0) >> 5;
+    }
+    Cols<COLS, HAS_C, HAS_ACT> ga, gb;      // deep form: two groups of columns in flight
+    auto fetch = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+#pragma unroll
+        for (int u = 0; u < COLS; ++u) {
+            if (t + u >= width) break;                  // warp-uniform; entries past the row are never used
+            const uint32_t e = e0 + lane + 32 * (t + u);
+            g.j[u] = __ldcs(nslot + e);
+            g.a[u] = __ldcs(kl + e);
+            if (HAS_C) g.c[u] = __ldcs(cc + e);
+            if (HAS_ACT) g.s[u] = __ldcs(act + e);
+        }
+    };
+    if (COLS > 2) {                         // layout data only: requested before the previous step is waited for
+        fetch(ga, 0);
+        fetch(gb, COLS);
     }
     // the state and the step counter are written by the previous step
     if (OVERLAP) ptx::grid_dep_wait();
@@ -243,7 +312,18 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
 
     const float ph = HAS_ACT ? actuation_clock(c, step) : 0.f;
     float fx = 0.f, fy = 0.f, fz = 0.f;
-    if (width) {
+    if (COLS > 2) {
+        auto evaluate = [&](const Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+            row_group<COLS, HAS_C, HAS_ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
+        };
+        for (uint32_t t = 0; t < width; t += 2 * COLS) {
+            evaluate(ga, t);
+            fetch(ga, t + 2 * COLS);
+            if (t + COLS >= width) break;
+            evaluate(gb, t + COLS);
+            fetch(gb, t + 3 * COLS);
+        }
+    } else if (width) {
         uint32_t e = e0 + lane;
         uint32_t n0 = __ldcs(nslot + e), n1 = __ldcs(nslot + e + 32);
         float2 na0 = __ldcs(kl + e), na1 = __ldcs(kl + e + 32);
@@ -288,8 +368,8 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
 // included, has L0 >= 0) may point at an empty cell of the box, whose table
 // slot holds whatever was there: they are skipped, never evaluated.  Holes -
 // device slots of empty cells, marked by own slot 0xFFFF - do nothing at all.
-template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP>
-__global__ void __launch_bounds__(kHaloThreads, kBoxMinBlocks)
+template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP, int COLS>
+__global__ void __launch_bounds__(kHaloThreads, COLS > 2 ? kDeepMinBlocks : kBoxMinBlocks)
 k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n,
            const uint32_t *__restrict__ slice_off, const uint32_t *__restrict__ col_off2,
            const float2 *__restrict__ kl, const float *__restrict__ cc, const float2 *__restrict__ act,
@@ -323,12 +403,32 @@ k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32
         // column counts, so a pair of int16 column offsets is one aligned word
         co = col_off2 + (e0 >> 6);
         e = e0 + lane;
-        if (width) {
+        if (COLS == 2 && width) {
             no = __ldg(co);
             na0 = __ldcs(kl + e); na1 = __ldcs(kl + e + 32);
             if (HAS_C) { nc0 = __ldcs(cc + e); nc1 = __ldcs(cc + e + 32); }
             if (HAS_ACT) { ns0 = __ldcs(act + e); ns1 = __ldcs(act + e + 32); }
         }
+    }
+    Cols<COLS, HAS_C, HAS_ACT> ga, gb;      // deep form: two groups of columns in flight
+    auto fetch = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+#pragma unroll
+        for (int u = 0; u < COLS; u += 2) {
+            if (t + u >= width) break;
+            const uint32_t o = __ldg(co + ((t + u) >> 1));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t x = e + 32 * (t + u + h);
+                g.a[u + h] = __ldcs(kl + x);
+                if (HAS_C) g.c[u + h] = __ldcs(cc + x);
+                if (HAS_ACT) g.s[u + h] = __ldcs(act + x);
+                g.j[u + h] = (uint32_t)(int32_t)(int16_t)(h ? o >> 16 : o & 0xffffu);
+            }
+        }
+    };
+    if (COLS > 2 && valid) {
+        fetch(ga, 0);
+        fetch(gb, COLS);
     }
     const uint32_t h0 = __ldg(ext_off + b), h1 = __ldg(ext_off + b + 1);
     // everything above reads layout data only; the state and the step counter
@@ -354,7 +454,21 @@ k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32
 
     const float ph = HAS_ACT ? actuation_clock(c, step) : 0.f;
     float fx = 0.f, fy = 0.f, fz = 0.f;
-    if (width) {
+    if (COLS > 2) {
+        // a padding entry is evaluated against the mass itself: exactly zero
+        auto evaluate = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+#pragma unroll
+            for (int u = 0; u < COLS; ++u) g.j[u] = g.a[u].y >= 0.f ? s_own + g.j[u] : s_own;
+            row_group<COLS, HAS_C, HAS_ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
+        };
+        for (uint32_t t = 0; t < width; t += 2 * COLS) {
+            evaluate(ga, t);
+            fetch(ga, t + 2 * COLS);
+            if (t + COLS >= width) break;
+            evaluate(gb, t + COLS);
+            fetch(gb, t + 3 * COLS);
+        }
+    } else if (width) {
         for (uint32_t t = 0; t < width; t += 2) {
             const uint32_t o = no;
             const float2 a0 = na0, a1 = na1;
@@ -1053,6 +1167,22 @@ static int carveout_for(size_t bytes, int resident) {
     return (int)std::min<size_t>(100, std::max<size_t>(50, (100 * need + (size_t)max_sm - 1) / (size_t)max_sm));
 }
 
+// Whether a grid of `blocks` CTAs takes the deep form of the halo and box
+// kernels: up to two CTAs per SM, where the two-column form leaves each warp
+// waiting for its next pair of columns and the deep form's registers cost no
+// residency.  Measured per step, three handles stepping at once (two-column ->
+// deep): 20,250-mass worm swarm 9.3 -> 4.6 us, 48,600 masses 15.6 -> 6.8, lattices
+// of 32,768 masses 3.7 -> 3.1 and 64,000 (250 CTAs) 4.9 -> 3.8, mesh of 50,000
+// points 3.5 -> 2.9; from 391 CTAs on it no longer gains (4.3 -> 4.4) and at 637
+// it loses (6.8 -> 8.8).  Groups of 4, 6 and 8 columns: 6.1, 5.8 and 8.8 us on
+// the 40,500-mass swarm (8 spill), 3.8, 4.2 and 4.3 on the 64,000-mass lattice.
+constexpr int kDeepCols = 4;
+static bool deep_grid(unsigned blocks) {
+    int dev = 0, sms = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && blocks <= 2u * (unsigned)sms;
+}
+
 // The launch attributes of a step kernel: the L2 window (optional) and
 // programmatic stream serialization (overlap).
 static unsigned step_attrs(cudaLaunchAttribute *attr, const cudaAccessPolicyWindow *l2win, bool overlap) {
@@ -1077,10 +1207,14 @@ cudaError_t launch_step_halo(const MassState *in, MassState *out, uint32_t n, co
     const bool hc = v.c != nullptr, ha = v.act != nullptr, gr = c.ground != 0;
     const unsigned g = n ? (n + kHaloThreads - 1) / kHaloThreads : 1;
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
-    const int carveout = carveout_for(bytes, kHaloMinBlocks);
+    const bool deep = deep_grid(g);
+    const int carveout = carveout_for(bytes, deep ? kDeepMinBlocks : kHaloMinBlocks);
 #define TITAN_HALO(HC, HA, GR)                                                                   \
     do {                                                                                         \
-        auto kern = overlap ? k_step_halo<HC, HA, GR, true> : k_step_halo<HC, HA, GR, false>;   \
+        auto kern = deep ? (overlap ? k_step_halo<HC, HA, GR, true, kDeepCols>                   \
+                                     : k_step_halo<HC, HA, GR, false, kDeepCols>)                 \
+                         : (overlap ? k_step_halo<HC, HA, GR, true, 2>                            \
+                                     : k_step_halo<HC, HA, GR, false, 2>);                        \
         if (bytes > 48 * 1024) {                                                                 \
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
             if (e != cudaSuccess) return e;                                                      \
@@ -1121,10 +1255,14 @@ cudaError_t launch_step_box(const MassState *in, MassState *out, uint32_t n, con
     const unsigned g = n ? (n + kHaloThreads - 1) / kHaloThreads : 1;
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
     if (reinterpret_cast<uintptr_t>(h.col_off) & 3) return cudaErrorInvalidValue;
-    const int carveout = carveout_for(bytes, kBoxMinBlocks);
+    const bool deep = deep_grid(g);
+    const int carveout = carveout_for(bytes, deep ? kDeepMinBlocks : kBoxMinBlocks);
 #define TITAN_BOX(HC, HA, GR)                                                                    \
     do {                                                                                         \
-        auto kern = overlap ? k_step_box<HC, HA, GR, true> : k_step_box<HC, HA, GR, false>;     \
+        auto kern = deep ? (overlap ? k_step_box<HC, HA, GR, true, kDeepCols>                    \
+                                     : k_step_box<HC, HA, GR, false, kDeepCols>)                  \
+                         : (overlap ? k_step_box<HC, HA, GR, true, 2>                             \
+                                     : k_step_box<HC, HA, GR, false, 2>);                         \
         if (bytes > 48 * 1024) {                                                                 \
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
             if (e != cudaSuccess) return e;                                                      \
