@@ -680,7 +680,7 @@ bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const s
 
 
 bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_springs *springs,
-                 const titan_actuation *act, BatchHost &out, std::string *why) {
+                 const titan_actuation *act, BatchHost &out, std::string *why, const BatchPlan &plan) {
     out = BatchHost();
     bool any_act = false;
     for (uint32_t r = 0; r < n_systems; ++r)
@@ -697,6 +697,7 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
     };
     std::vector<std::vector<CtaHost>> per_sys(n_systems);
     std::vector<uint32_t> cluster_of(n_systems);
+    std::vector<uint8_t> rows_of(n_systems, 0);     // planned for the row-register form
     uint32_t slot_cursor = 0;
     for (uint32_t r = 0; r < n_systems; ++r) {
         const titan_masses &m = masses[r];
@@ -728,16 +729,10 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
                 }
             return cnt;
         };
-        // smallest cluster whose per-CTA shared memory fits
-        uint32_t C = 1;
-        for (;; C *= 2) {
-            if (C > kBatchMaxCluster) {
-                if (why) *why = "system " + std::to_string(r) + " does not fit a cluster of 8 CTAs";
-                out = BatchHost();
-                return false;
-            }
+        // shared memory of the widest CTA on a cluster of C, or SIZE_MAX if its masses do not fit
+        auto smem_on = [&](uint32_t C, uint32_t most) -> size_t {
             const uint32_t per = ((m.n + C - 1) / C + 31) & ~31u;
-            if (per > kBatchMaxPerCta) continue;
+            if (per > most) return SIZE_MAX;
             // the layout of every CTA of the cluster reserves the largest halo
             uint32_t hc = 0;
             if (C > 1)
@@ -752,7 +747,24 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
                 edges = (edges + 63) & ~63u;
                 worst = std::max<size_t>(worst, batch_smem_layout(per, hc, ns, edges, any_act).total);
             }
-            if (worst <= kBatchSmemLimit && per + hc <= 65535) break;
+            return per + hc <= 65535 ? worst : SIZE_MAX;
+        };
+        // smallest cluster whose per-CTA shared memory fits
+        uint32_t C = 0;
+        if (plan.rows && *std::max_element(deg.begin(), deg.end()) <= kRowWidth)
+            for (uint32_t c : {1u, 2u, 3u, 4u, 5u, 6u, 8u})
+                if (smem_on(c, kRowSlots) <= kBatchSmemLimit) {
+                    C = c;
+                    rows_of[r] = 1;
+                    break;
+                }
+        for (uint32_t c = 1; !C; c *= 2) {
+            if (c > kBatchMaxCluster) {
+                if (why) *why = "system " + std::to_string(r) + " does not fit a cluster of 8 CTAs";
+                out = BatchHost();
+                return false;
+            }
+            if (smem_on(c, kBatchMaxPerCta) <= kBatchSmemLimit) C = c;
         }
         cluster_of[r] = C;
         const uint32_t per = ((m.n + C - 1) / C + 31) & ~31u;
@@ -840,6 +852,26 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
         uint32_t halo_slots = 0;
         for (const auto &hh : per_sys[r]) halo_slots = std::max(halo_slots, hh.d.halo_count);
         for (auto &hh : per_sys[r]) hh.d.halo_slots = halo_slots;
+        if (rows_of[r] && C > 1) {
+            // the halo lists the other way round: where each slot's mass is copied to
+            std::vector<std::vector<uint32_t>> to((size_t)C * per);
+            for (uint32_t q = 0; q < C; ++q)
+                for (uint32_t h = 0; h < (uint32_t)per_sys[r][q].halo.size(); ++h) {
+                    const uint32_t code = per_sys[r][q].halo[h];
+                    to[(size_t)(code >> 16) * per + (code & 0xffffu)].push_back(q << 16 | h);
+                }
+            out.push.resize(2 * (size_t)(slot_cursor + C * per), kNoPush);
+            for (size_t k = 0; k < to.size(); ++k) {
+                uint32_t *pc = &out.push[2 * (slot_cursor + k)];
+                if (to[k].size() > 0) pc[0] = to[k][0];
+                if (to[k].size() == 2) pc[1] = to[k][1];
+                if (to[k].size() > 2) {
+                    pc[1] = kMorePush | (uint32_t)out.push_more.size();
+                    out.push_more.push_back((uint32_t)to[k].size() - 1);
+                    out.push_more.insert(out.push_more.end(), to[k].begin() + 1, to[k].end());
+                }
+            }
+        }
         slot_cursor += C * per;
         // initial state of every slot of this system (padding slots: fixed, at rest)
         out.init_state.resize(8 * (size_t)slot_cursor, 0.f);
@@ -856,10 +888,17 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
         }
     }
     out.total_slots = slot_cursor;
+    if (!out.push.empty()) out.push.resize(2 * (size_t)slot_cursor, kNoPush);
     // launch groups by (cluster size, shared-memory class); a launch's
     // dynamic shared memory is the largest of its CTAs'
     static const uint32_t kPerSm[] = {1, 2, 3, 4, 6, 8};
     auto smem_class = [&](uint32_t r) {
+        if (rows_of[r]) {           // by the CTAs whose threads an SM's registers hold
+            uint32_t cls = 0;
+            for (uint32_t k = 0; k < sizeof(kPerSm) / sizeof(kPerSm[0]); ++k)
+                if (per_sys[r][0].d.slot_count * kPerSm[k] <= kRowSlots) cls = k;
+            return cls;
+        }
         size_t worst = 0;
         for (const auto &h : per_sys[r])
             worst = std::max<size_t>(worst, batch_smem_layout(h.d.slot_count, h.d.halo_slots, h.d.n_slices,
@@ -875,12 +914,14 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
     for (uint32_t r = 0; r < n_systems; ++r) order[r] = r;
     std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
         if (cluster_of[x] != cluster_of[y]) return cluster_of[x] > cluster_of[y];
+        if (rows_of[x] != rows_of[y]) return rows_of[x] < rows_of[y];
         if (class_of[x] != class_of[y]) return class_of[x] < class_of[y];
         return masses[x].n > masses[y].n;
     });
     for (uint32_t k = 0; k < n_systems; ++k) {
         const uint32_t r = order[k];
-        if (out.groups.empty() || out.groups.back().cluster != cluster_of[r] || class_of[order[k - 1]] != class_of[r]) {
+        if (out.groups.empty() || out.groups.back().cluster != cluster_of[r] || class_of[order[k - 1]] != class_of[r] ||
+            rows_of[order[k - 1]] != rows_of[r]) {
             BatchGroup g;
             g.cluster = cluster_of[r];
             g.cta_first = (uint32_t)out.ctas.size();
@@ -900,8 +941,12 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
             out.halo.insert(out.halo.end(), h.halo.begin(), h.halo.end());
             out.ctas.push_back(h.d);
             ++g.cta_count;
-            g.smem = std::max<size_t>(g.smem, batch_smem_layout(h.d.slot_count, h.d.halo_slots, h.d.n_slices,
-                                                                h.d.edge_count, any_act).total);
+            const BatchSmem L = batch_smem_layout(h.d.slot_count, h.d.halo_slots, h.d.n_slices, h.d.edge_count, any_act);
+            g.smem = std::max<size_t>(g.smem, L.total);
+            if (rows_of[r]) {
+                g.row_threads = std::max(g.row_threads, h.d.slot_count);
+                g.row_smem = std::max<size_t>(g.row_smem, L.inv);
+            }
         }
         per_sys[r].clear();
     }

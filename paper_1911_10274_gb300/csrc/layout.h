@@ -268,7 +268,21 @@ struct BatchGroup {
     uint32_t cluster = 1;
     uint32_t cta_first = 0, cta_count = 0;
     size_t smem = 0;
+    uint32_t row_threads = 0;            // largest slot_count if every CTA can run the row-register form, else 0
+    size_t row_smem = 0;                 // its shared memory: the two state buffers
 };
+
+// The row-register form of the batch kernel (k_batch_rows) keeps a mass's whole
+// row in its thread's registers: systems whose rows are at most kRowWidth wide
+// and whose masses fit 8 CTAs of kRowSlots take it.  4.5 registers per
+// actuated entry x 26 (the neighbours of a lattice site) and the arithmetic
+// need 168 registers a thread, so an SM holds 384 threads of it.
+constexpr uint32_t kRowWidth = 26;
+constexpr uint32_t kRowSlots = 384;
+struct BatchPlan {
+    bool rows = false;                   // plan the systems that qualify for the row-register form
+};
+constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
 
 struct BatchHost {
     std::vector<BatchCta> ctas;          // launch order: by group, systems in decreasing size within a group
@@ -284,14 +298,23 @@ struct BatchHost {
     std::vector<uint32_t> mass_of_slot;  // [slots] caller index (within its system) of the mass in each slot,
                                          // UINT32_MAX for padding: each CTA holds its masses by decreasing
                                          // degree, so that its SELL slices hold rows of similar length
+    // Row-register form, systems on several CTAs: the halo slots of other CTAs
+    // that hold a copy of each slot's mass (rank << 16 | halo index), two per
+    // slot (kNoPush: none); with more than two the second is kMorePush | an
+    // index into push_more, which holds the count and the remaining codes.
+    std::vector<uint32_t> push;          // [slots][2], empty if no system needs it
+    std::vector<uint32_t> push_more;
     uint32_t total_slots = 0;
     bool any_act = false;
 };
 
 // Builds the layout of n_systems validated systems (act may be null; act[r].amp
 // null: system r is not actuated).  False, with the reason in *why, if a
-// system fits no cluster of kBatchMaxCluster CTAs.
+// system fits no cluster of kBatchMaxCluster CTAs.  With plan.rows, systems that
+// qualify for the row-register form get the smallest cluster of 1, 2, 3, 4,
+// 5, 6 or 8 CTAs of at most kRowSlots masses and launch groups of their own, split
+// by how many of their CTAs an SM's registers hold.
 bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_springs *springs,
-                 const titan_actuation *act, BatchHost &out, std::string *why);
+                 const titan_actuation *act, BatchHost &out, std::string *why, const BatchPlan &plan = BatchPlan());
 
 }  // namespace titan
