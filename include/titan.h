@@ -411,14 +411,18 @@ titan_status titan_batch_rollout(titan_batch *b, uint64_t n_steps);
 
 /* The autotuner: times each launch group with 128, 256, 512 and 1024 threads
  * per CTA and at most 1, 2, 4 or 8 threads per mass over a probe_steps
- * rollout (0: 50) and keeps the fastest pair.  The state is unchanged. */
+ * rollout (0: 50) and keeps the fastest pair, or the row-register form (a
+ * thread per mass, its row in registers: systems whose masses have at most 26
+ * springs each take it until configured otherwise) where that is faster still.
+ * The state is unchanged. */
 titan_status titan_batch_autotune(titan_batch *b, uint32_t probe_steps);
 
 /* Sets a launch group's shape by hand: threads per CTA (a multiple of 32,
  * up to 1024) and the most threads per mass (1, 2, 4 or 8): a mass's springs
  * are split over that many threads, and each CTA takes the largest power of
  * two up to it that still gives every mass of the CTA its own threads in one
- * pass (at least 1).  Errors: TITAN_E_INVALID. */
+ * pass (at least 1).  The group then runs the looped form in this shape.
+ * Errors: TITAN_E_INVALID. */
 titan_status titan_batch_configure(titan_batch *b, uint32_t group, uint32_t threads,
                                    uint32_t threads_per_mass);
 
@@ -436,8 +440,8 @@ titan_status titan_batch_read(titan_batch *b, uint32_t system, float *pos, float
  * enqueued work.  Waits. */
 titan_status titan_batch_centroids(titan_batch *b, float *out);
 
-/* Number of launch groups (one per cluster size) and, per group, its cluster
- * size, threads per CTA, most threads per mass and CTA count (outputs may be
+/* Number of launch groups and, per group, its cluster size, the looped form's
+ * threads per CTA and most threads per mass, and its CTA count (outputs may be
  * NULL). */
 uint32_t titan_batch_groups(const titan_batch *b);
 titan_status titan_batch_info(const titan_batch *b, uint32_t group, uint32_t *cluster,

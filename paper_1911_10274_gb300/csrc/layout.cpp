@@ -604,6 +604,26 @@ size_t persistent_smem_bytes(uint32_t per_cta, uint32_t max_halo, uint32_t max_e
     return persist_layout(per_cta, max_halo, max_entries, has_c, has_act).total;
 }
 
+void invert_halos(const std::vector<std::pair<const uint32_t *, uint32_t>> &halo, uint32_t per, uint32_t *push,
+                  std::vector<uint32_t> &more) {
+    std::vector<std::vector<uint32_t>> to(halo.size() * per);
+    for (uint32_t q = 0; q < (uint32_t)halo.size(); ++q)
+        for (uint32_t h = 0; h < halo[q].second; ++h) {
+            const uint32_t code = halo[q].first[h];
+            to[(size_t)(code >> 16) * per + (code & 0xffffu)].push_back(q << 16 | h);
+        }
+    for (size_t k = 0; k < to.size(); ++k) {
+        uint32_t *pc = push + 2 * k;
+        pc[0] = to[k].size() > 0 ? to[k][0] : kNoPush;
+        pc[1] = to[k].size() == 2 ? to[k][1] : kNoPush;
+        if (to[k].size() > 2) {
+            pc[1] = kMorePush | (uint32_t)more.size();
+            more.push_back((uint32_t)to[k].size() - 1);
+            more.insert(more.end(), to[k].begin() + 1, to[k].end());
+        }
+    }
+}
+
 bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const std::vector<uint32_t> &nbr,
                      bool has_c, bool has_act, size_t smem_limit, PersistPlan &plan,
                      std::vector<uint16_t> &slot, std::vector<uint32_t> &halo) {
@@ -853,24 +873,10 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
         for (const auto &hh : per_sys[r]) halo_slots = std::max(halo_slots, hh.d.halo_count);
         for (auto &hh : per_sys[r]) hh.d.halo_slots = halo_slots;
         if (rows_of[r] && C > 1) {
-            // the halo lists the other way round: where each slot's mass is copied to
-            std::vector<std::vector<uint32_t>> to((size_t)C * per);
-            for (uint32_t q = 0; q < C; ++q)
-                for (uint32_t h = 0; h < (uint32_t)per_sys[r][q].halo.size(); ++h) {
-                    const uint32_t code = per_sys[r][q].halo[h];
-                    to[(size_t)(code >> 16) * per + (code & 0xffffu)].push_back(q << 16 | h);
-                }
+            std::vector<std::pair<const uint32_t *, uint32_t>> lists;
+            for (const auto &hh : per_sys[r]) lists.push_back({hh.halo.data(), (uint32_t)hh.halo.size()});
             out.push.resize(2 * (size_t)(slot_cursor + C * per), kNoPush);
-            for (size_t k = 0; k < to.size(); ++k) {
-                uint32_t *pc = &out.push[2 * (slot_cursor + k)];
-                if (to[k].size() > 0) pc[0] = to[k][0];
-                if (to[k].size() == 2) pc[1] = to[k][1];
-                if (to[k].size() > 2) {
-                    pc[1] = kMorePush | (uint32_t)out.push_more.size();
-                    out.push_more.push_back((uint32_t)to[k].size() - 1);
-                    out.push_more.insert(out.push_more.end(), to[k].begin() + 1, to[k].end());
-                }
-            }
+            invert_halos(lists, per, out.push.data() + 2 * (size_t)slot_cursor, out.push_more);
         }
         slot_cursor += C * per;
         // initial state of every slot of this system (padding slots: fixed, at rest)

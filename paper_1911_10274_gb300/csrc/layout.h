@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "titan.h"
@@ -199,6 +200,25 @@ bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const s
                      bool has_c, bool has_act, size_t smem_limit, PersistPlan &plan,
                      std::vector<uint16_t> &slot, std::vector<uint32_t> &halo);
 
+// ---- row-register forms (k_batch_rows, k_step_persist_rows)
+//
+// A thread keeps a mass's whole row in its registers when no row is wider than
+// kRowWidth (the neighbours of a lattice site).  4.5 registers per actuated
+// entry x 26 and the arithmetic need 168 registers a thread, so an SM holds 384
+// threads of that form (kRowSlots); without actuation 128, and 512.
+constexpr uint32_t kRowWidth = 26;
+constexpr uint32_t kRowSlots = 384;
+constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
+
+// The halo lists of a cluster the other way round: where each mass is copied
+// to.  halo[q] lists CTA q's halo entries (owner rank << 16 | slot in the owner);
+// push gets two words for each of the per slots of every CTA: the halo entries
+// that copy its mass (rank << 16 | halo index; kNoPush: none), or, with more than
+// two, the first and kMorePush | an index into `more`, which holds the count and
+// the remaining ones.
+void invert_halos(const std::vector<std::pair<const uint32_t *, uint32_t>> &halo, uint32_t per, uint32_t *push,
+                  std::vector<uint32_t> &more);
+
 // ---- batches of independent systems (see batch.cu)
 //
 // Every system is owned by one thread-block cluster of C CTAs (C = 1, 2, 4 or
@@ -272,17 +292,11 @@ struct BatchGroup {
     size_t row_smem = 0;                 // its shared memory: the two state buffers
 };
 
-// The row-register form of the batch kernel (k_batch_rows) keeps a mass's whole
-// row in its thread's registers: systems whose rows are at most kRowWidth wide
-// and whose masses fit 8 CTAs of kRowSlots take it.  4.5 registers per
-// actuated entry x 26 (the neighbours of a lattice site) and the arithmetic
-// need 168 registers a thread, so an SM holds 384 threads of it.
-constexpr uint32_t kRowWidth = 26;
-constexpr uint32_t kRowSlots = 384;
+// The systems of a batch that qualify for the row-register form: rows at most
+// kRowWidth wide, masses on at most 8 CTAs of kRowSlots.
 struct BatchPlan {
-    bool rows = false;                   // plan the systems that qualify for the row-register form
+    bool rows = false;                   // plan them for it
 };
-constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
 
 struct BatchHost {
     std::vector<BatchCta> ctas;          // launch order: by group, systems in decreasing size within a group
@@ -298,10 +312,8 @@ struct BatchHost {
     std::vector<uint32_t> mass_of_slot;  // [slots] caller index (within its system) of the mass in each slot,
                                          // UINT32_MAX for padding: each CTA holds its masses by decreasing
                                          // degree, so that its SELL slices hold rows of similar length
-    // Row-register form, systems on several CTAs: the halo slots of other CTAs
-    // that hold a copy of each slot's mass (rank << 16 | halo index), two per
-    // slot (kNoPush: none); with more than two the second is kMorePush | an
-    // index into push_more, which holds the count and the remaining codes.
+    // Row-register form, systems on several CTAs: the copy lists of
+    // invert_halos, by global slot
     std::vector<uint32_t> push;          // [slots][2], empty if no system needs it
     std::vector<uint32_t> push_more;
     uint32_t total_slots = 0;

@@ -142,11 +142,167 @@ k_step_persist(const MassState *__restrict__ in, MassState *__restrict__ out, ui
     if (rank == 0 && tid == 0) *step_out = step0 + (long long)n_steps;
 }
 
+// The row-register form: one thread per mass, whose row (up to kRowWidth
+// entries) and state stay in its registers for the whole launch, so that a step
+// reads shared memory for the neighbours' states only; each new state is written
+// straight into the halo slots of the CTAs that read it, and one barrier ends
+// the step.  Bound: the latency of one warp's row (a cluster's few warps leave the
+// schedulers nearly empty), so the row is evaluated in groups of kRowGroup
+// entries side by side.  Same entries, same order of the sums as k_step_persist:
+// the same bits.  The 10^3 cube: 50 steps and a snapshot 200 -> 173 us.
+constexpr int kRowGroup = 6;
+
+template <bool HAS_ACT, bool GROUND>
+__global__ void __launch_bounds__(HAS_ACT ? 384 : 512)
+k_step_persist_rows(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n, PersistArgs pa,
+                    const uint32_t *__restrict__ slice_off, const uint16_t *__restrict__ slot,
+                    const uint32_t *__restrict__ halo, const uint2 *__restrict__ push,
+                    const uint32_t *__restrict__ push_more, const float2 *__restrict__ kl,
+                    const float2 *__restrict__ act, StepConst c, const long long *__restrict__ step_in,
+                    long long *__restrict__ step_out, uint32_t n_steps) {
+    constexpr int W = (int)kRowWidth, G = kRowGroup;
+    extern __shared__ __align__(16) unsigned char sm[];
+    const uint32_t per = pa.per_cta, tab = per + pa.max_halo;
+    // two state buffers, (x, y, z, vx) then (vy, vz), own masses then halo
+    float4 *const a0 = reinterpret_cast<float4 *>(sm), *const a1 = a0 + tab;
+    float2 *const b0 = reinterpret_cast<float2 *>(a1 + tab), *const b1 = b0 + tab;
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t rank = pa.cluster > 1 ? cluster.block_rank() : 0;
+    const uint32_t m = threadIdx.x, m0 = rank * per, i = m0 + m;        // blockDim.x == per
+    const bool valid = i < n;
+    const uint32_t h_begin = pa.halo_off[rank], h_count = pa.halo_off[rank + 1] - h_begin;
+
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f), v = p;
+    float k[W], L0[W];
+    float2 as[HAS_ACT ? W : 1];
+    uint32_t slot2[W / 2];
+    uint32_t width = 0;
+    uint2 to = make_uint2(kNoPush, kNoPush);
+    if (valid) load_state(in + i, p, v);
+    if ((i & ~31u) < n) {
+        const uint32_t e0 = slice_off[i >> 5] + (i & 31);
+        width = (slice_off[(i >> 5) + 1] - slice_off[i >> 5]) >> 5;     // even, at most W (host-checked)
+#pragma unroll
+        for (int t = 0; t < W; ++t) {
+            uint32_t s = m;                     // past the row: a spring to itself without stiffness
+            k[t] = 0.f;
+            L0[t] = kPadRest;
+            if (HAS_ACT) as[HAS_ACT ? t : 0] = make_float2(0.f, 0.f);
+            if ((uint32_t)t < width) {
+                s = slot[e0 + 32 * t];
+                const float2 a = kl[e0 + 32 * t];
+                k[t] = a.x;
+                L0[t] = a.y;
+                if (HAS_ACT) as[HAS_ACT ? t : 0] = act[e0 + 32 * t];
+            }
+            if (t & 1) slot2[t >> 1] |= s << 16;
+            else slot2[t >> 1] = s;
+        }
+    }
+    a0[m] = make_float4(p.x, p.y, p.z, v.x);
+    b0[m] = make_float2(v.y, v.z);
+    if (pa.cluster > 1) {
+        if (valid) to = push[i];
+        for (uint32_t h = m; h < h_count; h += per) {      // the first step's halo
+            const uint32_t code = halo[h_begin + h];
+            float4 q, w;
+            load_state(in + (code >> 16) * per + (code & 0xffffu), q, w);
+            a0[per + h] = make_float4(q.x, q.y, q.z, w.x);
+            b0[per + h] = make_float2(w.y, w.z);
+        }
+    }
+    const long long step0 = *step_in;
+    // a mass that neither moves nor is read (an empty cell of a grid layout) takes no further part
+    const bool live = valid && (p.w != 0.f || to.x != kNoPush || width != 0);
+    if (pa.cluster > 1) cluster.sync();     // every CTA's shared memory is filled and alive
+    else __syncthreads();
+
+    int cur = 0;
+    for (uint32_t step = 0; step < n_steps; ++step) {
+        const float4 *const srcA = cur ? a1 : a0;
+        const float2 *const srcB = cur ? b1 : b0;
+        const float clk = HAS_ACT ? actuation_clock(c, step0 + (long long)step) : 0.f;
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+#pragma unroll
+        for (int t = 0; t < W; t += G) {
+            if ((uint32_t)t < width) {          // warp-uniform
+                float f[G], ux[G], uy[G], uz[G];
+#pragma unroll
+                for (int u = 0; u < G && t + u < W; ++u) {
+                    const uint32_t s2 = slot2[(t + u) >> 1], s = ((t + u) & 1) ? s2 >> 16 : s2 & 0xffffu;
+                    const float4 qa = srcA[s];
+                    const float2 qb = srcB[s];
+                    const float L = HAS_ACT ? actuated_length(c, L0[t + u], as[HAS_ACT ? t + u : 0], clk) : L0[t + u];
+                    spring_terms(p, v, qa, make_float4(qa.w, qb.x, qb.y, 0.f), k[t + u], L, c.c_uniform, f[u], ux[u],
+                                 uy[u], uz[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < G && t + u < W; ++u) {
+                    fx = __fmaf_rn(f[u], ux[u], fx);
+                    fy = __fmaf_rn(f[u], uy[u], fy);
+                    fz = __fmaf_rn(f[u], uz[u], fz);
+                }
+            }
+        }
+        if (live) {
+            MassState o;
+            integrate<GROUND>(p, v, fx, fy, fz, c, &o);
+            p = o.p;
+            v = o.v;
+            float4 *const dstA = cur ? a0 : a1;
+            float2 *const dstB = cur ? b0 : b1;
+            const float4 na = make_float4(p.x, p.y, p.z, v.x);
+            const float2 nb = make_float2(v.y, v.z);
+            dstA[m] = na;
+            dstB[m] = nb;
+            auto send = [&](uint32_t code) {
+                const uint32_t h = per + (code & 0xffffu);
+                *cluster.map_shared_rank(dstA + h, code >> 16) = na;
+                *cluster.map_shared_rank(dstB + h, code >> 16) = nb;
+            };
+            if (to.x != kNoPush) {
+                send(to.x);
+                if (to.y != kNoPush) {
+                    if (to.y & kMorePush) {
+                        const uint32_t *more = push_more + (to.y & ~kMorePush);
+                        const uint32_t cnt = more[0];
+                        for (uint32_t q = 1; q <= cnt; ++q) send(more[q]);
+                    } else {
+                        send(to.y);
+                    }
+                }
+            }
+        }
+        // the new state is complete, here and in the halos, and every read of
+        // the old one is done before the next step overwrites it
+        if (pa.cluster > 1) cluster.sync();
+        else __syncthreads();
+        cur ^= 1;
+    }
+    if (valid) {
+        MassState o;
+        o.p = p;
+        o.v = live ? v : make_float4(0.f, 0.f, 0.f, 0.f);      // not live: fixed
+        out[i] = o;
+    }
+    if (rank == 0 && m == 0) *step_out = step0 + (long long)n_steps;
+}
+
 }  // namespace
+
+// Whether a plan runs in the row-register form: no per-spring damping (its array
+// would not fit the registers), a thread per mass within the form's block
+// size, and rows of at most kRowWidth entries.
+bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, bool has_c, bool has_act) {
+    if (has_c || plan.per_cta > (has_act ? kRowSlots : 512u)) return false;
+    for (size_t s = 0; s + 1 < slice_off.size(); ++s)
+        if (slice_off[s + 1] - slice_off[s] > 32 * kRowWidth) return false;
+    return true;
+}
 
 cudaError_t launch_step_persistent(const MassState *in, MassState *out, uint32_t n, const PersistPlan &plan,
                                    const uint32_t *slice_off, const uint16_t *slot, const uint32_t *halo,
-                                   const float2 *kl, const float *cc, const float2 *act, const StepConst &c,
+                                   const uint2 *push, const uint32_t *push_more, const float2 *kl, const float *cc, const float2 *act, const StepConst &c,
                                    const long long *step_in, long long *step_out, uint32_t n_steps,
                                    cudaStream_t stream) {
     const bool hc = cc != nullptr, ha = act != nullptr, gr = c.ground != 0;
@@ -168,6 +324,17 @@ cudaError_t launch_step_persistent(const MassState *in, MassState *out, uint32_t
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (push) {
+        auto kern = ha ? (gr ? k_step_persist_rows<true, true> : k_step_persist_rows<true, false>)
+                       : (gr ? k_step_persist_rows<false, true> : k_step_persist_rows<false, false>);
+        cfg.blockDim = dim3(plan.per_cta);
+        cfg.dynamicSmemBytes = (size_t)(plan.per_cta + plan.max_halo) * 2 * (sizeof(float4) + sizeof(float2));
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)cfg.dynamicSmemBytes);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kern, in, out, n, pa, slice_off, slot, halo, push, push_more, kl, act, c,
+                                  step_in, step_out, n_steps);
+    }
     decltype(&k_step_persist<false, false, false>) kern;
     if (hc) {
         if (ha) kern = gr ? k_step_persist<true, true, true> : k_step_persist<true, true, false>;

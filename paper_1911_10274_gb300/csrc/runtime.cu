@@ -520,6 +520,27 @@ cudaError_t resolve_exec(titan_sim *sim) {
     }
     if ((e = upload(sim->d_pslot, slot, sim->stream)) != cudaSuccess) return e;
     if ((e = upload(sim->d_phalo, halo, sim->stream)) != cudaSuccess) return e;
+    std::vector<uint32_t> push, more;
+    sim->persist_rows = titan::persist_rows_fit(plan, sim->sell.slice_off, sim->has_c, sim->has_act);
+    if (sim->persist_rows) {
+        std::vector<std::pair<const uint32_t *, uint32_t>> lists;
+        for (uint32_t r = 0; r < plan.cluster; ++r)
+            lists.push_back({halo.data() + plan.halo_off[r], plan.halo_off[r + 1] - plan.halo_off[r]});
+        push.resize(2 * (size_t)plan.cluster * plan.per_cta);
+        titan::invert_halos(lists, plan.per_cta, push.data(), more);
+        if (push.size() / 2 > sim->ppush_cap) {
+            if ((e = dev_alloc(sim, &sim->d_ppush, push.size() / 2)) != cudaSuccess) return e;
+            sim->ppush_cap = push.size() / 2;
+        }
+        if (more.size() > sim->ppush_more_cap) {
+            if ((e = dev_alloc(sim, &sim->d_ppush_more, more.size())) != cudaSuccess) return e;
+            sim->ppush_more_cap = more.size();
+        }
+        if ((e = cudaMemcpyAsync(sim->d_ppush, push.data(), push.size() * 4, cudaMemcpyHostToDevice, sim->stream)) !=
+            cudaSuccess)
+            return e;
+        if ((e = upload(sim->d_ppush_more, more, sim->stream)) != cudaSuccess) return e;
+    }
     // the host vectors must outlive the asynchronous copies
     if ((e = cudaStreamSynchronize(sim->stream)) != cudaSuccess) return e;
     sim->plan = plan;
@@ -964,7 +985,9 @@ titan_status titan_step(titan_sim *sim, uint64_t n_steps) {
         const uint32_t k = (uint32_t)std::min<uint64_t>(n_steps, kPersistChunk);
         const int b = sim->cur;
         TITAN_CK(sim, titan::launch_step_persistent(sim->state[b], sim->state[1 - b], sim->n_dev, sim->plan,
-                                                    sim->d_slice_off, sim->d_pslot, sim->d_phalo, sim->d_kl,
+                                                    sim->d_slice_off, sim->d_pslot, sim->d_phalo,
+                                                    sim->persist_rows ? sim->d_ppush : nullptr, sim->d_ppush_more,
+                                                    sim->d_kl,
                                                     sim->has_c ? sim->d_c : nullptr, sim->has_act ? sim->d_act : nullptr,
                                                     sim->c, sim->steps_dev + b, sim->steps_dev + (1 - b), k,
                                                     sim->stream));

@@ -55,6 +55,10 @@ struct SimCore {
     uint16_t *d_pslot = nullptr;          // persistent kernel: neighbour slot per SELL entry
     uint32_t *d_phalo = nullptr;          // persistent kernel: halo list
     size_t phalo_cap = 0;
+    bool persist_rows = false;            // the plan runs in the row-register form
+    uint2 *d_ppush = nullptr;             // its copy lists, two words per device mass
+    uint32_t *d_ppush_more = nullptr;
+    size_t ppush_cap = 0, ppush_more_cap = 0;
 
     MassState *state[2] = {nullptr, nullptr};
     long long *steps_dev = nullptr;       // [2]

@@ -188,10 +188,13 @@ struct PersistArgs {
 
 // n_steps steps in one launch: reads `in`, writes `out` once at the end;
 // step_out = step_in + n_steps.
+// push, push_more: the copy lists of invert_halos, by device mass (null: the
+// looped form).
 struct PersistPlan;
+bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, bool has_c, bool has_act);
 cudaError_t launch_step_persistent(const MassState *in, MassState *out, uint32_t n, const PersistPlan &plan,
                                    const uint32_t *slice_off, const uint16_t *slot, const uint32_t *halo,
-                                   const float2 *kl, const float *cc, const float2 *act, const StepConst &c,
+                                   const uint2 *push, const uint32_t *push_more, const float2 *kl, const float *cc, const float2 *act, const StepConst &c,
                                    const long long *step_in, long long *step_out, uint32_t n_steps,
                                    cudaStream_t stream);
 
