@@ -3,23 +3,23 @@
 //
 // Forward: the ordinary step (Titan Sec. III-B, Eq. 1; Sec. III-A contact,
 // friction and constraints) with L = L0 (1 + A sin(2 pi f t + phi)).  The
-// rollout runs forward once, keeping the state every `every` steps
-// (checkpoints); then, segment by segment from the last, the segment's states
-// are recomputed from its checkpoint and the step is reversed one step at a
-// time.  Reversing a step takes two kernels:
-//   k_adj_mass   - per mass: the adjoint of x' = x + v' dt, v' = v + a dt and
-//                  a = F/m + g + contact/friction (the branch the forward step
-//                  took at each kink), giving dJ/dF and the direct terms of
-//                  dJ/dx, dJ/dv;
-//   k_adj_spring - per mass, gathering its SELL row in the forward's fixed
-//                  order: each spring's adjoint seen from this end (both ends
-//                  compute the same spring scalars), added to this mass only;
-//                  the half-edge of the spring's first end also adds dJ/dA and
-//                  dJ/dphi to the spring's gradient (one owner: no atomics,
-//                  a fixed summation order).
+// rollout runs forward once, keeping every state if they fit (kAdjTrajectory),
+// else the state every `every` steps (checkpoints) and the states of the last
+// segment; earlier segments are recomputed from their checkpoints.  Then, from
+// the last step back, k_adj_step reverses one step per launch, per mass:
+//   - the adjoint of x' = x + v' dt, v' = v + a dt and a = F/m + g +
+//     contact/friction (the branch the forward step took at each kink), giving
+//     dJ/dF and the direct terms of dJ/dx, dJ/dv;
+//   - its SELL row in the forward's fixed order: each spring's adjoint seen
+//     from this end (both ends compute the same spring scalars), added to this
+//     mass only; the half-edge of the spring's first end also adds to the
+//     spring's gradient (one owner: no atomics, a fixed summation order);
+//   - dJ/dF of the step before, which its neighbours gather in the next launch.
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -30,31 +30,35 @@ namespace {
 
 constexpr int kT = 256;
 constexpr uint32_t kOwner = 0x80000000u;
-constexpr uint32_t kNoSpring = 0xffffffffu;
+constexpr int kAdjT = 128;
+// The whole trajectory of a rollout is kept when it takes at most this (1/280 of
+// the memory), so that no step runs twice; longer ones are checkpointed.
+constexpr size_t kAdjTrajectory = (size_t)1 << 30;
 
+// The adjoint a force on a mass carries, from (x_b, v_b) of the state after the step:
+// v' = v + (F / m + ...) dt and x' = x + v' dt.
+__device__ __forceinline__ float4 force_adjoint(float4 xo, float4 vo, float im, float dt) {
+    const float vtx = vo.x + dt * xo.x, vty = vo.y + dt * xo.y, vtz = vo.z + dt * xo.z;
+    return make_float4(dt * vtx * im, dt * vty * im, dt * vtz * im, 0.f);
+}
+
+// The mass part of reversing a step at state (p, v): from (xo, vo), the adjoint
+// of the state after it, the direct terms (x_b, v_b) and the force's adjoint F.
 template <bool GROUND>
-__global__ void __launch_bounds__(kT)
-k_adj_mass(const MassState *__restrict__ X, const float4 *__restrict__ xbo, const float4 *__restrict__ vbo,
-           float4 *__restrict__ xb, float4 *__restrict__ vb, float4 *__restrict__ Fb, uint32_t n,
-           titan::StepConst c) {
-    const uint32_t i = blockIdx.x * kT + threadIdx.x;
-    if (i >= n) return;
-    const float4 p = X[i].p, v = X[i].v;
-    const float4 xo = xbo[i], vo = vbo[i];
+__device__ __forceinline__ void adj_mass(const float4 &p, const float4 &v, const float4 &xo, const float4 &vo,
+                                         const titan::StepConst &c, float4 &x_b, float4 &v_b, float4 &F) {
     const float im = p.w;
+    x_b = make_float4(xo.x, xo.y, xo.z, 0.f);
     if (im == 0.f) {                       // fixed: x' = x, v' = 0
-        xb[i] = make_float4(xo.x, xo.y, xo.z, 0.f);
-        vb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        Fb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        v_b = F = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
     const float dt = c.dt;
     const float vtx = vo.x + dt * xo.x, vty = vo.y + dt * xo.y, vtz = vo.z + dt * xo.z;
-    float4 x_b = make_float4(xo.x, xo.y, xo.z, 0.f);
-    float4 v_b = make_float4(vtx, vty, vtz, 0.f);
-    const float abx = dt * vtx, aby = dt * vty, abz = dt * vtz;
-    Fb[i] = make_float4(abx * im, aby * im, abz * im, 0.f);
+    v_b = make_float4(vtx, vty, vtz, 0.f);
+    F = force_adjoint(xo, vo, im, dt);
     if (GROUND && p.z < 0.f) {
+        const float abx = dt * vtx, aby = dt * vty, abz = dt * vtz;
         x_b.z += -c.ground_k * im * abz;                   // a_z += kg (-z) / m
         const float vt = sqrtf(v.x * v.x + v.y * v.y);
         if (vt > 0.f) {
@@ -72,96 +76,124 @@ k_adj_mass(const MassState *__restrict__ X, const float4 *__restrict__ xbo, cons
             v_b.y += (wby - wdot * wy) / vt + vtb * wy;
         }
     }
-    xb[i] = x_b;
-    vb[i] = v_b;
 }
 
-// The adjoint of one spring seen from the mass at (p, v): adds to x_b, v_b and,
-// for the spring's owner half-edge, to the spring's (dJ/dA, dJ/dphi) kept at
-// that half-edge's entry (coalesced with the rows; gathered per spring at the
-// end).
-template <bool HAS_C>
-__device__ __forceinline__ void adj_half_edge(const float4 &p, const float4 &v, const float4 &Fi, const float4 &q,
-                                              const float4 &w, const float4 &Fj, float2 a, float2 s, float cd,
-                                              float ph, uint32_t spr, float4 &x_b, float4 &v_b,
-                                              float2 *__restrict__ gacc) {
+// The adjoint of one spring seen from the mass at (p, v): adds to x_b, v_b and
+// returns dJ/dL.  a = {k, L0, A cos phi, A sin phi}, sc the step's (sin, cos)
+// of the clock phase.  A padding entry is a spring of the mass to itself.
+__device__ __forceinline__ float adj_half_edge(const float4 &p, const float4 &v, const float4 &Fi, const float4 &q,
+                                               const float4 &w, const float4 &Fj, const float4 &a, float2 sc, float cd,
+                                               float4 &x_b, float4 &v_b) {
     const float dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
     const float l2 = dx * dx + dy * dy + dz * dz;
-    if (!(l2 > 0.f)) return;                              // zero length: no force
+    if (!(l2 > 0.f)) return 0.f;                          // zero length: no force
     const float inv = rsqrtf(l2);
     const float l = l2 * inv;
     const float ux = dx * inv, uy = dy * inv, uz = dz * inv;
     const float k = a.x;
-    float sn, cs;
-    sincosf(ph + s.y, &sn, &cs);
-    const float L = a.y * (1.f + s.x * sn);
+    const float L = a.y + a.y * (a.z * sc.x + a.w * sc.y);
     const float dvx = w.x - v.x, dvy = w.y - v.y, dvz = w.z - v.z;
     const float rate = dvx * ux + dvy * uy + dvz * uz;
     const float f = k * (l - L) + cd * rate;
     const float gx = Fi.x - Fj.x, gy = Fi.y - Fj.y, gz = Fi.z - Fj.z;
     const float fb = gx * ux + gy * uy + gz * uz;
-    const float lb = k * fb, Lb = -k * fb, rb = cd * fb;
+    const float lb = k * fb, rb = cd * fb;
     const float ubx = f * gx + rb * dvx, uby = f * gy + rb * dvy, ubz = f * gz + rb * dvz;
     v_b.x -= rb * ux; v_b.y -= rb * uy; v_b.z -= rb * uz;
     const float udot = ubx * ux + uby * uy + ubz * uz;
     x_b.x -= (ubx - udot * ux) * inv + lb * ux;
     x_b.y -= (uby - udot * uy) * inv + lb * uy;
     x_b.z -= (ubz - udot * uz) * inv + lb * uz;
-    if (spr & kOwner) {                   // gacc points at this entry's accumulator
-        float2 g = *gacc;
-        g.x += Lb * a.y * sn;
-        g.y += Lb * a.y * s.x * cs;
-        *gacc = g;
-    }
+    return -lb;
 }
 
-// Widths are even: two entries per iteration, every load of both issued
-// before either is reversed (summation order unchanged: entry t, then t + 1).
-template <bool HAS_C>
-__global__ void __launch_bounds__(kT)
-k_adj_spring(const MassState *__restrict__ X, const float4 *__restrict__ Fb, float4 *__restrict__ xb,
-             float4 *__restrict__ vb, uint32_t n, const uint32_t *__restrict__ slice_off,
-             const uint32_t *__restrict__ nbr, const uint32_t *__restrict__ spring,
-             const float2 *__restrict__ kl, const float2 *__restrict__ act, const float *__restrict__ cc,
-             titan::StepConst c, long long step, float2 *__restrict__ gacc) {
-    const uint32_t i = blockIdx.x * kT + threadIdx.x;
+// One reversed step: the mass part of this thread's mass, then its row, then
+// the force adjoint of the step before (Fout; the neighbours' is read from Fin).
+// (xb, vb) are this mass's alone and updated in place.
+//
+// Bound by the gathers (48 bytes an entry, 45 % of them from L1: the masses of
+// 2,500 threads and their neighbours just fill it) and the row stream (20 bytes
+// an entry from L2).  Two entries are reversed per iteration, with the next
+// two's constants already requested; 128-thread blocks, six per SM.  The row
+// stream through an asynchronous ring in shared memory measured 9 % slower (it
+// takes L1 from the gathers), adding to the sums by load and store 6 %.  The sine
+// and cosine of each spring's own phase are in the row and the clock's come with
+// the launch, so no trigonometric function is left in the loop: the spring's
+// (dJ/dA, dJ/dphi) is a rotation of the two sums kept here, formed once at the
+// end (k_adj_gather).  256 robots, 107,193 masses: a mass and a spring kernel per
+// step 44 us, this 18.
+template <bool HAS_C, bool GROUND>
+__global__ void __launch_bounds__(kAdjT, 6)
+k_adj_step(const MassState *__restrict__ X, const float4 *__restrict__ Fin, float4 *__restrict__ Fout,
+           float4 *__restrict__ xb, float4 *__restrict__ vb, uint32_t n, const uint32_t *__restrict__ slice_off,
+           const uint32_t *__restrict__ nbr, const float4 *__restrict__ row, const float *__restrict__ cc,
+           titan::StepConst c, float2 sc, float2 *__restrict__ gacc) {
+    const uint32_t tid = threadIdx.x, i = blockIdx.x * kAdjT + tid;
     if (i >= n) return;
-    const uint32_t sl = i >> 5, lane = i & 31;
-    const uint32_t e0 = slice_off[sl];
-    const uint32_t width = (slice_off[sl + 1] - e0) >> 5;
-    float4 p, v;
+    const uint32_t sl = i >> 5;
+    uint32_t e = slice_off[sl] + (i & 31);
+    const uint32_t end = slice_off[sl + 1];               // widths are even
+    float4 p, v, x_b, v_b, Fi;
     titan::load_state(X + i, p, v);
-    const float4 Fi = Fb[i];
-    float4 x_b = xb[i], v_b = vb[i];
-    const float ph = titan::clock_phase(c, step);
-    for (uint32_t t = 0; t < width; t += 2) {
-        const uint32_t e = e0 + 32 * t + lane, f = e + 32;
-        const uint32_t spr0 = __ldg(spring + e), spr1 = __ldg(spring + f);
-        // padding entries point at the mass itself: their loads are harmless
-        const uint32_t j0 = __ldg(nbr + e), j1 = __ldg(nbr + f);
-        const float2 a0 = __ldg(kl + e), a1 = __ldg(kl + f), s0 = __ldg(act + e), s1 = __ldg(act + f);
-        const float c0 = HAS_C ? __ldg(cc + e) : c.c_uniform, c1 = HAS_C ? __ldg(cc + f) : c.c_uniform;
+    adj_mass<GROUND>(p, v, xb[i], vb[i], c, x_b, v_b, Fi);
+    uint32_t nj0, nj1;
+    float4 na0, na1;
+    auto request = [&](uint32_t x) {
+        if (x < end) {
+            nj0 = __ldcg(nbr + x);
+            nj1 = __ldcg(nbr + x + 32);
+            na0 = __ldcg(row + x);
+            na1 = __ldcg(row + x + 32);
+        }
+    };
+    request(e);
+    for (; e < end; e += 64) {
+        const uint32_t j0 = nj0, j1 = nj1;
+        const float4 a0 = na0, a1 = na1;
+        request(e + 64);
+        const uint32_t i0 = j0 & ~kOwner, i1 = j1 & ~kOwner;
+        const bool own0 = j0 & kOwner, own1 = j1 & kOwner;
         float4 q0, w0, q1, w1;
-        titan::load_state(X + j0, q0, w0);
-        titan::load_state(X + j1, q1, w1);
-        const float4 F0 = __ldg(Fb + j0), F1 = __ldg(Fb + j1);
-        if (spr0 != kNoSpring)
-            adj_half_edge<HAS_C>(p, v, Fi, q0, w0, F0, a0, s0, c0, ph, spr0, x_b, v_b, gacc + e);
-        if (spr1 != kNoSpring)
-            adj_half_edge<HAS_C>(p, v, Fi, q1, w1, F1, a1, s1, c1, ph, spr1, x_b, v_b, gacc + f);
+        titan::load_state(X + i0, q0, w0);
+        titan::load_state(X + i1, q1, w1);
+        const float4 F0 = __ldg(Fin + i0), F1 = __ldg(Fin + i1);
+        const float c0 = HAS_C ? __ldcg(cc + e) : c.c_uniform, c1 = HAS_C ? __ldcg(cc + e + 32) : c.c_uniform;
+        const float L0 = adj_half_edge(p, v, Fi, q0, w0, F0, a0, sc, c0, x_b, v_b);
+        const float L1 = adj_half_edge(p, v, Fi, q1, w1, F1, a1, sc, c1, x_b, v_b);
+        // one owner per entry and launch: no order is left open, and nothing is waited for
+        if (own0) atomicAdd(gacc + e, make_float2(L0 * sc.x, L0 * sc.y));
+        if (own1) atomicAdd(gacc + e + 32, make_float2(L1 * sc.x, L1 * sc.y));
     }
     xb[i] = x_b;
     vb[i] = v_b;
+    Fout[i] = force_adjoint(x_b, v_b, p.w, c.dt);
 }
 
-// grad[q] = the accumulator of spring q's owner entry.
-__global__ void k_adj_gather(const float2 *__restrict__ gacc, const uint32_t *__restrict__ owner, uint32_t S,
+// The rows of the reverse pass: {k, L0, A cos phi, A sin phi} per entry.
+__global__ void k_adj_rows(const float2 *__restrict__ kl, const float2 *__restrict__ act, uint32_t n,
+                           float4 *__restrict__ row) {
+    const uint32_t e = blockIdx.x * kT + threadIdx.x;
+    if (e >= n) return;
+    const float2 a = kl[e], s = act[e];
+    float sn, cs;
+    sincosf(s.y, &sn, &cs);
+    row[e] = make_float4(a.x, a.y, s.x * cs, s.x * sn);
+}
+
+// Spring q's gradient from the sums (P, Q) of dJ/dL sin(clock), dJ/dL cos(clock)
+// kept at its owner entry: L = L0 (1 + A sin(clock + phi)).
+__global__ void k_adj_gather(const float2 *__restrict__ gacc, const uint32_t *__restrict__ owner,
+                             const float2 *__restrict__ kl, const float2 *__restrict__ act, uint32_t S,
                              float *__restrict__ grad_amp, float *__restrict__ grad_phase) {
     const uint32_t q = blockIdx.x * kT + threadIdx.x;
     if (q >= S) return;
-    const float2 g = gacc[owner[q]];
-    grad_amp[q] = g.x;
-    grad_phase[q] = g.y;
+    const uint32_t e = owner[q];
+    const float2 g = gacc[e], s = act[e];
+    const float L0 = kl[e].y;
+    float sn, cs;
+    sincosf(s.y, &sn, &cs);
+    grad_amp[q] = L0 * (g.x * cs + g.y * sn);
+    grad_phase[q] = L0 * s.x * (g.y * cs - g.x * sn);
 }
 
 __global__ void k_adj_seed(const float *__restrict__ seed_pos, const float *__restrict__ seed_vel,
@@ -173,6 +205,43 @@ __global__ void k_adj_seed(const float *__restrict__ seed_pos, const float *__re
     xb[d] = make_float4(seed_pos[3 * (size_t)i], seed_pos[3 * (size_t)i + 1], seed_pos[3 * (size_t)i + 2], 0.f);
     if (seed_vel)
         vb[d] = make_float4(seed_vel[3 * (size_t)i], seed_vel[3 * (size_t)i + 1], seed_vel[3 * (size_t)i + 2], 0.f);
+}
+
+__global__ void k_adj_force0(const MassState *__restrict__ X, const float4 *__restrict__ xb,
+                             const float4 *__restrict__ vb, uint32_t n, float dt, float4 *__restrict__ F) {
+    const uint32_t i = blockIdx.x * kT + threadIdx.x;
+    if (i < n) F[i] = force_adjoint(xb[i], vb[i], X[i].p.w, dt);
+}
+
+// The workspaces of titan_adjoint come from a pool of the library's own per
+// device, stream-ordered like the default pool but keeping up to twice
+// kAdjTrajectory between calls (the default pool gives every byte back at each
+// synchronisation, and mapping them again took as long as dozens of steps).
+// adjoint_trim gives the memory back (titan_destroy).
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64] = {};
+
+cudaError_t adjoint_pool(int dev, cudaMemPool_t *out) {
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        cudaError_t e = cudaMemPoolCreate(&p, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = 2 * kAdjTrajectory;
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        g_pool[dev] = p;
+    }
+    *out = g_pool[dev];
+    return cudaSuccess;
 }
 
 titan_status afail(titan_sim *sim, titan_status st, const std::string &msg) {
@@ -192,6 +261,11 @@ titan_status afail(titan_sim *sim, titan_status st, const std::string &msg) {
 
 }  // namespace
 
+void titan::adjoint_trim(int dev) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (dev >= 0 && dev < 64 && g_pool[dev]) cudaMemPoolTrimTo(g_pool[dev], 0);
+}
+
 extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t every,
                                       const float *seed_pos_dev, const float *seed_vel_dev,
                                       float *grad_amp_dev, float *grad_phase_dev) {
@@ -204,9 +278,10 @@ extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t
     const size_t vec_bytes = (size_t)std::max(nd, 1u) * sizeof(float4);
     cudaStream_t s = sim->stream;
     MassState *ckpt = nullptr, *seg = nullptr;
-    float4 *xb[2] = {nullptr, nullptr}, *vb[2] = {nullptr, nullptr}, *Fb = nullptr;
+    float4 *xb = nullptr, *vb = nullptr, *Fb[2] = {nullptr, nullptr}, *row = nullptr;
     long long *seg_steps = nullptr;
     float2 *gacc = nullptr;
+    cudaMemPool_t pool = nullptr;
     uint64_t n_seg = 0;
     int cur = 0;
     if ((st_ = titan::ensure_layout(sim)) != TITAN_OK) goto out;
@@ -218,109 +293,116 @@ extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t
     cudaGetDevice(&prev);
     if (cudaSetDevice(sim->device) != cudaSuccess) { st_ = afail(sim, TITAN_E_CUDA, "cannot select the device"); goto out; }
     {
-        // per-entry neighbour and spring ownership for the reverse gather (built once)
-        if (!sim->d_adj_spring) {
-            std::vector<uint32_t> spr(sim->sell.entries, kNoSpring);
-            for (uint32_t e = 0; e < sim->sell.entries; ++e)
-                if (sim->sell.spring[e] != UINT32_MAX) spr[e] = sim->sell.spring[e];
-            for (uint32_t q = 0; q < S; ++q) spr[sim->sell.entry_of_end[2 * (size_t)q]] |= kOwner;
-            void *p1 = nullptr;
-            ADJ_CK(cudaMalloc(&p1, std::max<size_t>(spr.size(), 1) * 4));
-            sim->allocations.push_back(p1);
-            sim->d_adj_spring = static_cast<uint32_t *>(p1);
-            ADJ_CK(cudaMemcpy(sim->d_adj_spring, spr.data(), spr.size() * 4, cudaMemcpyHostToDevice));
+        const uint32_t E = sim->sell.entries;
+        // per entry the neighbour and whether this end owns the spring's gradient (built once)
+        if (!sim->d_adj_nbr) {
+            std::vector<uint32_t> nb(sim->sell.nbr);
+            nb.resize(std::max<size_t>(E, 1), 0);
             std::vector<uint32_t> owner(S);
-            for (uint32_t q = 0; q < S; ++q) owner[q] = sim->sell.entry_of_end[2 * (size_t)q];
-            void *p3 = nullptr;
-            ADJ_CK(cudaMalloc(&p3, std::max<size_t>(owner.size(), 1) * 4));
-            sim->allocations.push_back(p3);
-            sim->d_adj_owner = static_cast<uint32_t *>(p3);
-            ADJ_CK(cudaMemcpy(sim->d_adj_owner, owner.data(), owner.size() * 4, cudaMemcpyHostToDevice));
-            if (!sim->d_nbr) {
-                void *p2 = nullptr;
-                ADJ_CK(cudaMalloc(&p2, std::max<size_t>(sim->sell.nbr.size(), 1) * 4));
-                sim->allocations.push_back(p2);
-                sim->d_nbr = static_cast<uint32_t *>(p2);
-                ADJ_CK(cudaMemcpy(sim->d_nbr, sim->sell.nbr.data(), sim->sell.nbr.size() * 4, cudaMemcpyHostToDevice));
+            for (uint32_t q = 0; q < S; ++q) {
+                owner[q] = sim->sell.entry_of_end[2 * (size_t)q];
+                nb[owner[q]] |= kOwner;
             }
+            void *p1 = nullptr, *p2 = nullptr;
+            ADJ_CK(cudaMalloc(&p1, nb.size() * 4));
+            sim->allocations.push_back(p1);
+            ADJ_CK(cudaMalloc(&p2, std::max<size_t>(owner.size(), 1) * 4));
+            sim->allocations.push_back(p2);
+            ADJ_CK(cudaMemcpy(p1, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice));
+            ADJ_CK(cudaMemcpy(p2, owner.data(), owner.size() * 4, cudaMemcpyHostToDevice));
+            sim->d_adj_nbr = static_cast<uint32_t *>(p1);
+            sim->d_adj_owner = static_cast<uint32_t *>(p2);
         }
-        n_seg = (n_steps + every - 1) / every;
-        const unsigned gm = (nd + kT - 1) / kT;
-        ADJ_CK(cudaMallocAsync((void **)&ckpt, state_bytes * (n_seg + 1), s));
-        ADJ_CK(cudaMallocAsync((void **)&seg, state_bytes * (every + 1), s));
-        for (int b = 0; b < 2; ++b) {
-            ADJ_CK(cudaMallocAsync((void **)&xb[b], vec_bytes, s));
-            ADJ_CK(cudaMallocAsync((void **)&vb[b], vec_bytes, s));
+        const bool whole = n_steps < kAdjTrajectory / state_bytes;
+        const uint64_t len_max = whole ? n_steps : every;
+        n_seg = whole ? (n_steps ? 1 : 0) : (n_steps + every - 1) / every;
+        const unsigned gm = (nd + kT - 1) / kT, ga = (nd + kAdjT - 1) / kAdjT;
+        ADJ_CK(adjoint_pool(sim->device, &pool));
+        auto take = [&](auto **p, size_t bytes) { return cudaMallocFromPoolAsync((void **)p, bytes, pool, s); };
+        if (n_seg > 1) ADJ_CK(take(&ckpt, state_bytes * (n_seg - 1)));
+        ADJ_CK(take(&seg, state_bytes * (len_max + 1)));
+        ADJ_CK(take(&xb, vec_bytes));
+        ADJ_CK(take(&vb, vec_bytes));
+        for (int b = 0; b < 2; ++b) ADJ_CK(take(&Fb[b], vec_bytes));
+        ADJ_CK(take(&seg_steps, sizeof(long long) * (len_max + 1)));
+        ADJ_CK(take(&gacc, std::max<size_t>(E, 1) * sizeof(float2)));
+        ADJ_CK(take(&row, std::max<size_t>(E, 1) * sizeof(float4)));
+        ADJ_CK(cudaMemsetAsync(gacc, 0, std::max<size_t>(E, 1) * sizeof(float2), s));
+        if (E) {
+            k_adj_rows<<<(E + kT - 1) / kT, kT, 0, s>>>(sim->d_kl, sim->d_act, E, row);
+            ADJ_CK(cudaGetLastError());
         }
-        ADJ_CK(cudaMallocAsync((void **)&Fb, vec_bytes, s));
-        ADJ_CK(cudaMallocAsync((void **)&seg_steps, sizeof(long long) * (every + 1), s));
-        ADJ_CK(cudaMallocAsync((void **)&gacc, std::max<size_t>(sim->sell.entries, 1) * sizeof(float2), s));
-        ADJ_CK(cudaMemsetAsync(gacc, 0, std::max<size_t>(sim->sell.entries, 1) * sizeof(float2), s));
         const uint64_t step0 = sim->steps;
-        // forward rollout through the ordinary step, keeping checkpoints
-        ADJ_CK(cudaMemcpyAsync(ckpt, sim->state[sim->cur], state_bytes, cudaMemcpyDeviceToDevice, s));
+        // forward rollout through the ordinary step, keeping a checkpoint at the start of every
+        // segment but the last, whose states are all kept as they are formed
         for (uint64_t g = 0; g < n_seg; ++g) {
-            const uint64_t len = std::min<uint64_t>(every, n_steps - g * every);
-            for (uint64_t k = 0; k < len; ++k) {
-                ADJ_CK(titan::enqueue_sim_step(sim, s, sim->cur, k > 0));
-                sim->cur ^= 1;
-                ++sim->steps;
+            const uint64_t len = std::min<uint64_t>(len_max, n_steps - g * len_max);
+            const bool last = g + 1 == n_seg;
+            ADJ_CK(cudaMemcpyAsync(last ? seg : ckpt + g * nd, sim->state[sim->cur], state_bytes, cudaMemcpyDeviceToDevice, s));
+            if (!last) {
+                for (uint64_t k = 0; k < len; ++k) {
+                    ADJ_CK(titan::enqueue_sim_step(sim, s, sim->cur, k > 0));
+                    sim->cur ^= 1;
+                    ++sim->steps;
+                }
+                continue;
             }
-            ADJ_CK(cudaMemcpyAsync(ckpt + (g + 1) * nd, sim->state[sim->cur], state_bytes, cudaMemcpyDeviceToDevice, s));
+            ADJ_CK(cudaMemcpyAsync(seg_steps, sim->steps_dev + sim->cur, sizeof(long long), cudaMemcpyDeviceToDevice, s));
+            for (uint64_t k = 0; k < len; ++k)
+                ADJ_CK(titan::enqueue_sim_step_io(sim, s, seg + k * nd, seg + (k + 1) * nd, seg_steps + k,
+                                                  seg_steps + k + 1, k > 0));
+            ADJ_CK(cudaMemcpyAsync(sim->state[sim->cur], seg + len * nd, state_bytes, cudaMemcpyDeviceToDevice, s));
+            ADJ_CK(cudaMemcpyAsync(sim->steps_dev + sim->cur, seg_steps + len, sizeof(long long), cudaMemcpyDeviceToDevice, s));
+            sim->steps += len;
         }
         // seed dJ/dx_T, dJ/dv_T in device order; gradients start at zero
-        ADJ_CK(cudaMemsetAsync(xb[0], 0, vec_bytes, s));
-        ADJ_CK(cudaMemsetAsync(vb[0], 0, vec_bytes, s));
+        ADJ_CK(cudaMemsetAsync(xb, 0, vec_bytes, s));
+        ADJ_CK(cudaMemsetAsync(vb, 0, vec_bytes, s));
         if (sim->n) {
             k_adj_seed<<<(sim->n + kT - 1) / kT, kT, 0, s>>>(seed_pos_dev, seed_vel_dev, sim->d_dev_of_caller,
-                                                             sim->n, xb[0], vb[0]);
+                                                             sim->n, xb, vb);
+            ADJ_CK(cudaGetLastError());
+            k_adj_force0<<<gm, kT, 0, s>>>(sim->state[sim->cur], xb, vb, nd, sim->c.dt, Fb[0]);
             ADJ_CK(cudaGetLastError());
         }
 
         for (uint64_t g = n_seg; g-- > 0;) {
-            const uint64_t len = std::min<uint64_t>(every, n_steps - g * every);
-            const long long first = (long long)(step0 + g * every);
-            ADJ_CK(cudaMemcpyAsync(seg, ckpt + g * nd, state_bytes, cudaMemcpyDeviceToDevice, s));
-            ADJ_CK(cudaMemcpyAsync(seg_steps, &first, sizeof(long long), cudaMemcpyHostToDevice, s));
-            // the simulation's own step kernel (every CSR kernel gives bit-identical states)
-            for (uint64_t k = 0; k < len; ++k)
-                ADJ_CK(titan::enqueue_sim_step_io(sim, s, seg + k * nd, seg + (k + 1) * nd, seg_steps + k,
-                                                  seg_steps + k + 1, k > 0));
+            const uint64_t len = std::min<uint64_t>(len_max, n_steps - g * len_max);
+            const long long first = (long long)(step0 + g * len_max);
+            if (g + 1 < n_seg) {
+                ADJ_CK(cudaMemcpyAsync(seg, ckpt + g * nd, state_bytes, cudaMemcpyDeviceToDevice, s));
+                ADJ_CK(cudaMemcpyAsync(seg_steps, &first, sizeof(long long), cudaMemcpyHostToDevice, s));
+                // the simulation's own step kernel (every CSR kernel gives bit-identical states)
+                for (uint64_t k = 0; k < len; ++k)
+                    ADJ_CK(titan::enqueue_sim_step_io(sim, s, seg + k * nd, seg + (k + 1) * nd, seg_steps + k,
+                                                      seg_steps + k + 1, k > 0));
+            }
             for (uint64_t k = len; k-- > 0;) {
+                // the clock's phase as titan::clock_phase forms it
+                const unsigned long long turns = (unsigned long long)(first + (long long)k) * sim->c.act_turns;
+                const double ph = (double)((float)(turns >> 40) * 3.74507028e-7f);
+                const float2 sc = make_float2((float)std::sin(ph), (float)std::cos(ph));
                 const MassState *X = seg + k * nd;
-                if (sim->c.ground)
-                    k_adj_mass<true><<<gm, kT, 0, s>>>(X, xb[cur], vb[cur], xb[cur ^ 1], vb[cur ^ 1], Fb, nd, sim->c);
-                else
-                    k_adj_mass<false><<<gm, kT, 0, s>>>(X, xb[cur], vb[cur], xb[cur ^ 1], vb[cur ^ 1], Fb, nd, sim->c);
-                ADJ_CK(cudaGetLastError());
-                const long long stepk = first + (long long)k;
-                if (sim->has_c)
-                    k_adj_spring<true><<<gm, kT, 0, s>>>(X, Fb, xb[cur ^ 1], vb[cur ^ 1], nd, sim->d_slice_off, sim->d_nbr,
-                                                         sim->d_adj_spring, sim->d_kl, sim->d_act, sim->d_c, sim->c,
-                                                         stepk, gacc);
-                else
-                    k_adj_spring<false><<<gm, kT, 0, s>>>(X, Fb, xb[cur ^ 1], vb[cur ^ 1], nd, sim->d_slice_off, sim->d_nbr,
-                                                          sim->d_adj_spring, sim->d_kl, sim->d_act, sim->d_c, sim->c,
-                                                          stepk, gacc);
-                ADJ_CK(cudaGetLastError());
+                auto launch = [&](auto kern) {
+                    kern<<<ga, kAdjT, 0, s>>>(X, Fb[cur], Fb[cur ^ 1], xb, vb, nd, sim->d_slice_off, sim->d_adj_nbr,
+                                              row, sim->has_c ? sim->d_c : nullptr, sim->c, sc, gacc);
+                    return cudaGetLastError();
+                };
+                if (sim->c.ground) ADJ_CK(sim->has_c ? launch(k_adj_step<true, true>) : launch(k_adj_step<false, true>));
+                else ADJ_CK(sim->has_c ? launch(k_adj_step<true, false>) : launch(k_adj_step<false, false>));
                 cur ^= 1;
             }
         }
         if (S) {
-            k_adj_gather<<<(S + kT - 1) / kT, kT, 0, s>>>(gacc, sim->d_adj_owner, S, grad_amp_dev, grad_phase_dev);
+            k_adj_gather<<<(S + kT - 1) / kT, kT, 0, s>>>(gacc, sim->d_adj_owner, sim->d_kl, sim->d_act, S, grad_amp_dev,
+                                                          grad_phase_dev);
             ADJ_CK(cudaGetLastError());
         }
     }
 done:
-    if (ckpt) cudaFreeAsync(ckpt, s);
-    if (seg) cudaFreeAsync(seg, s);
-    for (int b = 0; b < 2; ++b) {
-        if (xb[b]) cudaFreeAsync(xb[b], s);
-        if (vb[b]) cudaFreeAsync(vb[b], s);
-    }
-    if (Fb) cudaFreeAsync(Fb, s);
-    if (seg_steps) cudaFreeAsync(seg_steps, s);
-    if (gacc) cudaFreeAsync(gacc, s);
+    for (void *p : {(void *)ckpt, (void *)seg, (void *)xb, (void *)vb, (void *)Fb[0], (void *)Fb[1], (void *)seg_steps,
+                    (void *)gacc, (void *)row})
+        if (p) cudaFreeAsync(p, s);
     if (prev >= 0) cudaSetDevice(prev);
 out:
     sim->busy.store(false);

@@ -1313,7 +1313,9 @@ titan_status titan_destroy(titan_sim *sim) {
         DeviceGuard dg(sim->device);
         if (cudaStreamSynchronize(sim->stream) != cudaSuccess) st = TITAN_E_CUDA;
         if (sim->side && cudaStreamSynchronize(sim->side) != cudaSuccess) st = TITAN_E_CUDA;
+        const bool adjoint = sim->d_adj_nbr != nullptr;
         release(sim);
+        if (adjoint) titan::adjoint_trim(sim->device);
     }
     delete sim;
     return st;

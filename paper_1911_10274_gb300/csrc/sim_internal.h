@@ -114,7 +114,7 @@ struct SimCore {
     double snap_t[2] = {0, 0};
     uint64_t last_ticket = 0;
 
-    uint32_t *d_adj_spring = nullptr;     // adjoint: spring id per SELL entry (+ owner bit)
+    uint32_t *d_adj_nbr = nullptr;        // adjoint: neighbour per SELL entry, top bit: this end owns the spring's gradient
     uint32_t *d_adj_owner = nullptr;      // adjoint: owner SELL entry of each spring
 
     std::vector<void *> allocations;
@@ -153,6 +153,8 @@ cudaError_t enqueue_sim_step(titan_sim *sim, cudaStream_t st, int b, bool after_
 cudaError_t enqueue_sim_step_io(titan_sim *sim, cudaStream_t st, const MassState *in, MassState *out,
                                 const long long *step_in, long long *step_out, bool after_step);
 void set_thread_error(const std::string &msg);
+// Gives back what the adjoint's workspace pool holds beyond the blocks in use (adjoint.cu).
+void adjoint_trim(int device);
 // Rebuilds the device layout if masses or springs were added (runtime.cu).
 titan_status ensure_layout(titan_sim *sim);
 }  // namespace titan
