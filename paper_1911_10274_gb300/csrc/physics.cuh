@@ -35,11 +35,16 @@ __device__ __forceinline__ float clock_phase(const StepConst &c, long long step)
     return __fmul_rn((float)(fr >> 40), 3.74507028e-7f);      // 2 pi / 2^24
 }
 
+// Which form of actuation a kernel is compiled for: one of the two, or either
+// (told apart at run time by act_mode).
+constexpr int kActNone = 0, kActSinusoid = 1, kActWorm = 2, kActAny = 3;
+
 // Per-thread actuation clock for step `step`: mode 1 the phase 2 pi f t mod
 // 2 pi, mode 2 (the worm of Sec. V-B, Eq. 3) the time t mod t_p (the same
 // fixed-point turns, of dt / t_p).
+template <int ACT = kActAny>
 __device__ __forceinline__ float actuation_clock(const StepConst &c, long long step) {
-    if (c.act_mode == 2) {
+    if (ACT == kActWorm || (ACT == kActAny && c.act_mode == 2)) {
         const unsigned long long fr = (unsigned long long)step * c.worm_turns;
         return __fmul_rn((float)(fr >> 40), c.worm_unit);
     }
@@ -48,8 +53,9 @@ __device__ __forceinline__ float actuation_clock(const StepConst &c, long long s
 
 // Rest length of an actuated spring: a = (A, phi) in mode 1,
 // (c, t_o mod t_p) in mode 2 where tau = (t - t_o) mod t_p (Eqs. 3-4).
+template <int ACT = kActAny>
 __device__ __forceinline__ float actuated_length(const StepConst &c, float L0, float2 a, float clk) {
-    if (c.act_mode == 2) {
+    if (ACT == kActWorm || (ACT == kActAny && c.act_mode == 2)) {
         float tau = clk - a.y;
         if (tau < 0.f) tau += (float)c.worm_period;
         return L0 * (1.f + a.x * sinf(c.worm_omega * tau));

@@ -172,8 +172,13 @@ __device__ __forceinline__ long long read_step(const long long *p) {
     return OVERLAP ? __ldcg(p) : *p;
 }
 constexpr uint32_t kBoxHoleSlot = 0xFFFF;   // own slot of a hole (layout.h: kBoxHole)
-constexpr int kHaloMinBlocks = 6;      // resident CTAs per SM of the coloured-table halo kernel
-constexpr int kBoxMinBlocks = 6;       // resident CTAs per SM the register budget is sized for
+constexpr int kHaloMinBlocks = 6;      // resident CTAs per SM of the table kernels (halo and box)
+// The same with actuation, whose sine needs registers: at six CTAs per SM (40
+// registers) the halo kernel spilled 164 bytes and the box kernel 88.  Per step,
+// 6 -> 5 -> 4 -> 3 CTAs per SM: 250 worms (101,250 masses, halo) 40.8, 24.8, 13.7, 13.1 us,
+// 400 worms 42.9, 25.7, 17.9, 17.6; 256 robots in one system (halo) 31.7, 23.0, 13.3, 13.2;
+// actuated 50^3 box 23.7, 17.3, 17.4, 17.4 and 70^3 39.4, 33.3, 34.7, 42.4.
+constexpr int kActMinBlocks = 4, kActBoxMinBlocks = 5;
 
 template <bool HAS_C, bool HAS_ACT>
 __device__ __forceinline__ void prefetch_slice(const uint32_t *slice_off, uint32_t sl, const uint16_t *nslot,
@@ -194,8 +199,17 @@ __device__ __forceinline__ void prefetch_slice(const uint32_t *slice_off, uint32
 // order of the sums: the same bits.
 constexpr int kDeepMinBlocks = 2;      // resident CTAs per SM the deep form's registers are sized for
 
-template <int COLS, bool HAS_C, bool HAS_ACT>
+// The resident CTAs per SM a step kernel's registers are sized for.
+constexpr int step_min_blocks(bool box, int act, int cols) {
+    return cols > 2                      ? kDeepMinBlocks
+           : act == kActNone             ? kHaloMinBlocks
+           : box && act == kActSinusoid ? kActBoxMinBlocks
+                                         : kActMinBlocks;
+}
+
+template <int COLS, bool HAS_C, int ACT>
 struct Cols {
+    static constexpr bool HAS_ACT = ACT != kActNone;
     uint32_t j[COLS];                  // table slot (halo) or slot offset (box) of the neighbour
     float2 a[COLS];                    // {k, L0}
     float c[HAS_C ? COLS : 1];
@@ -203,14 +217,15 @@ struct Cols {
 };
 
 // Adds the first `left` (at least one) columns of group g to the force.
-template <int COLS, bool HAS_C, bool HAS_ACT>
-__device__ __forceinline__ void row_group(const Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t left, const float4 &p,
+template <int COLS, bool HAS_C, int ACT>
+__device__ __forceinline__ void row_group(const Cols<COLS, HAS_C, ACT> &g, uint32_t left, const float4 &p,
                                           const float4 &v, const StepConst &c, float ph, const float4 *tA,
                                           const float2 *tB, float &fx, float &fy, float &fz) {
+    constexpr bool HAS_ACT = ACT != kActNone;
     auto term = [&](int u, float &f, float &ux, float &uy, float &uz) {
         const float4 qa = tA[g.j[u]];
         const float2 qb = tB[g.j[u]];
-        const float L = HAS_ACT ? actuated_length(c, g.a[u].y, g.s[HAS_ACT ? u : 0], ph) : g.a[u].y;
+        const float L = HAS_ACT ? actuated_length<ACT>(c, g.a[u].y, g.s[HAS_ACT ? u : 0], ph) : g.a[u].y;
         spring_terms(p, v, qa, make_float4(qa.w, qb.x, qb.y, 0.f), g.a[u].x, L, HAS_C ? g.c[HAS_C ? u : 0] : c.c_uniform,
                      f, ux, uy, uz);
     };
@@ -240,8 +255,8 @@ __device__ __forceinline__ void row_group(const Cols<COLS, HAS_C, HAS_ACT> &g, u
     }
 }
 
-template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP, int COLS>
-__global__ void __launch_bounds__(kHaloThreads, COLS > 2 ? kDeepMinBlocks : kHaloMinBlocks)
+template <bool HAS_C, int ACT, bool GROUND, bool OVERLAP, int COLS>
+__global__ void __launch_bounds__(kHaloThreads, step_min_blocks(false, ACT, COLS))
 k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n,
             const uint32_t *__restrict__ slice_off, const uint16_t *__restrict__ nslot,
             const float2 *__restrict__ kl, const float *__restrict__ cc,
@@ -249,6 +264,7 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
             const uint32_t *__restrict__ ext_off, const uint32_t *__restrict__ ext_idx,
             const uint16_t *__restrict__ ext_slot, uint32_t table_slots, uint32_t ahead, StepConst c,
             const long long *__restrict__ step_in, long long *__restrict__ step_out) {
+    constexpr bool HAS_ACT = ACT != kActNone;
     extern __shared__ float4 tab4[];
     float4 *tA = tab4;
     float2 *tB = reinterpret_cast<float2 *>(tab4 + table_slots);
@@ -272,8 +288,8 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
         e0 = __ldg(slice_off + sl);
         width = (__ldg(slice_off + sl + 1) - e0) >> 5;
     }
-    Cols<COLS, HAS_C, HAS_ACT> ga, gb;      // deep form: two groups of columns in flight
-    auto fetch = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+    Cols<COLS, HAS_C, ACT> ga, gb;      // deep form: two groups of columns in flight
+    auto fetch = [&](Cols<COLS, HAS_C, ACT> &g, uint32_t t) {
 #pragma unroll
         for (int u = 0; u < COLS; ++u) {
             if (t + u >= width) break;                  // warp-uniform; entries past the row are never used
@@ -310,11 +326,11 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
     __syncthreads();
     if (!valid) return;
 
-    const float ph = HAS_ACT ? actuation_clock(c, step) : 0.f;
+    const float ph = HAS_ACT ? actuation_clock<ACT>(c, step) : 0.f;
     float fx = 0.f, fy = 0.f, fz = 0.f;
     if (COLS > 2) {
-        auto evaluate = [&](const Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
-            row_group<COLS, HAS_C, HAS_ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
+        auto evaluate = [&](const Cols<COLS, HAS_C, ACT> &g, uint32_t t) {
+            row_group<COLS, HAS_C, ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
         };
         for (uint32_t t = 0; t < width; t += 2 * COLS) {
             evaluate(ga, t);
@@ -347,8 +363,8 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
             const float2 qb0 = tB[j0], qb1 = tB[j1];
             float L0 = a0.y, L1 = a1.y;
             if (HAS_ACT) {
-                L0 = actuated_length(c, a0.y, s0, ph);
-                L1 = actuated_length(c, a1.y, s1, ph);
+                L0 = actuated_length<ACT>(c, a0.y, s0, ph);
+                L1 = actuated_length<ACT>(c, a1.y, s1, ph);
             }
             spring_force(p, v, qa0, make_float4(qa0.w, qb0.x, qb0.y, 0.f), a0.x, L0, c0, fx, fy, fz);
             spring_force(p, v, qa1, make_float4(qa1.w, qb1.x, qb1.y, 0.f), a1.x, L1, c1, fx, fy, fz);
@@ -368,14 +384,15 @@ k_step_halo(const MassState *__restrict__ in, MassState *__restrict__ out, uint3
 // included, has L0 >= 0) may point at an empty cell of the box, whose table
 // slot holds whatever was there: they are skipped, never evaluated.  Holes -
 // device slots of empty cells, marked by own slot 0xFFFF - do nothing at all.
-template <bool HAS_C, bool HAS_ACT, bool GROUND, bool OVERLAP, int COLS>
-__global__ void __launch_bounds__(kHaloThreads, COLS > 2 ? kDeepMinBlocks : kBoxMinBlocks)
+template <bool HAS_C, int ACT, bool GROUND, bool OVERLAP, int COLS>
+__global__ void __launch_bounds__(kHaloThreads, step_min_blocks(true, ACT, COLS))
 k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n,
            const uint32_t *__restrict__ slice_off, const uint32_t *__restrict__ col_off2,
            const float2 *__restrict__ kl, const float *__restrict__ cc, const float2 *__restrict__ act,
            const uint16_t *__restrict__ own_slot, const uint32_t *__restrict__ ext_off,
            const uint32_t *__restrict__ ext_idx, const uint16_t *__restrict__ ext_slot, uint32_t table_slots,
            StepConst c, const long long *__restrict__ step_in, long long *__restrict__ step_out) {
+    constexpr bool HAS_ACT = ACT != kActNone;
     extern __shared__ float4 tab4[];
     float4 *tA = tab4;
     float2 *tB = reinterpret_cast<float2 *>(tab4 + table_slots);
@@ -410,8 +427,8 @@ k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32
             if (HAS_ACT) { ns0 = __ldcs(act + e); ns1 = __ldcs(act + e + 32); }
         }
     }
-    Cols<COLS, HAS_C, HAS_ACT> ga, gb;      // deep form: two groups of columns in flight
-    auto fetch = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+    Cols<COLS, HAS_C, ACT> ga, gb;      // deep form: two groups of columns in flight
+    auto fetch = [&](Cols<COLS, HAS_C, ACT> &g, uint32_t t) {
 #pragma unroll
         for (int u = 0; u < COLS; u += 2) {
             if (t + u >= width) break;
@@ -452,14 +469,14 @@ k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32
     __syncthreads();
     if (!valid) return;
 
-    const float ph = HAS_ACT ? actuation_clock(c, step) : 0.f;
+    const float ph = HAS_ACT ? actuation_clock<ACT>(c, step) : 0.f;
     float fx = 0.f, fy = 0.f, fz = 0.f;
     if (COLS > 2) {
         // a padding entry is evaluated against the mass itself: exactly zero
-        auto evaluate = [&](Cols<COLS, HAS_C, HAS_ACT> &g, uint32_t t) {
+        auto evaluate = [&](Cols<COLS, HAS_C, ACT> &g, uint32_t t) {
 #pragma unroll
             for (int u = 0; u < COLS; ++u) g.j[u] = g.a[u].y >= 0.f ? s_own + g.j[u] : s_own;
-            row_group<COLS, HAS_C, HAS_ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
+            row_group<COLS, HAS_C, ACT>(g, width - t, p, v, c, ph, tA, tB, fx, fy, fz);
         };
         for (uint32_t t = 0; t < width; t += 2 * COLS) {
             evaluate(ga, t);
@@ -486,8 +503,8 @@ k_step_box(const MassState *__restrict__ in, MassState *__restrict__ out, uint32
             const uint32_t j1 = s_own + (uint32_t)(int32_t)(int16_t)(o >> 16);
             float L0 = a0.y, L1 = a1.y;
             if (HAS_ACT) {
-                L0 = actuated_length(c, a0.y, s0, ph);
-                L1 = actuated_length(c, a1.y, s1, ph);
+                L0 = actuated_length<ACT>(c, a0.y, s0, ph);
+                L1 = actuated_length<ACT>(c, a1.y, s1, ph);
             }
             if (a0.y >= 0.f) {          // not padding
                 const float4 qa = tA[j0];
@@ -1208,13 +1225,14 @@ cudaError_t launch_step_halo(const MassState *in, MassState *out, uint32_t n, co
     const unsigned g = n ? (n + kHaloThreads - 1) / kHaloThreads : 1;
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
     const bool deep = deep_grid(g);
-    const int carveout = carveout_for(bytes, deep ? kDeepMinBlocks : kHaloMinBlocks);
-#define TITAN_HALO(HC, HA, GR)                                                                   \
+    const int act = ha ? (c.act_mode == 2 ? kActWorm : kActSinusoid) : kActNone;
+    const int carveout = carveout_for(bytes, step_min_blocks(false, act, deep ? kDeepCols : 2));
+#define TITAN_HALO(HC, AC, GR)                                                                   \
     do {                                                                                         \
-        auto kern = deep ? (overlap ? k_step_halo<HC, HA, GR, true, kDeepCols>                   \
-                                     : k_step_halo<HC, HA, GR, false, kDeepCols>)                 \
-                         : (overlap ? k_step_halo<HC, HA, GR, true, 2>                            \
-                                     : k_step_halo<HC, HA, GR, false, 2>);                        \
+        auto kern = deep ? (overlap ? k_step_halo<HC, AC, GR, true, kDeepCols>                   \
+                                     : k_step_halo<HC, AC, GR, false, kDeepCols>)                 \
+                         : (overlap ? k_step_halo<HC, AC, GR, true, 2>                            \
+                                     : k_step_halo<HC, AC, GR, false, 2>);                        \
         if (bytes > 48 * 1024) {                                                                 \
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
             if (e != cudaSuccess) return e;                                                      \
@@ -1237,13 +1255,15 @@ cudaError_t launch_step_halo(const MassState *in, MassState *out, uint32_t n, co
                                            h.ahead, c, step_in, step_out);                       \
         if (e != cudaSuccess) return e;                                                          \
     } while (0)
-    if (hc) {
-        if (ha) { if (gr) TITAN_HALO(true, true, true); else TITAN_HALO(true, true, false); }
-        else    { if (gr) TITAN_HALO(true, false, true); else TITAN_HALO(true, false, false); }
-    } else {
-        if (ha) { if (gr) TITAN_HALO(false, true, true); else TITAN_HALO(false, true, false); }
-        else    { if (gr) TITAN_HALO(false, false, true); else TITAN_HALO(false, false, false); }
-    }
+#define TITAN_ACT(HC, GR)                                        \
+    do {                                                         \
+        if (act == kActWorm) TITAN_HALO(HC, kActWorm, GR);       \
+        else if (act == kActSinusoid) TITAN_HALO(HC, kActSinusoid, GR); \
+        else TITAN_HALO(HC, kActNone, GR);                       \
+    } while (0)
+    if (hc) { if (gr) TITAN_ACT(true, true); else TITAN_ACT(true, false); }
+    else { if (gr) TITAN_ACT(false, true); else TITAN_ACT(false, false); }
+#undef TITAN_ACT
 #undef TITAN_HALO
     return cudaGetLastError();
 }
@@ -1256,13 +1276,14 @@ cudaError_t launch_step_box(const MassState *in, MassState *out, uint32_t n, con
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
     if (reinterpret_cast<uintptr_t>(h.col_off) & 3) return cudaErrorInvalidValue;
     const bool deep = deep_grid(g);
-    const int carveout = carveout_for(bytes, deep ? kDeepMinBlocks : kBoxMinBlocks);
-#define TITAN_BOX(HC, HA, GR)                                                                    \
+    const int act = ha ? (c.act_mode == 2 ? kActWorm : kActSinusoid) : kActNone;
+    const int carveout = carveout_for(bytes, step_min_blocks(true, act, deep ? kDeepCols : 2));
+#define TITAN_BOX(HC, AC, GR)                                                                    \
     do {                                                                                         \
-        auto kern = deep ? (overlap ? k_step_box<HC, HA, GR, true, kDeepCols>                    \
-                                     : k_step_box<HC, HA, GR, false, kDeepCols>)                  \
-                         : (overlap ? k_step_box<HC, HA, GR, true, 2>                             \
-                                     : k_step_box<HC, HA, GR, false, 2>);                         \
+        auto kern = deep ? (overlap ? k_step_box<HC, AC, GR, true, kDeepCols>                    \
+                                     : k_step_box<HC, AC, GR, false, kDeepCols>)                  \
+                         : (overlap ? k_step_box<HC, AC, GR, true, 2>                             \
+                                     : k_step_box<HC, AC, GR, false, 2>);                         \
         if (bytes > 48 * 1024) {                                                                 \
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
             if (e != cudaSuccess) return e;                                                      \
@@ -1286,13 +1307,15 @@ cudaError_t launch_step_box(const MassState *in, MassState *out, uint32_t n, con
                                            step_in, step_out);                                   \
         if (e != cudaSuccess) return e;                                                          \
     } while (0)
-    if (hc) {
-        if (ha) { if (gr) TITAN_BOX(true, true, true); else TITAN_BOX(true, true, false); }
-        else    { if (gr) TITAN_BOX(true, false, true); else TITAN_BOX(true, false, false); }
-    } else {
-        if (ha) { if (gr) TITAN_BOX(false, true, true); else TITAN_BOX(false, true, false); }
-        else    { if (gr) TITAN_BOX(false, false, true); else TITAN_BOX(false, false, false); }
-    }
+#define TITAN_ACT(HC, GR)                                        \
+    do {                                                         \
+        if (act == kActWorm) TITAN_BOX(HC, kActWorm, GR);       \
+        else if (act == kActSinusoid) TITAN_BOX(HC, kActSinusoid, GR); \
+        else TITAN_BOX(HC, kActNone, GR);                       \
+    } while (0)
+    if (hc) { if (gr) TITAN_ACT(true, true); else TITAN_ACT(true, false); }
+    else { if (gr) TITAN_ACT(false, true); else TITAN_ACT(false, false); }
+#undef TITAN_ACT
 #undef TITAN_BOX
     return cudaGetLastError();
 }
