@@ -20,11 +20,15 @@
 #include "layout.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <climits>
+#include <new>
 #include <numeric>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <utility>
 
 namespace titan {
@@ -65,6 +69,41 @@ void morton_order(const double *pos, uint32_t n, std::vector<uint32_t> &caller_o
     }
     std::sort(key.begin(), key.end());
     for (uint32_t d = 0; d < n; ++d) caller_of_dev[d] = key[d].second;
+}
+
+void component_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<uint32_t> &caller_of_dev) {
+    // disjoint sets over the springs (path halving, the lower root wins)
+    std::vector<uint32_t> root(n);
+    std::iota(root.begin(), root.end(), 0u);
+    auto find = [&](uint32_t i) {
+        while (root[i] != i) i = root[i] = root[root[i]];
+        return i;
+    };
+    for (uint32_t q = 0; q < s; ++q) {
+        const uint32_t a = find(ends[2 * (size_t)q]), b = find(ends[2 * (size_t)q + 1]);
+        if (a < b) root[b] = a;
+        else if (b < a) root[a] = b;
+    }
+    // components numbered as the order meets them; then a counting sort by number
+    std::vector<uint32_t> number(n, UINT32_MAX), size;
+    for (uint32_t d = 0; d < n; ++d) {
+        const uint32_t r = find(caller_of_dev[d]);
+        if (number[r] == UINT32_MAX) {
+            number[r] = (uint32_t)size.size();
+            size.push_back(0);
+        }
+        ++size[number[r]];
+    }
+    if (size.size() < 2) return;
+    uint32_t at = 0;
+    for (uint32_t &c : size) {          // sizes become first positions
+        const uint32_t len = c;
+        c = at;
+        at += len;
+    }
+    std::vector<uint32_t> in(std::move(caller_of_dev));
+    caller_of_dev.resize(n);
+    for (uint32_t d = 0; d < n; ++d) caller_of_dev[size[number[find(in[d])]]++] = in[d];
 }
 
 bool grid_tile_order(const double *pos, uint32_t n, double h, std::vector<uint32_t> &caller_of_dev,
@@ -284,116 +323,168 @@ bool build_halo(uint32_t n, const SellHost &sell, uint32_t max_slots, bool grid_
     out.ext_idx.clear();
     out.ext_slot.clear();
     out.max_table = 0;
-    uint64_t groups = 0, wavefronts = 0;
 
-    std::vector<uint32_t> local(n, UINT32_MAX);      // table entry of a device mass in the current block
-    std::vector<uint32_t> entries;                    // device index per table entry
-    std::vector<std::vector<uint32_t>> groups_of;     // access groups touching each entry
-    std::vector<std::vector<uint32_t>> group_members; // entries per access group (distinct)
-    std::vector<int> color;
-    for (uint32_t b = 0; b < n_blocks; ++b) {
-        const uint32_t m0 = b * kHaloBlock, m1 = std::min(n, m0 + kHaloBlock);
-        entries.clear();
-        for (uint32_t m = m0; m < m1; ++m) { local[m] = (uint32_t)entries.size(); entries.push_back(m); }
-        const uint32_t own = (uint32_t)entries.size();
-        group_members.clear();
-        // access groups: (slice, column, half-warp) -> distinct entries read
-        for (uint32_t w = 0; w < slices_per_block; ++w) {
-            const uint32_t sl = b * slices_per_block + w;
-            if (sl >= n_slices) break;
-            const uint32_t e0 = sell.slice_off[sl], width = (sell.slice_off[sl + 1] - e0) / 32;
-            for (uint32_t t = 0; t < width; ++t)
-                for (uint32_t h = 0; h < 2; ++h) {
-                    std::vector<uint32_t> g;
-                    for (uint32_t l = 16 * h; l < 16 * h + 16; ++l) {
-                        if (sl * 32 + l >= n) continue;
-                        const uint32_t j = sell.nbr[e0 + 32 * t + l];
-                        if (local[j] == UINT32_MAX) { local[j] = (uint32_t)entries.size(); entries.push_back(j); }
-                        g.push_back(local[j]);
+    // Blocks are independent: several threads each take a run of consecutive
+    // blocks, and their lists are joined in block order.  A thread holds one
+    // word per mass, 256 MB in all at most.
+    struct Part {
+        std::vector<uint32_t> ext_idx, ext_end;       // ext_end: of each block, within this part
+        std::vector<uint16_t> ext_slot;
+        uint32_t max_table = 0;
+        uint64_t groups = 0, wavefronts = 0;
+    };
+    const uint32_t nt = (uint32_t)std::max<uint64_t>(
+        1, std::min({(uint64_t)16, (uint64_t)std::max(1u, std::thread::hardware_concurrency()), (uint64_t)n_blocks / 16,
+                     ((uint64_t)256 << 20) / (4 * (uint64_t)std::max(1u, n))}));
+    std::vector<Part> parts(nt);
+    std::atomic<bool> fits{true};
+    auto build = [&](uint32_t part) {
+        Part &my = parts[part];
+        uint64_t groups = 0, wavefronts = 0;
+        std::vector<uint32_t> local(n, UINT32_MAX);      // table entry of a device mass in the current block
+        std::vector<uint32_t> entries;                    // device index per table entry
+        std::vector<std::vector<uint32_t>> groups_of;     // access groups touching each entry
+        std::vector<std::vector<uint32_t>> group_members; // entries per access group (distinct)
+        std::vector<int> color;
+        for (uint32_t b = (uint32_t)((uint64_t)n_blocks * part / nt); b < (uint32_t)((uint64_t)n_blocks * (part + 1) / nt); ++b) {
+            if (!fits.load(std::memory_order_relaxed)) return;
+            const uint32_t m0 = b * kHaloBlock, m1 = std::min(n, m0 + kHaloBlock);
+            entries.clear();
+            for (uint32_t m = m0; m < m1; ++m) { local[m] = (uint32_t)entries.size(); entries.push_back(m); }
+            const uint32_t own = (uint32_t)entries.size();
+            group_members.clear();
+            // access groups: (slice, column, half-warp) -> distinct entries read
+            for (uint32_t w = 0; w < slices_per_block; ++w) {
+                const uint32_t sl = b * slices_per_block + w;
+                if (sl >= n_slices) break;
+                const uint32_t e0 = sell.slice_off[sl], width = (sell.slice_off[sl + 1] - e0) / 32;
+                for (uint32_t t = 0; t < width; ++t)
+                    for (uint32_t h = 0; h < 2; ++h) {
+                        std::vector<uint32_t> g;
+                        for (uint32_t l = 16 * h; l < 16 * h + 16; ++l) {
+                            if (sl * 32 + l >= n) continue;
+                            const uint32_t j = sell.nbr[e0 + 32 * t + l];
+                            if (local[j] == UINT32_MAX) { local[j] = (uint32_t)entries.size(); entries.push_back(j); }
+                            g.push_back(local[j]);
+                        }
+                        std::sort(g.begin(), g.end());
+                        g.erase(std::unique(g.begin(), g.end()), g.end());
+                        if (g.size() > 1) group_members.push_back(std::move(g));
                     }
-                    std::sort(g.begin(), g.end());
-                    g.erase(std::unique(g.begin(), g.end()), g.end());
-                    if (g.size() > 1) group_members.push_back(std::move(g));
-                }
-        }
-        // the own-state writes: one group per half-warp of own masses
-        for (uint32_t h = 0; 16 * h < own; ++h) {
-            std::vector<uint32_t> g;
-            for (uint32_t l = 16 * h; l < std::min(own, 16 * h + 16); ++l) g.push_back(l);
-            if (g.size() > 1) group_members.push_back(std::move(g));
-        }
-        const uint32_t T = (uint32_t)entries.size();
-        groups_of.assign(T, {});
-        for (uint32_t gi = 0; gi < group_members.size(); ++gi)
-            for (uint32_t e : group_members[gi]) groups_of[e].push_back(gi);
-        // greedy colouring, most-constrained entries first; ties go to the least-used colour
-        std::vector<uint32_t> order(T);
-        std::iota(order.begin(), order.end(), 0u);
-        std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
-            return groups_of[x].size() > groups_of[y].size();
-        });
-        color.assign(T, -1);
-        std::vector<uint32_t> used(16, 0);
-        if (grid_colours) {
-            for (uint32_t e = 0; e < T; ++e) { color[e] = (int)(entries[e] & 15); ++used[color[e]]; }
-            order.clear();
-        }
-        for (uint32_t e : order) {
-            uint32_t cost[16] = {0};
-            for (uint32_t gi : groups_of[e])
-                for (uint32_t o : group_members[gi])
-                    if (o != e && color[o] >= 0) ++cost[color[o]];
-            int best = 0;
-            for (int c = 1; c < 16; ++c)
-                if (cost[c] < cost[best] || (cost[c] == cost[best] && used[c] < used[best])) best = c;
-            color[e] = best;
-            ++used[best];
-        }
-        uint32_t rows = 0;
-        for (int c = 0; c < 16; ++c) rows = std::max(rows, used[c]);
-        const uint32_t table = 16 * rows;
-        if (table > max_slots) {
-            for (uint32_t e = 0; e < T; ++e) local[entries[e]] = UINT32_MAX;
-            return false;
-        }
-        out.max_table = std::max(out.max_table, table);
-        std::vector<uint32_t> next_row(16, 0), slot(T);
-        for (uint32_t e = 0; e < T; ++e) slot[e] = 16 * next_row[color[e]]++ + (uint32_t)color[e];
-        for (uint32_t m = m0; m < m1; ++m) out.own_slot[m] = (uint16_t)slot[local[m]];
-        for (uint32_t e = own; e < T; ++e) {
-            out.ext_idx.push_back(entries[e]);
-            out.ext_slot.push_back((uint16_t)slot[e]);
-        }
-        out.ext_off[b + 1] = (uint32_t)out.ext_idx.size();
-        for (uint32_t w = 0; w < slices_per_block; ++w) {
-            const uint32_t sl = b * slices_per_block + w;
-            if (sl >= n_slices) break;
-            const uint32_t e0 = sell.slice_off[sl], e1 = sell.slice_off[sl + 1];
-            for (uint32_t e = e0; e < e1; ++e) {
-                const uint32_t l = (e - e0) % 32;
-                const uint32_t j = (sl * 32 + l < n) ? sell.nbr[e] : m0;
-                out.nbr_slot[e] = (uint16_t)slot[local[j]];
             }
-            // conflict statistics: wavefronts per half-warp access
-            const uint32_t width = (e1 - e0) / 32;
-            for (uint32_t t = 0; t < width; ++t)
-                for (uint32_t h = 0; h < 2; ++h) {
-                    uint32_t per_bank[16] = {0};
-                    std::vector<uint32_t> seen;
-                    for (uint32_t l = 16 * h; l < 16 * h + 16; ++l) {
-                        if (sl * 32 + l >= n) continue;
-                        const uint32_t sslot = out.nbr_slot[e0 + 32 * t + l];
-                        if (std::find(seen.begin(), seen.end(), sslot) != seen.end()) continue;
-                        seen.push_back(sslot);
-                        ++per_bank[sslot % 16];
-                    }
-                    uint32_t ways = 1;
-                    for (int c = 0; c < 16; ++c) ways = std::max(ways, per_bank[c]);
-                    wavefronts += ways;
-                    ++groups;
+            // the own-state writes: one group per half-warp of own masses
+            for (uint32_t h = 0; 16 * h < own; ++h) {
+                std::vector<uint32_t> g;
+                for (uint32_t l = 16 * h; l < std::min(own, 16 * h + 16); ++l) g.push_back(l);
+                if (g.size() > 1) group_members.push_back(std::move(g));
+            }
+            const uint32_t T = (uint32_t)entries.size();
+            groups_of.assign(T, {});
+            for (uint32_t gi = 0; gi < group_members.size(); ++gi)
+                for (uint32_t e : group_members[gi]) groups_of[e].push_back(gi);
+            // greedy colouring, most-constrained entries first; ties go to the least-used colour
+            std::vector<uint32_t> order(T);
+            std::iota(order.begin(), order.end(), 0u);
+            std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
+                return groups_of[x].size() > groups_of[y].size();
+            });
+            color.assign(T, -1);
+            std::vector<uint32_t> used(16, 0);
+            if (grid_colours) {
+                for (uint32_t e = 0; e < T; ++e) { color[e] = (int)(entries[e] & 15); ++used[color[e]]; }
+                order.clear();
+            }
+            for (uint32_t e : order) {
+                uint32_t cost[16] = {0};
+                for (uint32_t gi : groups_of[e])
+                    for (uint32_t o : group_members[gi])
+                        if (o != e && color[o] >= 0) ++cost[color[o]];
+                int best = 0;
+                for (int c = 1; c < 16; ++c)
+                    if (cost[c] < cost[best] || (cost[c] == cost[best] && used[c] < used[best])) best = c;
+                color[e] = best;
+                ++used[best];
+            }
+            uint32_t rows = 0;
+            for (int c = 0; c < 16; ++c) rows = std::max(rows, used[c]);
+            const uint32_t table = 16 * rows;
+            if (table > max_slots) {
+                fits.store(false, std::memory_order_relaxed);
+                return;
+            }
+            my.max_table = std::max(my.max_table, table);
+            std::vector<uint32_t> next_row(16, 0), slot(T);
+            for (uint32_t e = 0; e < T; ++e) slot[e] = 16 * next_row[color[e]]++ + (uint32_t)color[e];
+            for (uint32_t m = m0; m < m1; ++m) out.own_slot[m] = (uint16_t)slot[local[m]];
+            for (uint32_t e = own; e < T; ++e) {
+                my.ext_idx.push_back(entries[e]);
+                my.ext_slot.push_back((uint16_t)slot[e]);
+            }
+            my.ext_end.push_back((uint32_t)my.ext_idx.size());
+            for (uint32_t w = 0; w < slices_per_block; ++w) {
+                const uint32_t sl = b * slices_per_block + w;
+                if (sl >= n_slices) break;
+                const uint32_t e0 = sell.slice_off[sl], e1 = sell.slice_off[sl + 1];
+                for (uint32_t e = e0; e < e1; ++e) {
+                    const uint32_t l = (e - e0) % 32;
+                    const uint32_t j = (sl * 32 + l < n) ? sell.nbr[e] : m0;
+                    out.nbr_slot[e] = (uint16_t)slot[local[j]];
                 }
+                // conflict statistics: wavefronts per half-warp access
+                const uint32_t width = (e1 - e0) / 32;
+                for (uint32_t t = 0; t < width; ++t)
+                    for (uint32_t h = 0; h < 2; ++h) {
+                        uint32_t per_bank[16] = {0};
+                        std::vector<uint32_t> seen;
+                        for (uint32_t l = 16 * h; l < 16 * h + 16; ++l) {
+                            if (sl * 32 + l >= n) continue;
+                            const uint32_t sslot = out.nbr_slot[e0 + 32 * t + l];
+                            if (std::find(seen.begin(), seen.end(), sslot) != seen.end()) continue;
+                            seen.push_back(sslot);
+                            ++per_bank[sslot % 16];
+                        }
+                        uint32_t ways = 1;
+                        for (int c = 0; c < 16; ++c) ways = std::max(ways, per_bank[c]);
+                        wavefronts += ways;
+                        ++groups;
+                    }
+            }
+            for (uint32_t e = 0; e < T; ++e) local[entries[e]] = UINT32_MAX;
         }
-        for (uint32_t e = 0; e < T; ++e) local[entries[e]] = UINT32_MAX;
+        my.groups = groups;
+        my.wavefronts = wavefronts;
+    };
+    std::atomic<bool> no_memory{false};
+    auto guarded = [&](uint32_t part) {
+        try {
+            build(part);
+        } catch (const std::bad_alloc &) {
+            no_memory.store(true);
+        }
+    };
+    std::vector<std::thread> pool;
+    pool.reserve(nt);
+    for (uint32_t t = 1; t < nt; ++t) {
+        try {
+            pool.emplace_back(guarded, t);
+        } catch (const std::system_error &) {
+            guarded(t);                       // no thread to be had: on this one
+        }
+    }
+    guarded(0);
+    for (auto &th : pool) th.join();
+    if (no_memory.load()) throw std::bad_alloc();
+    if (!fits.load()) return false;
+    uint64_t groups = 0, wavefronts = 0;
+    uint32_t b = 0;
+    for (const Part &q : parts) {
+        const uint32_t base = (uint32_t)out.ext_idx.size();
+        for (uint32_t end : q.ext_end) out.ext_off[++b] = base + end;
+        out.ext_idx.insert(out.ext_idx.end(), q.ext_idx.begin(), q.ext_idx.end());
+        out.ext_slot.insert(out.ext_slot.end(), q.ext_slot.begin(), q.ext_slot.end());
+        out.max_table = std::max(out.max_table, q.max_table);
+        groups += q.groups;
+        wavefronts += q.wavefronts;
     }
     out.conflict_ways = groups ? (double)wavefronts / (double)groups : 1.0;
     return true;

@@ -15,6 +15,15 @@ namespace titan {
 // caller_of_dev[d] = caller index of the mass placed at device index d.
 void morton_order(const double *pos, uint32_t n, std::vector<uint32_t> &caller_of_dev);
 
+// Reorders caller_of_dev so that each connected component (over the springs)
+// takes consecutive device indices, components in the order they are first
+// met and each one's masses in their given order; one component changes
+// nothing.  Bodies that overlap in space, such as robots that all start at the
+// origin, are interleaved by a Morton order: a block of 256 masses then
+// touched a neighbourhood per body, no halo table fitted (4,096 slots) and the
+// step fell back to gathers without locality.
+void component_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<uint32_t> &caller_of_dev);
+
 // Grid-tile order for masses that sit on a cubic grid of pitch h (every
 // coordinate within 1e-3 h of lo + integer x h, at most one mass per cell):
 // cells are grouped in tiles of 4 x 4 x 2 and tiles in cubes of 2 x 2 x 2

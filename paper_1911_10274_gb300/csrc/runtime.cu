@@ -750,6 +750,7 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
         if (!sim->grid_order) {
             cells.clear();
             titan::morton_order(m->pos, n, sim->caller_of_dev);
+            titan::component_order(n, s, sp->ends, sim->caller_of_dev);
         }
     } else {
         sim->caller_of_dev.resize(n);
