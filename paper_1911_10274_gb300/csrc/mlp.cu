@@ -8,28 +8,26 @@
 // Network: in -> hidden -> hidden -> hidden -> 1, GELU after each hidden layer.
 //
 // GEMM kernel (k_gemm_tn): C[M, N] = A[M, K] * B[N, K]^T with A and B row-major
-// BF16 (K contiguous).  One CTA per 128 x BN output tile (BN = 64, 128 or
-// 256), optionally one K slice of it (split K), 256 threads:
+// BF16 (K contiguous; either operand may also be stored with K as its slow
+// dimension, which is how back-propagation multiplies by transposes).  One CTA
+// per 128 x BN output tile (BN = 64, 128 or 256), 512 threads:
 //   warp 0 lane 0  - TMA producer: 2-D tiled loads (128-byte swizzle) of the
 //                    A and B K-blocks (64 wide) into a 4-stage ring;
 //   warp 1 lane 0  - MMA issuer: tcgen05.mma.kind::f16 (M = 128, N = BN,
 //                    K = 16) into an FP32 accumulator in TMEM, releasing each
 //                    stage with tcgen05.commit;
-//   all 8 warps    - epilogue: tcgen05.ld of the accumulator (warp w reads
-//                    TMEM lanes 32 (w mod 4) .. + 31 = output rows, half
-//                    w / 4 of the columns), each 32 x 32 block staged in the
-//                    idle stage buffers so that global traffic runs along rows:
-//                    FP32 output, fused bias + GELU, or the GELU-derivative
-//                    product of back-propagation, with optional transposed
-//                    BF16 copies and bias-gradient column partials.
+//   all 16 warps   - epilogue, a row per lane: FP32 output, fused bias + GELU,
+//                    or the GELU-derivative product of back-propagation with
+//                    its bias-gradient column sums.
 // Every mbarrier wait is bounded (spin_limit polls); on expiry the kernel sets
 // *err, waits (bounded) for its own copies and products in flight, skips the
 // epilogue, frees its TMEM and returns.
 //
-// Training step: one CUDA graph per batch size (forward, loss, backward with
-// the weight-gradient products on a second stream, Adam), replayed by
-// titan_mlp_train_step; the learning rate and the Adam step counter live in
-// device memory so the replay needs no host values.
+// Training step: nine launches on one stream, each a programmatic dependent of
+// the one before: a copy of the batch, three forward products, the head (output
+// layer, loss, first step back), two input gradients, the three weight gradients,
+// and Adam (which adds the K slices and column sums up itself).  The learning rate
+// and the Adam step counter live in device memory.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -37,7 +35,6 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
-#include <map>
 #include <mutex>
 #include <random>
 #include <string>
@@ -55,14 +52,20 @@ namespace {
 // BM x BN output tile per CTA; BN = 64, 128 or 256 (wide tiles for large
 // products: each A tile then feeds twice the columns, halving the A traffic
 // from L2 per FLOP).
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 4;
-// 8 warps: warps 0 and 1 issue the loads and the products; after the
-// mainloop all 8 run the epilogue, warp w on TMEM lanes 32 (w mod 4) ..
-// + 31 (the lanes its quarter may read) and on half w / 4 of the columns
-constexpr int kGemmThreads = 256;
+constexpr int BM = 128, BN = 128, BK = 64;
+// 16 warps: warps 0 and 1 issue the loads and the products; after the
+// mainloop all 16 run the epilogue, warp w on TMEM lanes 32 (w mod 4) ..
+// + 31 (the lanes its quarter may read) and on quarter w / 4 of the columns,
+// 16 at a time (the GELU's arithmetic needs the warps: with 8, each epilogue
+// waited on its own instructions)
+constexpr int kGemmThreads = 512;
 constexpr uint32_t kStageA = BM * BK * 2;
 template <int BN_> constexpr uint32_t stage_b() { return (uint32_t)BN_ * BK * 2; }
-template <int BN_> constexpr size_t gemm_smem() { return (size_t)STAGES * (kStageA + stage_b<BN_>()) + 1024; }
+// Ring stages and resident CTAs per SM: two CTAs of the 64- and 128-wide tiles share
+// an SM (97 KB each), so that one's epilogue runs beside the other's products.
+template <int BN_> constexpr int stages() { return BN_ == 128 ? 3 : 4; }
+template <int BN_> constexpr int resident() { return BN_ == 256 ? 1 : 2; }
+template <int BN_> constexpr size_t gemm_smem() { return (size_t)stages<BN_>() * (kStageA + stage_b<BN_>()) + 1024; }
 
 enum Epi { EPI_F32 = 0, EPI_BIAS_GELU = 1, EPI_GELU_GRAD = 2 };
 
@@ -70,12 +73,10 @@ struct EpiArgs {
     int mode;
     int ldc;                      // row stride of the outputs (elements)
     const float *bias;            // [N]            (BIAS_GELU)
-    float *out_f32;               // [M, ldc]       (F32: C; BIAS_GELU: pre-activation Z)
+    float *out_f32;               // [M, ldc]       (F32: C; BIAS_GELU: pre-activation Z, if wanted)
     __nv_bfloat16 *out_bf16;      // [M, ldc]       (BIAS_GELU: GELU(Z); GELU_GRAD: dZ)
     const float *z;               // [M, ldc]       (GELU_GRAD: the forward pre-activation)
-    __nv_bfloat16 *out_t = nullptr;   // [N, ldt] the transpose of out_bf16, if given (BIAS_GELU, GELU_GRAD)
-    int ldt = 0;
-    float *colsum = nullptr;          // [M / 32, ldc] GELU_GRAD: per 32 rows, the column sums of out_bf16
+    float *colsum = nullptr;      // [M / 32, ldc] GELU_GRAD: per 32 rows, the column sums of out_bf16
 };
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
@@ -84,34 +85,71 @@ __device__ __forceinline__ float gelu_grad(float z) {
 }
 
 // Instruction descriptor of tcgen05.mma.kind::f16: FP32 accumulator, BF16 A
-// and B, both K-major, N = BN_, M = BM.
-template <int BN_>
+// and B, each K-major or (MN) with K as the slow dimension, N = BN_, M = BM.
+template <int BN_, bool AMN, bool BMN>
 constexpr uint32_t idesc() {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN_ >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((AMN ? 1u : 0u) << 15) | ((BMN ? 1u : 0u) << 16) |
+           ((uint32_t)(BN_ >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-template <int BN_>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-k_gemm_tn(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, int K, EpiArgs ep,
-          uint32_t spin_limit, int *__restrict__ err) {
+// 16 consecutive values of one row (one lane of an epilogue warp) as whole
+// 32-byte sectors; the row start is 32-byte aligned.
+__device__ __forceinline__ void store_row16(float *o, const float *v) {
+#pragma unroll
+    for (int x = 0; x < 16; x += 8)
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + x), "f"(v[x]), "f"(v[x + 1]),
+                     "f"(v[x + 2]), "f"(v[x + 3]), "f"(v[x + 4]), "f"(v[x + 5]), "f"(v[x + 6]), "f"(v[x + 7])
+                     : "memory");
+}
+__device__ __forceinline__ void store_row16(__nv_bfloat16 *o, const uint32_t *v) {      // 8 pairs
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+// Through L2: the row was written by an earlier kernel of the same chain.
+__device__ __forceinline__ void load_row16(const float *o, float *v) {
+#pragma unroll
+    for (int x = 0; x < 16; x += 8)
+        asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[x]), "=f"(v[x + 1]), "=f"(v[x + 2]), "=f"(v[x + 3]), "=f"(v[x + 4]), "=f"(v[x + 5]),
+                       "=f"(v[x + 6]), "=f"(v[x + 7])
+                     : "l"(o + x)
+                     : "memory");
+}
+__device__ __forceinline__ uint32_t bf16_bits(__nv_bfloat16 lo, __nv_bfloat16 hi) {
+    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+}
+
+// One 128 x BN_ tile of C = A B^T over num_kb k-blocks from k0: the whole CTA.
+// AMN / BMN: the operand is stored with K as its slow dimension (A[K][M],
+// B[K][N]); its tiles are staged as 64 x 64 boxes, one per 64 rows of the tile
+// (8 KB each, rows of K 128 bytes apart), which the tensor cores read directly:
+// back-propagation multiplies by transposes that are never formed.
+// zoff: offset of this tile's block of out_f32 (split K).
+//
+// The accumulator leaves TMEM one row per lane, 16 columns at a time, and every
+// global access of the epilogue is a lane's own whole 32-byte sectors (3 stores a
+// row of 16 instead of one per column through shared memory; no staging but for the
+// column sums).
+template <int BN_, bool AMN, bool BMN>
+__device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtensorMap *tma_b, int m0, int n0, int k0,
+                                          int num_kb, const EpiArgs &ep, size_t zoff, uint32_t spin_limit, int *err) {
+    constexpr int STAGES = stages<BN_>();
     extern __shared__ uint8_t gsm_raw[];
     __shared__ uint64_t full[STAGES], empty[STAGES], accf;
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
     __shared__ int n_issued;                          // k blocks whose TMA loads were issued
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    titan::ptx::grid_dep_launch();                    // the next kernel's prologue may overlap this one
     // 1024-byte aligned tiles (the 128-byte swizzle pattern repeats every 1024 bytes)
     const uint32_t raw = titan::ptx::smem_u32(gsm_raw);
     uint8_t *gsm = gsm_raw + (((raw + 1023u) & ~1023u) - raw);
     constexpr uint32_t kStageB = stage_b<BN_>();
     constexpr uint32_t kTmemCols = (uint32_t)BN_;      // one FP32 column per output column
+    constexpr uint32_t kBox = 64 * 128;                // bytes of a 64 x 64 box
     auto tileA = [&](int s) { return gsm + (size_t)s * (kStageA + kStageB); };
     auto tileB = [&](int s) { return gsm + (size_t)s * (kStageA + kStageB) + kStageA; };
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN_;
-    // split K (gridDim.z slices): slice z multiplies columns [z K, (z + 1) K) of A
-    // and B and writes its partial product to its own M x ldc block of out_f32
-    const int num_kb = K / BK;
-    const int k0 = (int)blockIdx.z * K;
 
     if (warp == 0) titan::ptx::tmem_alloc(&tmem_base, kTmemCols);
     if (tid == 32) {
@@ -128,18 +166,35 @@ k_gemm_tn(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUt
     __syncthreads();
     titan::ptx::tc_fence_after();
     const uint32_t taddr = tmem_base;
+    if (tid == 0) {
+        titan::ptx::prefetch_tensormap(tma_a);
+        titan::ptx::prefetch_tensormap(tma_b);
+    }
+    titan::ptx::grid_dep_wait();                      // the operands are in place
 
     if (warp == 0 && lane == 0) {                      // TMA producer
         for (int kb = 0; kb < num_kb; ++kb) {
-            const int s = kb % STAGES;
+            const int s = kb % STAGES, k = k0 + kb * BK;
             const uint32_t use = kb / STAGES;
             if (kb >= STAGES && !titan::ptx::mbar_wait_bounded(&empty[s], (use & 1) ^ 1, spin_limit)) {
                 atomicExch(&failed, 1);
                 break;
             }
             titan::ptx::mbar_arrive_expect_tx(&full[s], kStageA + kStageB);
-            titan::ptx::tma_load_2d(tileA(s), &tma_a, k0 + kb * BK, m0, &full[s]);
-            titan::ptx::tma_load_2d(tileB(s), &tma_b, k0 + kb * BK, n0, &full[s]);
+            if (AMN) {
+#pragma unroll
+                for (int j = 0; j < BM / 64; ++j)
+                    titan::ptx::tma_load_2d(tileA(s) + j * kBox, tma_a, m0 + 64 * j, k, &full[s]);
+            } else {
+                titan::ptx::tma_load_2d(tileA(s), tma_a, k, m0, &full[s]);
+            }
+            if (BMN) {
+#pragma unroll
+                for (int j = 0; j < BN_ / 64; ++j)
+                    titan::ptx::tma_load_2d(tileB(s) + j * kBox, tma_b, n0 + 64 * j, k, &full[s]);
+            } else {
+                titan::ptx::tma_load_2d(tileB(s), tma_b, k, n0, &full[s]);
+            }
             n_issued = kb + 1;
         }
     } else if (warp == 1 && lane == 0) {               // MMA issuer
@@ -155,14 +210,38 @@ k_gemm_tn(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUt
             const uint32_t a0 = titan::ptx::smem_u32(tileA(s)), b0 = titan::ptx::smem_u32(tileB(s));
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
-                titan::ptx::tc_mma_bf16(taddr, titan::ptx::smem_desc_sw128(a0 + 32 * k),
-                                        titan::ptx::smem_desc_sw128(b0 + 32 * k), idesc<BN_>(), (kb | k) != 0);
+                titan::ptx::tc_mma_bf16(taddr,
+                                        AMN ? titan::ptx::smem_desc_mn_sw128(a0 + 2048 * k, kBox)
+                                            : titan::ptx::smem_desc_sw128(a0 + 32 * k),
+                                        BMN ? titan::ptx::smem_desc_mn_sw128(b0 + 2048 * k, kBox)
+                                            : titan::ptx::smem_desc_sw128(b0 + 32 * k),
+                                        idesc<BN_, AMN, BMN>(), (kb | k) != 0);
             titan::ptx::tc_commit(&empty[s]);
         }
         titan::ptx::tc_commit(&accf);                  // fires when every issued MMA is done
     }
     __syncwarp();
-    // epilogue: every thread owns one output row (its TMEM lane)
+    // epilogue: every thread owns one output row (its TMEM lane); what its first
+    // columns need from memory is requested while the products run
+    constexpr int W = 16;                              // columns at a time
+    const int quarter = (int)(warp & 3), group = (int)(warp >> 2);
+    const int row = m0 + quarter * 32 + (int)lane;
+    float z[W];
+    auto request = [&](int col) {
+        if (ep.mode == EPI_GELU_GRAD) {
+            load_row16(ep.z + (size_t)row * ep.ldc + col, z);
+        } else if (ep.mode == EPI_BIAS_GELU) {
+#pragma unroll
+            for (int k = 0; k < W; k += 4) {
+                const float4 b = __ldcg(reinterpret_cast<const float4 *>(ep.bias + col + k));
+                z[k] = b.x;
+                z[k + 1] = b.y;
+                z[k + 2] = b.z;
+                z[k + 3] = b.w;
+            }
+        }
+    };
+    request(n0 + group * (BN_ / 4));
     const bool acc_ok = titan::ptx::mbar_wait_bounded(&accf, 0, spin_limit);
     titan::ptx::tc_fence_after();
     __syncthreads();
@@ -184,68 +263,95 @@ k_gemm_tn(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUt
         }
         __syncthreads();
     } else {
-        // The accumulator comes out of TMEM one row per lane.  Each 32 x 32
-        // block goes through this warp's scratch in the (now idle) stage
-        // buffers so that global reads and writes run along rows (lane =
-        // column, 128-byte lines), and the transposed copy, if any, along
-        // its columns (lane = row).
-        float *scr = reinterpret_cast<float *>(gsm) + warp * (32 * 33);
-        const int quarter = (int)(warp & 3), half = (int)(warp >> 2);
-        const int row0 = m0 + quarter * 32;
-        const size_t zoff = (size_t)blockIdx.z * gridDim.y * BM * ep.ldc;   // split-K slice (EPI_F32)
-        for (int c0 = half * (BN_ / 2); c0 < (half + 1) * (BN_ / 2); c0 += 32) {
-            float v[32];
-            titan::ptx::tmem_ld32(taddr + (((uint32_t)quarter * 32u) << 16) + (uint32_t)c0, v);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) scr[lane * 33 + k] = v[k];
-            __syncwarp();
-            const int col = n0 + c0 + lane;
+        const bool sectors = !(reinterpret_cast<uintptr_t>(ep.out_f32) & 31);
+        // this warp's scratch in the idle stage buffers, rows 17 (values) or 9 (pairs) words apart
+        float *scr = reinterpret_cast<float *>(gsm) + warp * (32 * (W + 1));
+#pragma unroll 1
+        for (int c0 = group * (BN_ / 4); c0 < (group + 1) * (BN_ / 4); c0 += W) {
+            float v[W];
+            titan::ptx::tmem_ld16(taddr + (((uint32_t)quarter * 32u) << 16) + (uint32_t)c0, v);
+            const int col = n0 + c0;
+            const size_t o = (size_t)row * ep.ldc + col;
             if (ep.mode == EPI_F32) {
-#pragma unroll 8
-                for (int r = 0; r < 32; ++r) ep.out_f32[zoff + (size_t)(row0 + r) * ep.ldc + col] = scr[r * 33 + lane];
-            } else {
-                if (ep.mode == EPI_BIAS_GELU) {
-                    const float b = ep.bias[col];
-#pragma unroll 8
-                    for (int r = 0; r < 32; ++r) {
-                        const size_t o = (size_t)(row0 + r) * ep.ldc + col;
-                        const float z = scr[r * 33 + lane] + b;
-                        ep.out_f32[o] = z;
-                        const __nv_bfloat16 hb = __float2bfloat16_rn(gelu(z));
-                        ep.out_bf16[o] = hb;
-                        scr[r * 33 + lane] = __bfloat162float(hb);     // exact: read back for the transpose
-                    }
+                if (sectors) {
+                    store_row16(ep.out_f32 + zoff + o, v);
                 } else {
-                    // the block's 32 rows of Z requested together, then the products;
-                    // the column sums of the BF16 results (rows in order) feed the bias gradient
-                    float zr[32];
+                    // a caller's C off the 32-byte grid: columns across the lanes, two rows a store
 #pragma unroll
-                    for (int r = 0; r < 32; ++r) zr[r] = ep.z[(size_t)(row0 + r) * ep.ldc + col];
-                    float cs = 0.f;
-#pragma unroll
-                    for (int r = 0; r < 32; ++r) {
-                        const size_t o = (size_t)(row0 + r) * ep.ldc + col;
-                        const __nv_bfloat16 hb = __float2bfloat16_rn(scr[r * 33 + lane] * gelu_grad(zr[r]));
-                        ep.out_bf16[o] = hb;
-                        const float hf = __bfloat162float(hb);
-                        cs += hf;
-                        scr[r * 33 + lane] = hf;                        // exact: read back for the transpose
-                    }
-                    if (ep.colsum) ep.colsum[(size_t)(row0 >> 5) * ep.ldc + col] = cs;
-                }
-                if (ep.out_t) {
+                    for (int k = 0; k < W; ++k) scr[lane * (W + 1) + k] = v[k];
                     __syncwarp();
 #pragma unroll 8
-                    for (int k = 0; k < 32; ++k)
-                        ep.out_t[(size_t)(n0 + c0 + k) * ep.ldt + row0 + lane] = __float2bfloat16_rn(scr[lane * 33 + k]);
+                    for (int r = (int)lane / W; r < 32; r += 32 / W)
+                        ep.out_f32[zoff + (size_t)(m0 + quarter * 32 + r) * ep.ldc + col + lane % W] =
+                            scr[r * (W + 1) + lane % W];
+                    __syncwarp();
                 }
+            } else if (ep.mode == EPI_BIAS_GELU) {
+#pragma unroll
+                for (int k = 0; k < W; ++k) v[k] += z[k];
+                if (ep.out_f32) store_row16(ep.out_f32 + o, v);
+                uint32_t h[W / 2];
+#pragma unroll
+                for (int k = 0; k < W / 2; ++k)
+                    h[k] = bf16_bits(__float2bfloat16_rn(gelu(v[2 * k])), __float2bfloat16_rn(gelu(v[2 * k + 1])));
+                store_row16(ep.out_bf16 + o, h);
+            } else {
+                uint32_t h[W / 2];
+#pragma unroll
+                for (int k = 0; k < W / 2; ++k)
+                    h[k] = bf16_bits(__float2bfloat16_rn(v[2 * k] * gelu_grad(z[2 * k])),
+                                     __float2bfloat16_rn(v[2 * k + 1] * gelu_grad(z[2 * k + 1])));
+                store_row16(ep.out_bf16 + o, h);
+                // the column sums of the 32 rows, rows in order
+                uint32_t *pairs = reinterpret_cast<uint32_t *>(scr);
+#pragma unroll
+                for (int k = 0; k < W / 2; ++k) pairs[lane * (W / 2 + 1) + k] = h[k];
+                __syncwarp();
+                float cs = 0.f;
+#pragma unroll
+                for (int r = 0; r < 32; ++r) {
+                    const uint32_t q = pairs[r * (W / 2 + 1) + (lane % W >> 1)];
+                    cs += __uint_as_float((lane & 1) ? q & 0xffff0000u : q << 16);
+                }
+                __syncwarp();
+                if (lane < W) ep.colsum[(size_t)((m0 >> 5) + quarter) * ep.ldc + col + lane] = cs;
             }
-            __syncwarp();
+            if (c0 + W < (group + 1) * (BN_ / 4)) request(col + W);
         }
     }
     titan::ptx::tc_fence_before();
     __syncthreads();
     if (warp == 0) titan::ptx::tmem_dealloc(taddr, kTmemCols);
+}
+
+// split K (gridDim.z slices): slice z multiplies k-columns [z K, (z + 1) K) of A
+// and B and writes its partial product to its own M x ldc block of out_f32.
+template <int BN_, bool AMN, bool BMN>
+__global__ void __launch_bounds__(kGemmThreads, resident<BN_>())
+k_gemm_tn(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, int K, EpiArgs ep,
+          uint32_t spin_limit, int *__restrict__ err) {
+    gemm_tile<BN_, AMN, BMN>(&tma_a, &tma_b, (int)blockIdx.y * BM, (int)blockIdx.x * BN_, (int)blockIdx.z * K, K / BK,
+                             ep, (size_t)blockIdx.z * gridDim.y * BM * ep.ldc, spin_limit, err);
+}
+
+// The three weight gradients of a step in one launch: dW_l^T (hid x in_l) =
+// dZ_l^T A_{l-1}, both operands as back-propagation left them, [batch][...], K
+// their slow dimension.  Blocks run layer by layer, K slice by K slice, tile by
+// tile; a slice's partial product lands in its own block of out[l].
+struct WgradArgs {
+    CUtensorMap a[3], b[3];
+    float *out[3];
+    int first[3], tiles[3], tiles_n[3], ld[3], kslice[3];   // first block, tiles a slice, tiles per tile row, in_l
+};
+
+__global__ void __launch_bounds__(kGemmThreads, resident<BN>())
+k_wgrad(const __grid_constant__ WgradArgs w, int hid, uint32_t spin_limit, int *__restrict__ err) {
+    const int t = (int)blockIdx.x;
+    const int l = t >= w.first[1] ? (t >= w.first[2] ? 2 : 1) : 0;
+    const int z = (t - w.first[l]) / w.tiles[l], in_slice = (t - w.first[l]) % w.tiles[l];
+    EpiArgs ep{EPI_F32, w.ld[l], nullptr, w.out[l], nullptr, nullptr};
+    gemm_tile<BN, true, true>(&w.a[l], &w.b[l], in_slice / w.tiles_n[l] * BM, in_slice % w.tiles_n[l] * BN,
+                               z * w.kslice[l], w.kslice[l] / BK, ep, (size_t)z * hid * w.ld[l], spin_limit, err);
 }
 
 // ---- large products: CTA pairs, persistent
@@ -408,240 +514,305 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
 
 // ------------------------------------------------------------------ CUDA-core kernels
 
-// out[c][r] = in[r][c] for a rows x cols BF16 matrix (32 x 32 tiles through shared memory).
-__global__ void k_transpose_bf16(const __nv_bfloat16 *__restrict__ in, __nv_bfloat16 *__restrict__ out, int rows,
-                                 int cols) {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += 8) {
-        const int r = by + k, c = bx + threadIdx.x;
-        if (r < rows && c < cols) t[k][threadIdx.x] = in[(size_t)r * cols + c];
-    }
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += 8) {
-        const int c = bx + k, r = by + threadIdx.x;
-        if (r < rows && c < cols) out[(size_t)c * rows + r] = t[threadIdx.x][k];
-    }
-}
-
-// out[c][r] = in[r][c] for a rows x cols BF16 matrix, both multiples of 64
-// and 16-byte aligned: 64 x 64 tiles, 16-byte global loads and stores (256
-// threads).  Tile rows are 37 words apart in shared memory, so the eight
-// input rows a warp gathers for one output vector fall in different banks.
-__global__ void __launch_bounds__(256) k_transpose64_bf16(const __nv_bfloat16 *__restrict__ in,
-                                                          __nv_bfloat16 *__restrict__ out, int rows, int cols) {
-    constexpr int kW = 37;                              // words per tile row (64 values + 5 words pad)
-    __shared__ uint32_t t[64 * kW];
-    const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64, tid = threadIdx.x;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int q = tid + 256 * h, r = q >> 3, seg = (q & 7) * 8;
-        const uint4 v = *reinterpret_cast<const uint4 *>(in + (size_t)(r0 + r) * cols + c0 + seg);
-        uint32_t *d = t + r * kW + seg / 2;
-        d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
-    }
-    __syncthreads();
-    const __nv_bfloat16 *tb = reinterpret_cast<const __nv_bfloat16 *>(t);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int q = tid + 256 * h, c = q >> 3, seg = (q & 7) * 8;   // output row c, input rows seg..seg+7
-        __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) o[k] = tb[(seg + k) * (2 * kW) + c];
-        *reinterpret_cast<uint4 *>(out + (size_t)(c0 + c) * rows + r0 + seg) = *reinterpret_cast<const uint4 *>(o);
-    }
-}
-
 __global__ void k_f32_to_bf16(const float *__restrict__ in, __nv_bfloat16 *__restrict__ out, size_t n) {
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i < n) out[i] = __float2bfloat16_rn(in[i]);
 }
 
+// The kernels of a pass are launched as programmatic dependents of one another:
+// each starts while the one before it drains, and touches nothing of global
+// memory before grid_dep_wait().  What an earlier kernel of the chain wrote is read
+// through L2 (an L1 line may be older than the wait).
+
+// A training step's own copy of its batch (the caller's arrays are free again
+// once it has run): n16 16-byte pieces of x, B targets.
+__global__ void k_take_batch(const uint4 *__restrict__ x, uint4 *__restrict__ gx, size_t n16, const float *__restrict__ t,
+                             float *__restrict__ gt, uint32_t B) {
+    titan::ptx::grid_dep_launch();
+    titan::ptx::grid_dep_wait();
+    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    for (size_t k = i; k < n16; k += step) gx[k] = __ldcg(x + k);
+    for (size_t k = i; k < B; k += step) gt[k] = __ldcg(t + k);
+}
+
+// This warp's dot product of a BF16 row of H with w, the same on every lane.
+__device__ __forceinline__ float row_dot(const __nv_bfloat16 *H, const float *w, int cols, uint32_t lane) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int c = (int)lane; c < cols; c += 32)
+        s += __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short *>(H) + c))) * __ldcg(w + c);
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // y[b] = H[b, :] . w + bias (one warp per row).
 __global__ void k_out_layer(const __nv_bfloat16 *__restrict__ H, const float *__restrict__ w, const float *__restrict__ b,
                             float *__restrict__ y, int rows, int cols) {
+    titan::ptx::grid_dep_launch();
+    titan::ptx::grid_dep_wait();
     const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
     if (row >= rows) return;
-    float s = 0.f;
-    for (int c = lane; c < cols; c += 32) s += __bfloat162float(H[(size_t)row * cols + c]) * w[c];
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) y[row] = s + b[0];
+    const float s = row_dot(H + (size_t)row * cols, w, cols, lane);
+    if (lane == 0) y[row] = s + __ldcg(b);
 }
 
-constexpr int kLossThreads = 1024;
+// The head of a training pass, a block per kHeadRows rows: the output layer's y,
+// diff = y - t, dy = 2 diff / B, and from them per column
+//   part[c]   = sum of dy H[., c]          (the block's share of dw4)
+//   dZ[b, c]  = dy w4[c] GELU'(Z[b, c])    in BF16
+//   part_b[c] = sum of that dZ             (of the last hidden layer's db)
+// every sum in row order; the blocks' shares are added where they are used.  It
+// replaces four kernels (output layer, loss in one block, backward by columns,
+// transpose) that passed y and dy through memory; what bounds it is the GELU
+// derivative's arithmetic.
+constexpr int kHeadRows = 32, kHeadThreads = 512;
 
-// dy = 2 (y - t) / B and the mean-squared error (one block, fixed order).
-// The output bias's gradient db = sum_b dy[b] is reduced alongside, in the
-// same fixed order.
-// tick (training steps only): the device Adam step counter, advanced here.
-__global__ void k_loss(const float *__restrict__ y, const float *__restrict__ t, float *__restrict__ dy,
-                       float *__restrict__ loss, int B, float *__restrict__ db, unsigned long long *__restrict__ tick) {
-    __shared__ float part[kLossThreads], pdb[kLossThreads];
-    float s = 0.f, sd = 0.f;
-#pragma unroll 8
-    for (int i = threadIdx.x; i < B; i += kLossThreads) {
-        const float d = y[i] - t[i];
-        const float g = 2.f * d / (float)B;
-        dy[i] = g;
-        s += d * d;
-        sd += g;
+__global__ void __launch_bounds__(kHeadThreads, 2)
+k_head(const __nv_bfloat16 *__restrict__ H, const float *__restrict__ Z, const float *__restrict__ t,
+       const float *__restrict__ w, const float *__restrict__ b, int B, int cols, __nv_bfloat16 *__restrict__ dZ,
+       float *__restrict__ part, float *__restrict__ part_b, float *__restrict__ diff,
+       unsigned long long *__restrict__ tick) {
+    __shared__ float s_dy[kHeadRows];
+    titan::ptx::grid_dep_launch();
+    titan::ptx::grid_dep_wait();
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t b0 = (size_t)blockIdx.x * kHeadRows;
+#pragma unroll
+    for (uint32_t r = warp; r < kHeadRows; r += kHeadThreads / 32) {
+        const float s = row_dot(H + (b0 + r) * cols, w, cols, lane);
+        if (lane == 0) {
+            const float d = s + __ldcg(b) - __ldcg(t + b0 + r);
+            s_dy[r] = 2.f * d / (float)B;
+            diff[b0 + r] = d;
+        }
     }
-    part[threadIdx.x] = s;
-    pdb[threadIdx.x] = sd;
     __syncthreads();
-    for (int o = kLossThreads / 2; o; o >>= 1) {
-        if (threadIdx.x < o) {
-            part[threadIdx.x] += part[threadIdx.x + o];
-            pdb[threadIdx.x] += pdb[threadIdx.x + o];
+    if (tick && blockIdx.x == 0 && tid == 0) atomicAdd(tick, 1ull);   // the Adam step counter (in L2), read by later kernels
+    for (int c = (int)tid; c < cols; c += kHeadThreads) {
+        const float wc = __ldcg(w + c);
+        float s = 0.f, sb = 0.f;
+#pragma unroll 1
+        for (int r0 = 0; r0 < kHeadRows; r0 += 16) {           // 16 rows' loads in flight
+            float hv[16], zv[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const size_t o = (b0 + r0 + r) * cols + c;
+                hv[r] = __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short *>(H) + o)));
+                zv[r] = __ldcg(Z + o);
+            }
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const float d = s_dy[r0 + r];
+                s += d * hv[r];
+                const __nv_bfloat16 g = __float2bfloat16_rn(d * wc * gelu_grad(zv[r]));
+                dZ[(b0 + r0 + r) * cols + c] = g;
+                sb += __bfloat162float(g);
+            }
+        }
+        part[(size_t)blockIdx.x * cols + c] = s;
+        part_b[(size_t)blockIdx.x * cols + c] = sb;
+    }
+}
+
+// The sum over chunks of part[k][c0 + x] for the 32 columns from c0, in a fixed
+// order: for each j < 32 the chunks j, j + 32, ... in turn, then those 32 sums
+// pairwise (256 threads, thread 32 q + x taking j = q, q + 8, q + 16, q + 24).
+// Returned to threads 0 .. 31.
+__device__ __forceinline__ float column_sum(const float *part, int chunks, int cols, int c0, float (*s)[33]) {
+    const int x = threadIdx.x & 31, q = threadIdx.x >> 5;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    int k = q;
+    for (; k + 120 < chunks; k += 128) {              // 16 loads in flight
+        float p[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p[u] = __ldcg(part + (size_t)(k + 8 * u) * cols + c0 + x);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u & 3] += p[u];
+    }
+    for (; k < chunks; k += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k + 8 * u < chunks) v[u] += __ldcg(part + (size_t)(k + 8 * u) * cols + c0 + x);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[q + 8 * u][x] = v[u];
+    __syncthreads();
+    for (int o = 16; o; o >>= 1) {
+        for (int j = q; j < o; j += 8) s[j][x] += s[j + o][x];
+        __syncthreads();
+    }
+    return s[0][x];
+}
+
+// The sums of diff^2 (x) and dy = 2 diff / B (y) over the batch in a fixed order: for
+// each i < 1,024 the rows i, i + 1,024, ... in turn, then those sums pairwise.
+__device__ __forceinline__ float2 loss_sum(const float *diff, uint32_t B, float2 *s) {
+    float2 v[4] = {};
+    for (uint32_t k0 = threadIdx.x; k0 < B; k0 += 4096) {
+        float d[16];                                  // all in flight before the first division
+#pragma unroll
+        for (int j = 0; j < 16; ++j) d[j] = k0 + 256 * j < B ? __ldcg(diff + k0 + 256 * j) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (k0 + 256 * j < B) {
+                v[j & 3].x += d[j] * d[j];
+                v[j & 3].y += 2.f * d[j] / (float)B;
+            }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[threadIdx.x + 256 * u] = v[u];
+    __syncthreads();
+    for (uint32_t o = 512; o; o >>= 1) {
+        for (uint32_t i = threadIdx.x; i < o; i += 256) {
+            s[i].x += s[i + o].x;
+            s[i].y += s[i + o].y;
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        if (loss) *loss = part[0] / (float)B;
-        if (db) *db = pdb[0];
-        if (tick) *tick += 1;
-    }
+    return s[0];
 }
 
-// Column reductions over the batch run in two fixed-order stages so that the
-// whole GPU takes part: stage one sums chunks of kRowChunk rows per column
-// (grid: column blocks x row chunks), stage two adds the chunk sums in order.
-constexpr int kRowChunk = 32;
-
-// Output layer backward, stage one: per (chunk, column) the partial of
-// dw[c] = sum_b dy[b] H[b, c]; elementwise dZ[b, c] = dy[b] w[c] GELU'(Z[b, c])
-// in BF16; and per (chunk, column) the partial column sum of that BF16 dZ
-// (the last hidden layer's bias gradient).
-__global__ void k_out_backward(const __nv_bfloat16 *__restrict__ H, const float *__restrict__ Z, const float *__restrict__ dy,
-                               const float *__restrict__ w, float *__restrict__ part, __nv_bfloat16 *__restrict__ dZ,
-                               float *__restrict__ part_b, int B, int cols) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
-    if (c >= cols) return;
-    const int b0 = k * kRowChunk;               // B is a multiple of 128: every chunk is whole
-    const float wc = w[c];
-    // the chunk's loads first (all in flight together), then the arithmetic
-    float hv[kRowChunk], zv[kRowChunk];
-#pragma unroll
-    for (int r = 0; r < kRowChunk; ++r) {
-        const size_t o = (size_t)(b0 + r) * cols + c;
-        hv[r] = __bfloat162float(H[o]);
-        zv[r] = Z[o];
-    }
-    float s = 0.f, sb = 0.f;
-#pragma unroll
-    for (int r = 0; r < kRowChunk; ++r) {
-        const float d = dy[b0 + r];
-        s += d * hv[r];
-        const __nv_bfloat16 g = __float2bfloat16_rn(d * wc * gelu_grad(zv[r]));
-        dZ[(size_t)(b0 + r) * cols + c] = g;
-        sb += __bfloat162float(g);
-    }
-    part[(size_t)k * cols + c] = s;
-    part_b[(size_t)k * cols + c] = sb;
-}
-
-// Stage two: out[c] = the sum over chunks of part[k][c], in a fixed order:
-// thread (c, j) of a 32 x 32 block adds chunks j, j + 32, ... in turn, then
-// the 32 partial sums of a column are added pairwise in a fixed tree.
-__global__ void __launch_bounds__(1024) k_col_sum_final(const float *__restrict__ part, int chunks, int cols,
-                                                        float *__restrict__ out) {
-    __shared__ float t[32][33];
-    const int c = blockIdx.x * 32 + threadIdx.x, j = threadIdx.y;
-    float s = 0.f;
-    if (c < cols) {
-#pragma unroll 4
-        for (int k = j; k < chunks; k += 32) s += part[(size_t)k * cols + c];
-    }
-    t[j][threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 16; o; o >>= 1) {
-        if (j < o) t[j][threadIdx.x] += t[j + o][threadIdx.x];
-        __syncthreads();
-    }
-    if (j == 0 && c < cols) out[c] = t[0][threadIdx.x];
-}
-
-// out[i] = sum over z of part[z][i], z in order (a split-K product's
-// slices); four entries per thread (n a multiple of 4, arrays 16-byte aligned).
-__global__ void k_sum_splits(float *__restrict__ out, const float *__restrict__ part, int splits, size_t n) {
-    const size_t i = 4 * (blockIdx.x * (size_t)blockDim.x + threadIdx.x);
-    if (i >= n) return;
-    float4 s = *reinterpret_cast<const float4 *>(part + i);
-    for (int z = 1; z < splits; ++z) {
-        const float4 q = *reinterpret_cast<const float4 *>(part + (size_t)z * n + i);
-        s.x += q.x; s.y += q.y; s.z += q.z; s.w += q.w;
-    }
-    *reinterpret_cast<float4 *>(out + i) = s;
-}
-
-// Adam (beta1, beta2, eps; bias corrections c1 = 1 - b1^t, c2 = 1 - b2^t)
-// on parameter i: updates m, v and p, returns the new p.
+// What the gradients are formed from, and Adam's state.  Weights: the K slices'
+// partial products of each layer; vectors (b1, b2, b3, w4): sums by column of 32 rows
+// each; loss and b4: the head's y - t.
+struct GradArgs {
+    const float *part[3];                 // [splits][hid][in_l]
+    uint32_t off[3], n[3];                // parameter offset and count of W_l^T
+    uint32_t splits[3], hid;
+    const float *vpart[4];
+    uint32_t voff[4];
+    const float *diff;
+    uint32_t off_b4, B;
+    float *loss;                          // may be null
+};
 struct AdamArgs {
-    float *p;
-    const float *g;
-    float *m, *v;
-    const float *lr;                      // device: a captured step reads the current rate
-    const unsigned long long *t;          // device step counter (advanced by k_loss of the same step)
+    float *p, *m, *v;
+    __nv_bfloat16 *wt[3];                 // the BF16 copies of the new weights, same layout
+    const float *lr;                      // device memory, with the step counter
+    const unsigned long long *t;
     float b1, b2, eps;
 };
 
-__device__ __forceinline__ float adam_one(const AdamArgs &a, size_t i, float c1, float c2, float lr) {
-    const float gi = a.g[i];
-    const float mi = a.b1 * a.m[i] + (1.f - a.b1) * gi;
-    const float vi = a.b2 * a.v[i] + (1.f - a.b2) * gi * gi;
-    a.m[i] = mi;
-    a.v[i] = vi;
-    const float pi = a.p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + a.eps);
-    a.p[i] = pi;
-    return pi;
+__device__ __forceinline__ float adam_one(const AdamArgs &a, float gi, float &m, float &v, float pi, float c1, float c2,
+                                          float lr) {
+    const float mi = __fmaf_rn(1.f - a.b1, gi, a.b1 * m);
+    const float vi = __fmaf_rn((1.f - a.b2) * gi, gi, a.b2 * v);
+    m = mi;
+    v = vi;
+    return pi - lr * (mi / c1) / (sqrtf(vi / c2) + a.eps);
 }
 
-// The three weight matrices W_l^T ([hid][in_l] at off_w[l], blockIdx.z = l),
-// 32 x 32 tiles: Adam on every entry, then the BF16 copies the next step's
-// products read - W^T itself (wt, same layout) and W (w, [in_l][hid], the
-// tile transposed through shared memory) - written coalesced.  Blocks of
-// blockIdx.z = 3 take the vectors (b1, b2, and b3, w4, b4: three ranges from
-// voff, of rows, rows and 2 rows + 1 entries), 256 entries per block.
-struct AdamW {
-    uint32_t off[3], cols[3];
-    __nv_bfloat16 *wt[3], *w[3];
-    uint32_t rows;
-    uint32_t voff[3];
-};
-
-__global__ void k_adam_w(AdamArgs a, AdamW W) {
-    __shared__ __nv_bfloat16 tile[32][34];
-    // the layer's fields picked without indexing the parameter block at run time
-    const uint32_t l = blockIdx.z, rows = W.rows;
-    if (l == 3) {
-        const uint32_t v = (blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.y * 32 + threadIdx.x;
-        if (v >= 4 * rows + 1) return;
-        const float tf = (float)*a.t;
-        const float c1 = 1.f - powf(a.b1, tf), c2 = 1.f - powf(a.b2, tf);
-        const uint32_t i = v < rows ? W.voff[0] + v : (v < 2 * rows ? W.voff[1] + (v - rows) : W.voff[2] + (v - 2 * rows));
-        adam_one(a, i, c1, c2, *a.lr);
+// Forms every gradient and hands it on: first blocks of 32 columns of the four
+// vectors and one for the loss and b4 (the longest chains), then blocks of 1,024
+// weights layer by layer (four per thread).  state(layer, index) requests what
+// weight(layer, index, state, gradient of four) needs besides the gradient, so that
+// it arrives together with the slices; scalar(index, gradient) takes the others.
+template <class S, class W, class V>
+__device__ __forceinline__ void for_gradients(const GradArgs &g, S &&state, W &&weight, V &&scalar) {
+    __shared__ union {
+        float col[32][33];
+        float2 loss[1024];
+    } s;
+    const uint32_t tid = threadIdx.x, per = g.hid >> 5;
+    uint32_t blk = blockIdx.x;
+    if (blk > 4 * per) {
+        blk -= 4 * per + 1;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const uint32_t blocks = g.n[l] >> 10;             // n is a multiple of 128 x 128
+            if (blk < blocks) {
+                const uint32_t i = 1024 * blk + 4 * tid, splits = g.splits[l];     // at most 8
+                const auto st = state(l, i);
+                float4 r[8];
+#pragma unroll
+                for (uint32_t z = 0; z < 8; ++z)
+                    if (z < splits) r[z] = __ldcg(reinterpret_cast<const float4 *>(g.part[l] + (size_t)z * g.n[l] + i));
+                float4 q = r[0];
+#pragma unroll
+                for (uint32_t z = 1; z < 8; ++z)              // slices in order
+                    if (z < splits) {
+                        q.x += r[z].x;
+                        q.y += r[z].y;
+                        q.z += r[z].z;
+                        q.w += r[z].w;
+                    }
+                weight(l, i, st, q);
+                return;
+            }
+            blk -= blocks;
+        }
         return;
     }
-    const uint32_t cols = l == 0 ? W.cols[0] : (l == 1 ? W.cols[1] : W.cols[2]);
-    const uint32_t off = l == 0 ? W.off[0] : (l == 1 ? W.off[1] : W.off[2]);
-    __nv_bfloat16 *const wt = l == 0 ? W.wt[0] : (l == 1 ? W.wt[1] : W.wt[2]);
-    __nv_bfloat16 *const wn = l == 0 ? W.w[0] : (l == 1 ? W.w[1] : W.w[2]);
-    const uint32_t bx = blockIdx.x * 32, by = blockIdx.y * 32;
-    if (bx >= cols || by >= rows) return;       // layers narrower than the grid
-    const float tf = (float)*a.t;
-    const float c1 = 1.f - powf(a.b1, tf), c2 = 1.f - powf(a.b2, tf), lr = *a.lr;
-    for (uint32_t k = threadIdx.y; k < 32; k += 8) {
-        const uint32_t r = by + k, c = bx + threadIdx.x;
-        const size_t o = (size_t)r * cols + c;
-        const __nv_bfloat16 h = __float2bfloat16_rn(adam_one(a, off + o, c1, c2, lr));
-        wt[o] = h;
-        tile[k][threadIdx.x] = h;
+    if (blk < 4 * per) {
+        const uint32_t k = blk / per, c0 = 32 * (blk - k * per);
+        const float *part = k == 0 ? g.vpart[0] : k == 1 ? g.vpart[1] : k == 2 ? g.vpart[2] : g.vpart[3];
+        const uint32_t off = k == 0 ? g.voff[0] : k == 1 ? g.voff[1] : k == 2 ? g.voff[2] : g.voff[3];
+        const float v = column_sum(part, (int)(g.B / 32), (int)g.hid, (int)c0, s.col);
+        if (tid < 32) scalar(off + c0 + tid, v);
+        return;
     }
-    __syncthreads();
-    for (uint32_t k = threadIdx.y; k < 32; k += 8) {
-        const uint32_t c = bx + k, r = by + threadIdx.x;
-        wn[(size_t)c * rows + r] = tile[threadIdx.x][k];
+    const float2 v = loss_sum(g.diff, g.B, s.loss);
+    if (tid == 0) {
+        if (g.loss) *g.loss = v.x / (float)g.B;
+        scalar(g.off_b4, v.y);
     }
+}
+
+struct AdamState {
+    float4 p, m, v;
+};
+
+// One Adam step on every parameter.  The slices and chunk sums are added here, in
+// registers, instead of by seven kernels through a gradient array, and four weights
+// per thread keep all of a thread's loads in flight together (24 bytes of state a
+// weight, 4 a slice, 2 for the copy: bound by L2 and HBM).
+__global__ void __launch_bounds__(256) k_adam(GradArgs g, AdamArgs a) {
+    titan::ptx::grid_dep_launch();
+    titan::ptx::grid_dep_wait();
+    const float tf = (float)__ldcg(a.t), lr = __ldcg(a.lr);
+    auto corrections = [&](float &c1, float &c2) {      // after the loads are on their way
+        c1 = 1.f - powf(a.b1, tf);
+        c2 = 1.f - powf(a.b2, tf);
+    };
+    for_gradients(
+        g,
+        [&](int l, uint32_t i) {
+            const size_t o = (size_t)g.off[l] + i;
+            return AdamState{__ldcg(reinterpret_cast<float4 *>(a.p + o)), __ldcg(reinterpret_cast<float4 *>(a.m + o)),
+                             __ldcg(reinterpret_cast<float4 *>(a.v + o))};
+        },
+        [&](int l, uint32_t i, const AdamState &st, float4 q) {
+            const size_t o = (size_t)g.off[l] + i;
+            float4 p = st.p, m = st.m, v = st.v;
+            float c1, c2;
+            corrections(c1, c2);
+            p.x = adam_one(a, q.x, m.x, v.x, p.x, c1, c2, lr);
+            p.y = adam_one(a, q.y, m.y, v.y, p.y, c1, c2, lr);
+            p.z = adam_one(a, q.z, m.z, v.z, p.z, c1, c2, lr);
+            p.w = adam_one(a, q.w, m.w, v.w, p.w, c1, c2, lr);
+            *reinterpret_cast<float4 *>(a.m + o) = m;
+            *reinterpret_cast<float4 *>(a.v + o) = v;
+            *reinterpret_cast<float4 *>(a.p + o) = p;
+            *reinterpret_cast<uint2 *>(a.wt[l] + i) =
+                make_uint2(bf16_bits(__float2bfloat16_rn(p.x), __float2bfloat16_rn(p.y)),
+                           bf16_bits(__float2bfloat16_rn(p.z), __float2bfloat16_rn(p.w)));
+        },
+        [&](size_t i, float q) {
+            float m = __ldcg(a.m + i), v = __ldcg(a.v + i), c1, c2;
+            corrections(c1, c2);
+            a.p[i] = adam_one(a, q, m, v, __ldcg(a.p + i), c1, c2, lr);
+            a.m[i] = m;
+            a.v[i] = v;
+        });
+}
+
+// The same gradients into the flat array out.
+__global__ void __launch_bounds__(256) k_form_gradient(GradArgs g, float *__restrict__ out) {
+    titan::ptx::grid_dep_launch();
+    titan::ptx::grid_dep_wait();
+    for_gradients(
+        g, [](int, uint32_t) { return 0; },
+        [&](int l, uint32_t i, int, float4 q) { *reinterpret_cast<float4 *>(out + g.off[l] + i) = q; },
+        [&](size_t i, float q) { out[i] = q; });
 }
 
 // ------------------------------------------------------------------ host helpers
@@ -663,7 +834,7 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Tensor map of a row-major [rows, cols] BF16 matrix read in 64 x 128 boxes.
+// Tensor map of a row-major [rows, cols] BF16 matrix read in boxes of box_rows rows of 64.
 bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows = 128) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
@@ -676,23 +847,45 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// C[M, N] = A[M, K] B[N, K]^T with the given epilogue.  M, N multiples of 128,
-// K a multiple of 64; A, B 16-byte aligned with row strides of K elements.
-template <int BN_>
-cudaError_t gemm_tn_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, const EpiArgs &ep,
-                           cudaStream_t st, uint32_t spin_limit, int *err, int splits = 1) {
-    static std::atomic<uint64_t> attr_set{0};
+// Launches kern as a programmatic dependent of the operation before it on st (it
+// may start early and waits in grid_dep_wait).
+template <typename... Par, typename... Arg>
+cudaError_t launch_dependent(void (*kern)(Par...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Arg &&...arg) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Arg>(arg)...);
+}
+
+// The dynamic shared memory of a GEMM kernel, allowed once per device.
+template <typename Kern>
+cudaError_t allow_smem(Kern kern, size_t bytes, std::atomic<uint64_t> &set) {
     int dev = 0;
     cudaGetDevice(&dev);
-    if (!(attr_set.load() & (1ull << (dev & 63)))) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<BN_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gemm_smem<BN_>());
-        if (e != cudaSuccess) return e;
-        attr_set.fetch_or(1ull << (dev & 63));
-    }
-    dim3 grid(N / BN_, M / BM, splits);
-    k_gemm_tn<BN_><<<grid, kGemmThreads, gemm_smem<BN_>(), st>>>(ma, mb, K / splits, ep, spin_limit, err);
-    return cudaGetLastError();
+    if (set.load() & (1ull << (dev & 63))) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) set.fetch_or(1ull << (dev & 63));
+    return e;
+}
+
+// C[M, N] = A B^T with the given epilogue; A is [M, K], B [N, K] or, with BMN,
+// [K, N].  M, N multiples of 128, K a multiple of 64; A, B 16-byte aligned, rows
+// contiguous.
+template <int BN_, bool BMN>
+cudaError_t gemm_tn_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, const EpiArgs &ep,
+                           cudaStream_t st, uint32_t spin_limit, int *err) {
+    static std::atomic<uint64_t> set{0};
+    const auto kern = k_gemm_tn<BN_, false, BMN>;
+    cudaError_t e = allow_smem(kern, gemm_smem<BN_>(), set);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(kern, dim3(N / BN_, M / BM), kGemmThreads, gemm_smem<BN_>(), st, ma, mb, K, ep, spin_limit, err);
 }
 
 cudaError_t gemm_pair_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, const EpiArgs &ep,
@@ -715,38 +908,42 @@ cudaError_t gemm_pair_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M
     return cudaLaunchKernelEx(&cfg, k_gemm_pair, ma, mb, K, tm, tn, ep.ldc, ep.out_f32, spin_limit, err);
 }
 
-// splits > 1 (EPI_F32 only): K is cut into `splits` equal slices, each a
-// multiple of BK, whose partial products land in consecutive M x ldc blocks of
-// ep.out_f32 (the caller sums them, k_sum_splits).
+template <bool BMN = false>
 cudaError_t gemm_tn(const void *A, const void *B, int M, int N, int K, const EpiArgs &ep, cudaStream_t st,
-                    uint32_t spin_limit, int *err, int splits = 1) {
+                    uint32_t spin_limit, int *err) {
     if (M % BM || N % BN || K % BK || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-    if (splits < 1 || (splits > 1 && (ep.mode != EPI_F32 || (K / splits) % BK || K % splits)))
-        return cudaErrorInvalidValue;
     if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return cudaErrorInvalidValue;
-    // 256-wide tiles once there are at least two waves of them on 152 SMs;
-    // 64-wide tiles when 128-wide ones (split-K slices included) would not
-    // fill one wave: twice the CTAs, two resident per SM (97 KB of shared
-    // memory each), so one CTA's epilogue overlaps another's products
-    const int64_t tiles128 = (int64_t)(N / 128) * (M / BM) * splits;
-    const bool wide = splits == 1 && N % 256 == 0 && (int64_t)(N / 256) * (M / BM) >= 2 * 152;
+    // 64-wide tiles when 128-wide ones would not fill one wave of 152 SMs; 256-wide
+    // ones for plain products once there are at least two waves of them (with a GELU in
+    // the epilogue, 128-wide tiles at two CTAs per SM hide it: hidden layer of 512 at a
+    // batch of 32,768, K = 512: 57 -> 46 us)
+    const int64_t tiles128 = (int64_t)(N / 128) * (M / BM);
+    const bool wide = ep.mode == EPI_F32 && N % 256 == 0 && (int64_t)(N / 256) * (M / BM) >= 2 * 152;
     const bool narrow = !wide && tiles128 <= 152;
     CUtensorMap ma, mb;
+    if (!make_map(&ma, A, M, K)) return cudaErrorInvalidValue;
     // CTA pairs once every pair of SMs has a tile of its own; the epilogue
     // writes whole 32-byte sectors
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (splits == 1 && ep.mode == EPI_F32 && M % kPairTile == 0 && N % kPairTile == 0 &&
+    if (!BMN && ep.mode == EPI_F32 && M % kPairTile == 0 && N % kPairTile == 0 &&
         (int64_t)(M / kPairTile) * (N / kPairTile) >= sms / 2 && !(reinterpret_cast<uintptr_t>(ep.out_f32) & 31)) {
-        if (!make_map(&ma, A, M, K) || !make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
+        if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
         return gemm_pair_launch(ma, mb, M, N, K, ep, st, spin_limit, err, sms);
     }
-    if (!make_map(&ma, A, M, K) || !make_map(&mb, B, N, K, wide ? 256 : (narrow ? 64 : 128)))
+    if (!(BMN ? make_map(&mb, B, K, N, 64) : make_map(&mb, B, N, K, wide ? 256 : (narrow ? 64 : 128))))
         return cudaErrorInvalidValue;
-    if (wide) return gemm_tn_launch<256>(ma, mb, M, N, K, ep, st, spin_limit, err);
-    if (narrow) return gemm_tn_launch<64>(ma, mb, M, N, K, ep, st, spin_limit, err, splits);
-    return gemm_tn_launch<128>(ma, mb, M, N, K, ep, st, spin_limit, err, splits);
+    if (wide) return gemm_tn_launch<256, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
+    if (narrow) return gemm_tn_launch<64, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
+    return gemm_tn_launch<128, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
+}
+
+cudaError_t wgrad_launch(const WgradArgs &w, int blocks, int hid, cudaStream_t st, uint32_t spin_limit, int *err) {
+    static std::atomic<uint64_t> set{0};
+    cudaError_t e = allow_smem(k_wgrad, gemm_smem<BN>(), set);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_wgrad, dim3(blocks), kGemmThreads, gemm_smem<BN>(), st, w, hid, spin_limit, err);
 }
 
 inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -765,33 +962,23 @@ struct titan_mlp {
     // parameters: [W1t (hid x in), b1, W2t (hid x hid), b2, W3t, b3, w4 (hid), b4 (1)]
     size_t off_w[3] = {0, 0, 0}, off_b[3] = {0, 0, 0}, off_w4 = 0, off_b4 = 0;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    __nv_bfloat16 *wt[3] = {nullptr, nullptr, nullptr};   // BF16 W^T (out x in): forward B operand
-    __nv_bfloat16 *w[3] = {nullptr, nullptr, nullptr};    // BF16 W (in x out): backward B operand
+    // BF16 W^T [hid][in_l]: B operand of the forward product and, read with hid as
+    // its K, of the input gradient
+    __nv_bfloat16 *wt[3] = {nullptr, nullptr, nullptr};
     uint32_t cap = 0;                                      // batch capacity of the activations
     float *Z[3] = {nullptr, nullptr, nullptr};
     __nv_bfloat16 *H[3] = {nullptr, nullptr, nullptr};
     __nv_bfloat16 *dZ[3] = {nullptr, nullptr, nullptr};
-    // transposes for the weight gradients: x^T, H_0^T and H_1^T (written by
-    // the forward products' epilogues), dZ_l^T (one buffer, layer by layer)
-    __nv_bfloat16 *xT = nullptr, *HT[2] = {nullptr, nullptr}, *bT = nullptr, *bT2 = nullptr;
-    // the weight-gradient products run on a second stream beside the
-    // input-gradient products (fork and join events per layer)
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork[3] = {nullptr, nullptr, nullptr}, ev_join[3] = {nullptr, nullptr, nullptr};
-    float *y = nullptr, *dy = nullptr;
-    float *part = nullptr;                                 // column-reduction chunk sums [B / kRowChunk][hidden]
-    float *partb = nullptr;                                // the same for the bias gradient of one layer
-    float *wsk = nullptr;                                  // split-K partial weight gradients [splits][hid][in]
+    float *part = nullptr;                                 // dw4: sums of 32 rows [B / 32][hidden]
+    float *partb[3] = {nullptr, nullptr, nullptr};         // the same for db_l
+    float *diff = nullptr;                                 // y - t
+    float *wsk = nullptr;                                  // K slices of the weight gradients
     size_t wsk_cap = 0;                                    // floats
+    volatile int *err_host = nullptr;                      // bounded-wait flag: pinned, mapped
     int *err = nullptr;
-    // the training step replayed as one CUDA graph per batch size: it reads its
-    // batch from gx / gt (the caller's arrays are copied there first) and the
-    // learning rate and step count from device memory
-    cudaStream_t capture = nullptr;
-    std::map<uint32_t, cudaGraphExec_t> train_graph;
-    bool graphs_ok = true;
+    // a training step's own copy of its batch, learning rate and step count
     __nv_bfloat16 *gx = nullptr;
-    float *gt = nullptr, *gloss = nullptr, *d_lr = nullptr;
+    float *gt = nullptr, *d_lr = nullptr;
     unsigned long long *d_step = nullptr;
     uint32_t g_cap = 0;
     float lr_set = -1.f;
@@ -840,34 +1027,12 @@ int wgrad_splits(uint32_t hid, uint32_t in, uint32_t B) {
     return s;
 }
 
-// Refreshes both BF16 layouts of the hidden-layer weights from the FP32 master.
+// Refreshes the BF16 hidden-layer weights from the FP32 master.
 cudaError_t refresh_bf16(titan_mlp *m) {
     for (int l = 0; l < 3; ++l) {
         const size_t n = (size_t)m->hid * layer_in(m, l);
         k_f32_to_bf16<<<nblk(n, 256), 256, 0, m->stream>>>(m->p + m->off_w[l], m->wt[l], n);
-        dim3 grid(nblk(layer_in(m, l), 32), nblk(m->hid, 32));
-        k_transpose_bf16<<<grid, dim3(32, 8), 0, m->stream>>>(m->wt[l], m->w[l], (int)m->hid, (int)layer_in(m, l));
     }
-    return cudaGetLastError();
-}
-
-// One Adam step on every parameter (at the step count k_loss advanced on the
-// device) and the BF16 copies of the new weights, in one launch.
-cudaError_t adam_step(titan_mlp *m) {
-    AdamArgs a{m->p, m->g, m->m, m->v, m->d_lr, m->d_step, 0.9f, 0.999f, 1e-8f};
-    AdamW W;
-    // b1, b2 and (b3, w4, b4): the parameter layout keeps the last three contiguous
-    W.voff[0] = (uint32_t)m->off_b[0];
-    W.voff[1] = (uint32_t)m->off_b[1];
-    W.voff[2] = (uint32_t)m->off_b[2];
-    for (int l = 0; l < 3; ++l) {
-        W.off[l] = (uint32_t)m->off_w[l];
-        W.cols[l] = layer_in(m, l);
-        W.wt[l] = m->wt[l];
-        W.w[l] = m->w[l];
-    }
-    W.rows = m->hid;
-    k_adam_w<<<dim3(std::max(m->in, m->hid) / 32, m->hid / 32, 4), dim3(32, 8), 0, m->stream>>>(a, W);
     return cudaGetLastError();
 }
 
@@ -878,134 +1043,99 @@ cudaError_t ensure_batch(titan_mlp *m, uint32_t B) {
         if ((e = malloc_t(m, &m->Z[l], (size_t)B * m->hid)) != cudaSuccess) return e;
         if ((e = malloc_t(m, &m->H[l], (size_t)B * m->hid)) != cudaSuccess) return e;
         if ((e = malloc_t(m, &m->dZ[l], (size_t)B * m->hid)) != cudaSuccess) return e;
+        if ((e = malloc_t(m, &m->partb[l], (size_t)(B / 32) * m->hid)) != cudaSuccess) return e;
     }
-    if ((e = malloc_t(m, &m->xT, (size_t)B * m->in)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->HT[0], (size_t)B * m->hid)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->HT[1], (size_t)B * m->hid)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->bT, (size_t)B * m->hid)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->bT2, (size_t)B * m->hid)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->y, B)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->dy, B)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->part, (size_t)((B + kRowChunk - 1) / kRowChunk) * m->hid)) != cudaSuccess) return e;
-    if ((e = malloc_t(m, &m->partb, (size_t)((B + kRowChunk - 1) / kRowChunk) * m->hid)) != cudaSuccess) return e;
-    size_t ws = 0;
-    for (int l = 0; l < 3; ++l)
-        ws = std::max(ws, (size_t)wgrad_splits(m->hid, layer_in(m, l), B) * m->hid * layer_in(m, l));
-    if (ws > m->wsk_cap) {
-        if ((e = malloc_t(m, &m->wsk, ws)) != cudaSuccess) return e;
-        m->wsk_cap = ws;
-    }
+    if ((e = malloc_t(m, &m->part, (size_t)(B / 32) * m->hid)) != cudaSuccess) return e;
+    if ((e = malloc_t(m, &m->diff, B)) != cudaSuccess) return e;
     m->cap = B;
     return cudaSuccess;
 }
 
-// keep_t: also write H_0^T and H_1^T (the backward pass's weight gradients read them).
-cudaError_t forward_pass(titan_mlp *m, const __nv_bfloat16 *x, uint32_t B, float *y, bool keep_t = false) {
+// The slices of the weight gradients (their number depends on the batch).
+cudaError_t ensure_slices(titan_mlp *m, uint32_t B) {
+    size_t ws = 0;
+    for (int l = 0; l < 3; ++l)
+        ws += (size_t)wgrad_splits(m->hid, layer_in(m, l), B) * m->hid * layer_in(m, l);
+    if (ws <= m->wsk_cap) return cudaSuccess;
+    cudaError_t e = malloc_t(m, &m->wsk, ws);
+    if (e == cudaSuccess) m->wsk_cap = ws;
+    return e;
+}
+
+// keep: the pre-activations are written too (a backward pass follows).
+cudaError_t hidden_layers(titan_mlp *m, const __nv_bfloat16 *x, uint32_t B, bool keep) {
     cudaError_t e;
     const __nv_bfloat16 *a = x;
     for (int l = 0; l < 3; ++l) {
-        EpiArgs ep{EPI_BIAS_GELU, (int)m->hid, m->p + m->off_b[l], m->Z[l], m->H[l], nullptr};
-        if (keep_t && l < 2) {
-            ep.out_t = m->HT[l];
-            ep.ldt = (int)B;
-        }
+        EpiArgs ep{EPI_BIAS_GELU, (int)m->hid, m->p + m->off_b[l], keep ? m->Z[l] : nullptr, m->H[l], nullptr};
         if ((e = gemm_tn(a, m->wt[l], (int)B, (int)m->hid, (int)layer_in(m, l), ep, m->stream, m->spin_limit, m->err)) != cudaSuccess)
             return e;
         a = m->H[l];
     }
-    k_out_layer<<<nblk(B, 8), 256, 0, m->stream>>>(m->H[2], m->p + m->off_w4, m->p + m->off_b4, y, (int)B, (int)m->hid);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
-// train: a training step follows (k_loss advances the Adam step counter).
-cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, uint32_t B, float *loss,
-                          bool train = false) {
-    cudaError_t e = forward_pass(m, x, B, m->y, true);
-    if (e != cudaSuccess) return e;
-    k_loss<<<1, kLossThreads, 0, m->stream>>>(m->y, t, m->dy, loss, (int)B, m->g + m->off_b4,
-                                              train ? m->d_step : nullptr);
-    const int chunks = ((int)B + kRowChunk - 1) / kRowChunk;
-    k_out_backward<<<dim3(nblk(m->hid, 128), chunks), 128, 0, m->stream>>>(m->H[2], m->Z[2], m->dy, m->p + m->off_w4,
-                                                                          m->part, m->dZ[2], m->partb, (int)B,
-                                                                          (int)m->hid);
-    const dim3 cs_grid(nblk(m->hid, 32)), cs_block(32, 32);
-    k_col_sum_final<<<cs_grid, cs_block, 0, m->stream>>>(m->part, chunks, (int)m->hid, m->g + m->off_w4);
-    // dZ_l^T alternates between two buffers (layer 2 and 0: bT, layer 1: bT2),
-    // so that layer l's weight-gradient product (second stream) can read its
-    // own while the input-gradient product (this stream) writes the next
-    __nv_bfloat16 *const bt[2] = {m->bT, m->bT2};
-    k_transpose64_bf16<<<dim3(m->hid / 64, B / 64), 256, 0, m->stream>>>(m->dZ[2], bt[0], (int)B, (int)m->hid);
-    for (int l = 2; l >= 0; --l) {
-        // dW_l^T (hid x in_l) = dZ_l^T (hid x B) . A_{l-1}^T (in_l x B)^T, on the second stream
-        const uint32_t in = layer_in(m, l);
-        const __nv_bfloat16 *actT = l == 0 ? m->xT : m->HT[l - 1];
-        if (l == 0)
-            k_transpose64_bf16<<<dim3(in / 64, B / 64), 256, 0, m->stream>>>(x, m->xT, (int)B, (int)in);
-        if ((e = cudaEventRecord(m->ev_fork[l], m->stream)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(m->side, m->ev_fork[l], 0)) != cudaSuccess) return e;
-        const int splits = wgrad_splits(m->hid, in, B);
-        EpiArgs ep{EPI_F32, (int)in, nullptr, splits > 1 ? m->wsk : m->g + m->off_w[l], nullptr, nullptr};
-        if ((e = gemm_tn(bt[l & 1], actT, (int)m->hid, (int)in, (int)B, ep, m->side, m->spin_limit, m->err, splits)) !=
-            cudaSuccess)
+// Forward and backward for a batch in device memory: 7 launches on one stream, each
+// a programmatic dependent of the one before.  Leaves what the gradients are formed
+// from in *g.  train: the head advances the Adam step counter.
+cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, uint32_t B, float *loss, GradArgs *g,
+                          bool train) {
+    cudaError_t e;
+    const int hid = (int)m->hid;
+    if ((e = ensure_slices(m, B)) != cudaSuccess) return e;
+    if ((e = hidden_layers(m, x, B, true)) != cudaSuccess) return e;
+    if ((e = launch_dependent(k_head, dim3(B / kHeadRows), kHeadThreads, 0, m->stream, m->H[2], m->Z[2], t,
+                              m->p + m->off_w4, m->p + m->off_b4, (int)B, hid, m->dZ[2], m->part, m->partb[2], m->diff,
+                              train ? m->d_step : nullptr)) != cudaSuccess)
+        return e;
+    for (int l = 2; l > 0; --l) {
+        // dZ_{l-1} = (dZ_l W_l^T) * GELU'(Z_{l-1}):  A = dZ_l, B = W_l^T [hid][in] with hid as K
+        EpiArgs ep{EPI_GELU_GRAD, hid, nullptr, nullptr, m->dZ[l - 1], m->Z[l - 1], m->partb[l - 1]};
+        if ((e = gemm_tn<true>(m->dZ[l], m->wt[l], (int)B, hid, hid, ep, m->stream, m->spin_limit, m->err)) != cudaSuccess)
             return e;
-        if (splits > 1) {
-            const size_t n = (size_t)m->hid * in;
-            k_sum_splits<<<nblk(n / 4, 256), 256, 0, m->side>>>(m->g + m->off_w[l], m->wsk, splits, n);
-        }
-        if ((e = cudaEventRecord(m->ev_join[l], m->side)) != cudaSuccess) return e;
-        // db_l: the chunk sums of dZ_l's columns came with dZ_l (k_out_backward, or the
-        // epilogue of the product that formed it); the next product overwrites them
-        k_col_sum_final<<<cs_grid, cs_block, 0, m->stream>>>(m->partb, chunks, (int)m->hid, m->g + m->off_b[l]);
-        if (l > 0) {
-            // dZ_{l-1} = (dZ_l . W_l^T) * GELU'(Z_{l-1}):  A = dZ_l (B x hid), B operand = W_l (in x hid);
-            // its transpose goes to the buffer layer l + 1's weight gradient read: wait for it
-            if (l == 1 && (e = cudaStreamWaitEvent(m->stream, m->ev_join[2], 0)) != cudaSuccess) return e;
-            EpiArgs ep2{EPI_GELU_GRAD, (int)m->hid, nullptr, nullptr, m->dZ[l - 1], m->Z[l - 1]};
-            ep2.out_t = bt[(l - 1) & 1];
-            ep2.ldt = (int)B;
-            ep2.colsum = m->partb;
-            if ((e = gemm_tn(m->dZ[l], m->w[l], (int)B, (int)in, (int)m->hid, ep2, m->stream, m->spin_limit, m->err)) != cudaSuccess)
-                return e;
-        }
     }
-    // every weight gradient is in place before anything reads it (the side stream runs in order)
-    if ((e = cudaStreamWaitEvent(m->stream, m->ev_join[0], 0)) != cudaSuccess) return e;
-    return cudaGetLastError();
+    WgradArgs w;
+    int blocks = 0;
+    size_t at = 0;
+    for (int l = 0; l < 3; ++l) {
+        const uint32_t in = layer_in(m, l);
+        const int splits = wgrad_splits(m->hid, in, B);
+        if (!make_map(&w.a[l], m->dZ[l], B, m->hid, 64) || !make_map(&w.b[l], l ? m->H[l - 1] : x, B, in, 64))
+            return cudaErrorInvalidValue;
+        w.out[l] = m->wsk + at;
+        w.first[l] = blocks;
+        w.tiles_n[l] = (int)(in / BN);
+        w.tiles[l] = (int)(m->hid / BM) * w.tiles_n[l];
+        w.ld[l] = (int)in;
+        w.kslice[l] = (int)B / splits;
+        blocks += splits * w.tiles[l];
+        at += (size_t)splits * m->hid * in;
+        g->part[l] = w.out[l];
+        g->off[l] = (uint32_t)m->off_w[l];
+        g->n[l] = m->hid * in;
+        g->splits[l] = (uint32_t)splits;
+        g->vpart[l] = m->partb[l];
+        g->voff[l] = (uint32_t)m->off_b[l];
+    }
+    g->hid = m->hid;
+    g->vpart[3] = m->part;
+    g->voff[3] = (uint32_t)m->off_w4;
+    g->diff = m->diff;
+    g->off_b4 = (uint32_t)m->off_b4;
+    g->B = B;
+    g->loss = loss;
+    return wgrad_launch(w, blocks, hid, m->stream, m->spin_limit, m->err);
 }
 
-// One training step for a batch of B read from gx / gt, captured into a graph:
-// the forward and backward products, the step counter, Adam, and the BF16
-// copies of the new weights.
-cudaError_t capture_train(titan_mlp *m, uint32_t B, cudaGraphExec_t *out) {
-    cudaError_t e = cudaStreamBeginCapture(m->capture, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return e;
-    cudaStream_t saved = m->stream;
-    m->stream = m->capture;
-    cudaError_t le = backward_pass(m, m->gx, m->gt, B, m->gloss, true);
-    if (le == cudaSuccess) le = adam_step(m);
-    m->stream = saved;
-    cudaGraph_t g = nullptr;
-    e = cudaStreamEndCapture(m->capture, &g);
-    if (le != cudaSuccess || e != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return le != cudaSuccess ? le : e;
-    }
-    e = cudaGraphInstantiate(out, g, 0);
-    cudaGraphDestroy(g);
-    return e;
-}
-
-void drop_train_graphs(titan_mlp *m) {
-    for (auto &kv : m->train_graph) cudaGraphExecDestroy(kv.second);
-    m->train_graph.clear();
+// The grid of k_adam and k_form_gradient (see for_gradients).
+unsigned gradient_blocks(const GradArgs &g) {
+    return (g.n[0] >> 10) + (g.n[1] >> 10) + (g.n[2] >> 10) + 4 * (g.hid >> 5) + 1;
 }
 
 titan_status check_err(titan_mlp *m) {
-    int flag = 0;
     MLP_CK(m, cudaStreamSynchronize(m->stream));
-    MLP_CK(m, cudaMemcpy(&flag, m->err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flag) {
-        cudaMemset(m->err, 0, sizeof(int));
+    if (*m->err_host) {
+        *m->err_host = 0;
         return mfail(m, TITAN_E_TIMEOUT, "a bounded wait in the tensor-core GEMM expired");
     }
     return TITAN_OK;
@@ -1104,12 +1234,7 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     auto bail = [&](titan_status st) {
         titan::set_thread_error(m->error);
         for (void *p : m->allocs) cudaFree(p);
-        for (int l = 0; l < 3; ++l) {
-            if (m->ev_fork[l]) cudaEventDestroy(m->ev_fork[l]);
-            if (m->ev_join[l]) cudaEventDestroy(m->ev_join[l]);
-        }
-        if (m->side) cudaStreamDestroy(m->side);
-        if (m->capture) cudaStreamDestroy(m->capture);
+        if (m->err_host) cudaFreeHost(const_cast<int *>(m->err_host));
         if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
         delete m;
         return st;
@@ -1127,20 +1252,19 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     C_CK(malloc_t(m, &m->g, o));
     C_CK(malloc_t(m, &m->m, o));
     C_CK(malloc_t(m, &m->v, o));
-    C_CK(malloc_t(m, &m->err, 1));
+    {
+        void *h = nullptr, *d = nullptr;
+        C_CK(cudaHostAlloc(&h, sizeof(int), cudaHostAllocMapped));
+        m->err_host = static_cast<volatile int *>(h);
+        *m->err_host = 0;
+        C_CK(cudaHostGetDevicePointer(&d, h, 0));
+        m->err = static_cast<int *>(d);
+    }
     C_CK(malloc_t(m, &m->d_lr, 1));
-    C_CK(malloc_t(m, &m->gloss, 1));
     C_CK(malloc_t(m, &m->d_step, 1));
     C_CK(cudaMemset(m->d_step, 0, sizeof(unsigned long long)));
-    C_CK(cudaStreamCreateWithFlags(&m->capture, cudaStreamNonBlocking));
-    C_CK(cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking));
-    for (int l = 0; l < 3; ++l) {
-        C_CK(cudaEventCreateWithFlags(&m->ev_fork[l], cudaEventDisableTiming));
-        C_CK(cudaEventCreateWithFlags(&m->ev_join[l], cudaEventDisableTiming));
-    }
     for (int l = 0; l < 3; ++l) {
         C_CK(malloc_t(m, &m->wt[l], (size_t)hidden * layer_in(m, l)));
-        C_CK(malloc_t(m, &m->w[l], (size_t)hidden * layer_in(m, l)));
     }
     // He-style initialisation (uniform, variance 2 / fan_in for GELU layers), zero biases
     std::vector<float> h(o, 0.f);
@@ -1159,7 +1283,6 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     C_CK(cudaMemset(m->m, 0, o * 4));
     C_CK(cudaMemset(m->v, 0, o * 4));
     C_CK(cudaMemset(m->g, 0, o * 4));
-    C_CK(cudaMemset(m->err, 0, sizeof(int)));
     C_CK(refresh_bf16(m));
     C_CK(cudaStreamSynchronize(m->stream));
 #undef C_CK
@@ -1189,7 +1312,9 @@ titan_status titan_mlp_forward(titan_mlp *m, const uint16_t *x_dev, uint32_t bat
         return mfail(m, TITAN_E_INVALID, "titan_mlp_forward: batch must be a positive multiple of 128");
     MLP_CK(m, cudaSetDevice(m->device));
     MLP_CK(m, ensure_batch(m, batch));
-    MLP_CK(m, forward_pass(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), batch, y_dev));
+    MLP_CK(m, hidden_layers(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), batch, false));
+    MLP_CK(m, launch_dependent(k_out_layer, dim3(nblk(batch, 8)), 256, 0, m->stream, m->H[2], m->p + m->off_w4,
+                               m->p + m->off_b4, y_dev, (int)batch, (int)m->hid));
     return check_err(m);
 }
 
@@ -1199,7 +1324,9 @@ titan_status titan_mlp_gradient(titan_mlp *m, const uint16_t *x_dev, const float
         return mfail(m, TITAN_E_INVALID, "titan_mlp_gradient: batch must be a positive multiple of 128");
     MLP_CK(m, cudaSetDevice(m->device));
     MLP_CK(m, ensure_batch(m, batch));
-    MLP_CK(m, backward_pass(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), t_dev, batch, loss_dev));
+    GradArgs g;
+    MLP_CK(m, backward_pass(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), t_dev, batch, loss_dev, &g, false));
+    MLP_CK(m, launch_dependent(k_form_gradient, dim3(gradient_blocks(g)), 256, 0, m->stream, g, m->g));
     if (grad_dev) MLP_CK(m, cudaMemcpyAsync(grad_dev, m->g, m->n_params * 4, cudaMemcpyDeviceToDevice, m->stream));
     return check_err(m);
 }
@@ -1209,40 +1336,28 @@ titan_status titan_mlp_train_step(titan_mlp *m, const uint16_t *x_dev, const flo
     if (!m || !x_dev || !t_dev || batch % 128 || !batch)
         return mfail(m, TITAN_E_INVALID, "titan_mlp_train_step: batch must be a positive multiple of 128");
     MLP_CK(m, cudaSetDevice(m->device));
-    const uint32_t cap0 = m->cap;
     MLP_CK(m, ensure_batch(m, batch));
-    if (m->cap != cap0) drop_train_graphs(m);           // the activations moved
+    if (batch > m->g_cap) {
+        MLP_CK(m, malloc_t(m, &m->gx, (size_t)batch * m->in));
+        MLP_CK(m, malloc_t(m, &m->gt, batch));
+        m->g_cap = batch;
+    }
     if (lr != m->lr_set) {                              // pageable source: staged before the call returns
         MLP_CK(m, cudaMemcpyAsync(m->d_lr, &lr, sizeof(float), cudaMemcpyHostToDevice, m->stream));
         m->lr_set = lr;
     }
-    if (m->graphs_ok) {
-        if (batch > m->g_cap) {
-            drop_train_graphs(m);
-            MLP_CK(m, malloc_t(m, &m->gx, (size_t)batch * m->in));
-            MLP_CK(m, malloc_t(m, &m->gt, batch));
-            m->g_cap = batch;
-        }
-        auto it = m->train_graph.find(batch);
-        if (it == m->train_graph.end()) {
-            cudaGraphExec_t ge = nullptr;
-            if (capture_train(m, batch, &ge) == cudaSuccess) {
-                it = m->train_graph.emplace(batch, ge).first;
-            } else {                                    // capture refused: launch the kernels directly
-                cudaGetLastError();
-                m->graphs_ok = false;
-            }
-        }
-        if (m->graphs_ok) {
-            MLP_CK(m, cudaMemcpyAsync(m->gx, x_dev, (size_t)batch * m->in * 2, cudaMemcpyDeviceToDevice, m->stream));
-            MLP_CK(m, cudaMemcpyAsync(m->gt, t_dev, (size_t)batch * 4, cudaMemcpyDeviceToDevice, m->stream));
-            MLP_CK(m, cudaGraphLaunch(it->second, m->stream));
-            if (loss_dev) MLP_CK(m, cudaMemcpyAsync(loss_dev, m->gloss, 4, cudaMemcpyDeviceToDevice, m->stream));
-            return TITAN_OK;
-        }
+    size_t n16 = (size_t)batch * m->in / 8;
+    if (reinterpret_cast<uintptr_t>(x_dev) & 15) {      // a view off the 16-byte grid
+        MLP_CK(m, cudaMemcpyAsync(m->gx, x_dev, n16 * 16, cudaMemcpyDeviceToDevice, m->stream));
+        n16 = 0;
     }
-    MLP_CK(m, backward_pass(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), t_dev, batch, loss_dev, true));
-    MLP_CK(m, adam_step(m));
+    MLP_CK(m, launch_dependent(k_take_batch, dim3((unsigned)std::min<size_t>(nblk(std::max<size_t>(n16, batch), 256), 152 * 8)), 256, 0, m->stream,
+                               reinterpret_cast<const uint4 *>(x_dev), reinterpret_cast<uint4 *>(m->gx), n16, t_dev, m->gt,
+                               batch));
+    GradArgs g;
+    MLP_CK(m, backward_pass(m, m->gx, m->gt, batch, loss_dev, &g, true));
+    AdamArgs a{m->p, m->m, m->v, {m->wt[0], m->wt[1], m->wt[2]}, m->d_lr, m->d_step, 0.9f, 0.999f, 1e-8f};
+    MLP_CK(m, launch_dependent(k_adam, dim3(gradient_blocks(g)), 256, 0, m->stream, g, a));
     return TITAN_OK;
 }
 
@@ -1253,14 +1368,7 @@ const char *titan_mlp_last_error(const titan_mlp *m) { return m ? m->error.c_str
 titan_status titan_mlp_destroy(titan_mlp *m) {
     if (!m) return TITAN_OK;
     cudaStreamSynchronize(m->stream);
-    if (m->side) cudaStreamSynchronize(m->side);
-    drop_train_graphs(m);
-    for (int l = 0; l < 3; ++l) {
-        if (m->ev_fork[l]) cudaEventDestroy(m->ev_fork[l]);
-        if (m->ev_join[l]) cudaEventDestroy(m->ev_join[l]);
-    }
-    if (m->side) cudaStreamDestroy(m->side);
-    if (m->capture) cudaStreamDestroy(m->capture);
+    if (m->err_host) cudaFreeHost(const_cast<int *>(m->err_host));
     for (void *p : m->allocs) cudaFree(p);
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     delete m;

@@ -228,6 +228,25 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *out) {
     for (int k = 0; k < 32; ++k) out[k] = __uint_as_float(r[k]);
 }
 
+// The same for 16 columns.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *out) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int k = 0; k < 16; ++k) out[k] = __uint_as_float(r[k]);
+}
+
+// Starts fetching the tensor map of a later TMA load (a __grid_constant__ kernel parameter).
+__device__ __forceinline__ void prefetch_tensormap(const void *tmap) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
+}
+
 // Shared-memory matrix descriptor of a K-major tile stored with the 128-byte
 // swizzle (rows of 128 bytes, 8-row groups 1024 bytes apart).
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
@@ -235,6 +254,19 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
     d |= (uint64_t)((saddr & 0x3FFFF) >> 4);          // start address
     d |= (uint64_t)1 << 16;                            // leading byte offset (unused for this layout)
     d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset: 8 rows x 128 B
+    d |= (uint64_t)1 << 46;                            // descriptor version for tcgen05
+    d |= (uint64_t)2 << 61;                            // 128-byte swizzle
+    return d;
+}
+
+// The same for a tile with K as its slow dimension: 64 x 64 boxes of BF16 (64
+// values of M or N along a row of 128 bytes, one row per k, 128-byte swizzle),
+// `box` bytes apart along M or N; 8-row groups of k 1024 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t saddr, uint32_t box) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);          // start address
+    d |= (uint64_t)(box >> 4) << 16;                   // leading byte offset: next 64 of M or N
+    d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset: next 8 of K
     d |= (uint64_t)1 << 46;                            // descriptor version for tcgen05
     d |= (uint64_t)2 << 61;                            // 128-byte swizzle
     return d;
