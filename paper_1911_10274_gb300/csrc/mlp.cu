@@ -11,9 +11,9 @@
 // BF16 (K contiguous; either operand may also be stored with K as its slow
 // dimension, which is how back-propagation multiplies by transposes).  One CTA
 // per 128 x BN output tile (BN = 64, 128 or 256), 512 threads:
-//   warp 0 lane 0  - TMA producer: 2-D tiled loads (128-byte swizzle) of the
+//   warp 0         - TMA producer: 2-D tiled loads (128-byte swizzle) of the
 //                    A and B K-blocks (64 wide) into a 4-stage ring;
-//   warp 1 lane 0  - MMA issuer: tcgen05.mma.kind::f16 (M = 128, N = BN,
+//   warp 1         - MMA issuer: tcgen05.mma.kind::f16 (M = 128, N = BN,
 //                    K = 16) into an FP32 accumulator in TMEM, releasing each
 //                    stage with tcgen05.commit;
 //   all 16 warps   - epilogue, a row per lane: FP32 output, fused bias + GELU,
@@ -140,7 +140,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
     __shared__ int n_issued;                          // k blocks whose TMA loads were issued
-    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // known to be the same in every lane
     titan::ptx::grid_dep_launch();                    // the next kernel's prologue may overlap this one
     // 1024-byte aligned tiles (the 128-byte swizzle pattern repeats every 1024 bytes)
     const uint32_t raw = titan::ptx::smem_u32(gsm_raw);
@@ -172,53 +173,75 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
     }
     titan::ptx::grid_dep_wait();                      // the operands are in place
 
-    if (warp == 0 && lane == 0) {                      // TMA producer
-        for (int kb = 0; kb < num_kb; ++kb) {
-            const int s = kb % STAGES, k = k0 + kb * BK;
-            const uint32_t use = kb / STAGES;
-            if (kb >= STAGES && !titan::ptx::mbar_wait_bounded(&empty[s], (use & 1) ^ 1, spin_limit)) {
-                atomicExch(&failed, 1);
+    // Both issuing warps run their loops whole, on values the same in every lane, and
+    // one elected lane issues: loops of a single lane moved every descriptor, address
+    // and barrier through vector registers and were the bound themselves (528 cycles a
+    // k-block, whatever the tile).
+    if (warp == 0) {                                   // TMA producer
+        const bool leader = titan::ptx::elect_one();
+        uint32_t s = 0, parity = 1;
+        int issued = 0;
+        for (int kb = 0, k = k0; kb < num_kb; ++kb, k += BK) {
+            if (kb >= STAGES && !titan::ptx::mbar_wait_bounded(&empty[s], parity, spin_limit)) {
+                if (leader) atomicExch(&failed, 1);
                 break;
             }
-            titan::ptx::mbar_arrive_expect_tx(&full[s], kStageA + kStageB);
-            if (AMN) {
+            if (leader) {
+                titan::ptx::mbar_arrive_expect_tx(&full[s], kStageA + kStageB);
+                if (AMN) {
 #pragma unroll
-                for (int j = 0; j < BM / 64; ++j)
-                    titan::ptx::tma_load_2d(tileA(s) + j * kBox, tma_a, m0 + 64 * j, k, &full[s]);
-            } else {
-                titan::ptx::tma_load_2d(tileA(s), tma_a, k, m0, &full[s]);
-            }
-            if (BMN) {
+                    for (int j = 0; j < BM / 64; ++j)
+                        titan::ptx::tma_load_2d(tileA(s) + j * kBox, tma_a, m0 + 64 * j, k, &full[s]);
+                } else {
+                    titan::ptx::tma_load_2d(tileA(s), tma_a, k, m0, &full[s]);
+                }
+                if (BMN) {
 #pragma unroll
-                for (int j = 0; j < BN_ / 64; ++j)
-                    titan::ptx::tma_load_2d(tileB(s) + j * kBox, tma_b, n0 + 64 * j, k, &full[s]);
-            } else {
-                titan::ptx::tma_load_2d(tileB(s), tma_b, k, n0, &full[s]);
+                    for (int j = 0; j < BN_ / 64; ++j)
+                        titan::ptx::tma_load_2d(tileB(s) + j * kBox, tma_b, n0 + 64 * j, k, &full[s]);
+                } else {
+                    titan::ptx::tma_load_2d(tileB(s), tma_b, k, n0, &full[s]);
+                }
             }
-            n_issued = kb + 1;
+            __syncwarp();
+            issued = kb + 1;
+            if (++s == STAGES) {
+                s = 0;
+                parity ^= 1;
+            }
         }
-    } else if (warp == 1 && lane == 0) {               // MMA issuer
-        bool ok = true;
-        for (int kb = 0; kb < num_kb && ok; ++kb) {
-            const int s = kb % STAGES;
-            if (!titan::ptx::mbar_wait_bounded(&full[s], (kb / STAGES) & 1, spin_limit)) {
-                atomicExch(&failed, 1);
-                ok = false;
+        if (leader) n_issued = issued;
+    } else if (warp == 1) {                            // MMA issuer
+        const bool leader = titan::ptx::elect_one();
+        // the descriptors of stage 0, moved by an addition (a stage, or 16 of K, in units of 16 bytes)
+        uint64_t a = AMN ? titan::ptx::smem_desc_mn_sw128(titan::ptx::smem_u32(tileA(0)), kBox)
+                         : titan::ptx::smem_desc_sw128(titan::ptx::smem_u32(tileA(0)));
+        uint64_t b = BMN ? titan::ptx::smem_desc_mn_sw128(titan::ptx::smem_u32(tileB(0)), kBox)
+                         : titan::ptx::smem_desc_sw128(titan::ptx::smem_u32(tileB(0)));
+        constexpr uint32_t kStep = (kStageA + kStageB) >> 4, kStepA = (AMN ? 2048 : 32) >> 4, kStepB = (BMN ? 2048 : 32) >> 4;
+        uint32_t s = 0, parity = 0;
+        bool ready = false;                            // this k-block was seen to have arrived
+        for (int kb = 0; kb < num_kb; ++kb) {
+            if (!ready && !titan::ptx::mbar_wait_bounded(&full[s], parity, spin_limit)) {
+                if (leader) atomicExch(&failed, 1);
                 break;
             }
             titan::ptx::tc_fence_after();
-            const uint32_t a0 = titan::ptx::smem_u32(tileA(s)), b0 = titan::ptx::smem_u32(tileB(s));
+            const uint32_t s1 = s + 1 == STAGES ? 0 : s + 1, parity1 = parity ^ (s1 == 0);
+            ready = kb + 1 < num_kb && titan::ptx::mbar_test(&full[s1], parity1);
+            if (leader) {
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-                titan::ptx::tc_mma_bf16(taddr,
-                                        AMN ? titan::ptx::smem_desc_mn_sw128(a0 + 2048 * k, kBox)
-                                            : titan::ptx::smem_desc_sw128(a0 + 32 * k),
-                                        BMN ? titan::ptx::smem_desc_mn_sw128(b0 + 2048 * k, kBox)
-                                            : titan::ptx::smem_desc_sw128(b0 + 32 * k),
-                                        idesc<BN_, AMN, BMN>(), (kb | k) != 0);
-            titan::ptx::tc_commit(&empty[s]);
+                for (int k = 0; k < BK / 16; ++k)
+                    titan::ptx::tc_mma_bf16(taddr, a + kStepA * k, b + kStepB * k, idesc<BN_, AMN, BMN>(), (kb | k) != 0);
+                titan::ptx::tc_commit(&empty[s]);
+            }
+            __syncwarp();
+            a += s1 ? (int64_t)kStep : (int64_t)kStep - STAGES * (int64_t)kStep;
+            b += s1 ? (int64_t)kStep : (int64_t)kStep - STAGES * (int64_t)kStep;
+            s = s1;
+            parity = parity1;
         }
-        titan::ptx::tc_commit(&accf);                  // fires when every issued MMA is done
+        if (leader) titan::ptx::tc_commit(&accf);      // fires when every issued MMA is done
     }
     __syncwarp();
     // epilogue: every thread owns one output row (its TMEM lane); what its first
@@ -242,15 +265,20 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
         }
     };
     request(n0 + group * (BN_ / 4));
-    const bool acc_ok = titan::ptx::mbar_wait_bounded(&accf, 0, spin_limit);
-    titan::ptx::tc_fence_after();
+    // one warp polls; the others sleep at the barrier
+    bool acc_ok = true;
+    if (warp == 1) {
+        acc_ok = titan::ptx::mbar_wait_bounded(&accf, 0, spin_limit);
+        if (!acc_ok) atomicExch(&failed, 1);
+    }
     __syncthreads();
-    if (!acc_ok || failed) {
+    titan::ptx::tc_fence_after();
+    if (failed) {
         // a bounded wait expired: record it, then wait (bounded again) for
         // this CTA's own copies and products still in flight - the last TMA
         // load issued on each stage and every committed MMA - before the
         // tensor memory is freed and the CTA exits
-        if (tid == 0) {
+        if (tid == 32) {
             // a plain store: the flag may live in pinned host memory
             *reinterpret_cast<volatile int *>(err) = 1;
             __threadfence_system();
@@ -362,8 +390,8 @@ k_wgrad(const __grid_constant__ WgradArgs w, int hid, uint32_t spin_limit, int *
 // one-CTA 128 x 256 tile costs 48, which bounded that kernel by shared-memory
 // bandwidth).  A pair keeps taking tiles; two accumulators of 256 TMEM columns
 // let a tile's epilogue run beside the next tile's products.
-//   warp 0 lane 0          - TMA producer of this CTA's halves (6-stage ring)
-//   warp 1 lane 0, leader  - MMA issuer for the pair
+//   warp 0                 - TMA producer of this CTA's halves (6-stage ring)
+//   warp 1, leading CTA    - MMA issuer for the pair
 //   warps 4 .. 7           - epilogue: TMEM lanes 32 (w - 4) .. + 31 of this CTA's 128 rows
 // Barriers: full[s] lives in the leader (both CTAs' bytes), empty[s] and
 // acc_full[b] in each CTA (multicast commits), acc_empty[b] in the leader (one
@@ -382,7 +410,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
     __shared__ uint64_t full[kPairStages], empty[kPairStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
-    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // known to be the same in every lane
     const uint32_t rank = px::cluster_ctarank();
     const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1), tiles = tiles_m * tiles_n;
     const uint32_t raw = px::smem_u32(gsm_raw);
@@ -417,35 +446,48 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
     px::tc_fence_after();
     const uint32_t taddr = tmem_base;
 
-    if (warp == 0 && lane == 0) {                          // TMA producer
-        int it = 0, issued = 0;
+    if (warp == 0) {                                       // TMA producer (one lane issues, as in gemm_tile)
+        const bool leader = px::elect_one();
+        const uint32_t bar0 = px::cluster_smem(&full[0], 0);
+        int it = 0;
+        uint32_t s = 0, parity = 1;
         bool ok = true;
         for (int t = pair; t < tiles && ok; t += pairs) {
             int m0, n0;
             tile_at(t, m0, n0);
             for (int kb = 0; kb < num_kb; ++kb, ++it) {
-                const int s = it % kPairStages;
-                if (it >= kPairStages && !px::mbar_wait_bounded(&empty[s], ((it / kPairStages) & 1) ^ 1, spin_limit)) {
+                if (it >= kPairStages && !px::mbar_wait_bounded(&empty[s], parity, spin_limit)) {
                     ok = false;
                     break;
                 }
-                if (rank == 0) px::mbar_arrive_expect_tx(&full[s], 4 * kPairHalf);
-                const uint32_t bar = px::cluster_smem(&full[s], 0);
-                px::tma_load_2d_pair(tileA(s), &tma_a, kb * BK, m0 + 128 * (int)rank, bar);
-                px::tma_load_2d_pair(tileB(s), &tma_b, kb * BK, n0 + 128 * (int)rank, bar);
-                issued = it + 1;
+                if (leader) {
+                    if (rank == 0) px::mbar_arrive_expect_tx(&full[s], 4 * kPairHalf);
+                    const uint32_t bar = bar0 + 8 * s;
+                    px::tma_load_2d_pair(tileA(s), &tma_a, kb * BK, m0 + 128 * (int)rank, bar);
+                    px::tma_load_2d_pair(tileB(s), &tma_b, kb * BK, n0 + 128 * (int)rank, bar);
+                }
+                __syncwarp();
+                if (++s == kPairStages) {
+                    s = 0;
+                    parity ^= 1;
+                }
             }
         }
-        if (!ok) atomicExch(&failed, 1);
+        if (!ok && leader) atomicExch(&failed, 1);
         // the leader sees the last copies of both CTAs land before the pair may leave
         if (rank == 0)
-            for (int j = max(0, issued - kPairStages); j < issued; ++j)
-                if (!px::mbar_wait_bounded(&full[j % kPairStages], (j / kPairStages) & 1, spin_limit)) atomicExch(&failed, 1);
-    } else if (warp == 1 && lane == 0 && rank == 0) {      // MMA issuer
+            for (int j = max(0, it - kPairStages); j < it; ++j)
+                if (!px::mbar_wait_bounded(&full[j % kPairStages], (j / kPairStages) & 1, spin_limit) && leader)
+                    atomicExch(&failed, 1);
+    } else if (warp == 1 && rank == 0) {                   // MMA issuer
         constexpr uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kPairTile >> 3) << 17) |
                                     ((uint32_t)(kPairTile >> 4) << 24);
-        int it = 0, i = 0;
-        bool ok = true;
+        const bool leader = px::elect_one();
+        uint64_t da = px::smem_desc_sw128(px::smem_u32(tileA(0))), db = px::smem_desc_sw128(px::smem_u32(tileB(0)));
+        constexpr int64_t kStep = 2 * kPairHalf >> 4;
+        uint32_t s = 0, parity = 0;
+        int i = 0;
+        bool ok = true, ready = false;                     // ready: the next k-block was seen to have arrived
         for (int t = pair; t < tiles && ok; t += pairs, ++i) {
             const int b = i & 1;
             if (i >= 2 && !px::mbar_wait_bounded(&acc_empty[b], ((i >> 1) & 1) ^ 1, spin_limit)) {
@@ -453,23 +495,29 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
                 break;
             }
             px::tc_fence_after();
-            for (int kb = 0; kb < num_kb; ++kb, ++it) {
-                const int s = it % kPairStages;
-                if (!px::mbar_wait_bounded(&full[s], (it / kPairStages) & 1, spin_limit)) {
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!ready && !px::mbar_wait_bounded(&full[s], parity, spin_limit)) {
                     ok = false;
                     break;
                 }
                 px::tc_fence_after();
-                const uint32_t a0 = px::smem_u32(tileA(s)), b0 = px::smem_u32(tileB(s));
+                const uint32_t s1 = s + 1 == kPairStages ? 0 : s + 1, parity1 = parity ^ (s1 == 0);
+                ready = (kb + 1 < num_kb || t + pairs < tiles) && px::mbar_test(&full[s1], parity1);
+                if (leader) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    px::tc_mma_bf16_pair(taddr + (uint32_t)(b * kPairTile), px::smem_desc_sw128(a0 + 32 * k),
-                                         px::smem_desc_sw128(b0 + 32 * k), idesc2, (kb | k) != 0);
-                px::tc_commit_pair(&empty[s]);
+                    for (int k = 0; k < BK / 16; ++k)
+                        px::tc_mma_bf16_pair(taddr + (uint32_t)(b * kPairTile), da + 2 * k, db + 2 * k, idesc2, (kb | k) != 0);
+                    px::tc_commit_pair(&empty[s]);
+                }
+                __syncwarp();
+                da += s1 ? kStep : kStep - kPairStages * kStep;
+                db += s1 ? kStep : kStep - kPairStages * kStep;
+                s = s1;
+                parity = parity1;
             }
-            px::tc_commit_pair(&acc_full[b]);
+            if (leader) px::tc_commit_pair(&acc_full[b]);
         }
-        if (!ok) atomicExch(&failed, 1);
+        if (!ok && leader) atomicExch(&failed, 1);
     } else if (warp >= 4) {                                // epilogue
         const uint32_t q = warp & 3;
         int i = 0;
