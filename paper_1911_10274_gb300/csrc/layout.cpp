@@ -106,6 +106,21 @@ void component_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<u
     for (uint32_t d = 0; d < n; ++d) caller_of_dev[size[number[find(in[d])]]++] = in[d];
 }
 
+void degree_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<uint32_t> &caller_of_dev,
+                  std::vector<uint32_t> &rank) {
+    std::vector<uint32_t> deg(n, 0);
+    for (size_t e = 0; e < 2 * (size_t)s; ++e) ++deg[ends[e]];
+    rank.resize(n);
+    std::iota(rank.begin(), rank.end(), 0u);
+    for (uint32_t b = 0; b < n; b += kHaloBlock)
+        std::stable_sort(rank.begin() + b, rank.begin() + std::min(n, b + kHaloBlock), [&](uint32_t x, uint32_t y) {
+            return deg[caller_of_dev[x]] > deg[caller_of_dev[y]];
+        });
+    std::vector<uint32_t> in(std::move(caller_of_dev));
+    caller_of_dev.resize(n);
+    for (uint32_t d = 0; d < n; ++d) caller_of_dev[d] = in[rank[d]];
+}
+
 bool grid_tile_order(const double *pos, uint32_t n, double h, std::vector<uint32_t> &caller_of_dev,
                      std::vector<int32_t> *cell_of_dev) {
     caller_of_dev.clear();
@@ -182,7 +197,7 @@ uint32_t direction_class(const double *a, const double *b) {
 }  // namespace
 
 bool build_sell(uint32_t n, uint32_t s, const uint32_t *ends, const double *pos,
-                const std::vector<uint32_t> &dev_of, SellHost &out, const int32_t *cell) {
+                const std::vector<uint32_t> &dev_of, SellHost &out, const int32_t *cell, const uint32_t *rank) {
     const uint32_t n_slices = (n + 31) / 32;
     std::vector<uint32_t> deg(n, 0);
     for (uint32_t q = 0; q < s; ++q) {
@@ -232,9 +247,10 @@ bool build_sell(uint32_t n, uint32_t s, const uint32_t *ends, const double *pos,
     }
     for (uint32_t i = 0; i < n; ++i)
         std::sort(he.begin() + rowptr[i], he.begin() + rowptr[i + 1],
-                  [](const HalfEdge &x, const HalfEdge &y) {
+                  [rank](const HalfEdge &x, const HalfEdge &y) {
                       if (x.key != y.key) return x.key < y.key;
-                      return x.nbr != y.nbr ? x.nbr < y.nbr : x.spring < y.spring;
+                      if (x.nbr == y.nbr) return x.spring < y.spring;
+                      return rank ? rank[x.nbr] < rank[y.nbr] : x.nbr < y.nbr;
                   });
     // Column of every half-edge within its slice.  Default: its position in
     // the row.  On a grid: one run of columns per distinct key of the slice

@@ -733,6 +733,7 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
     // ---- host-side layout
     const uint32_t n = m->n, s = sp->n;
     std::vector<int32_t> cells;           // grid cell per device index (grid-tile order only)
+    std::vector<uint32_t> rank;           // Morton position per device index (Morton order only)
     if (p->order == TITAN_ORDER_MORTON) {
         // masses on a grid (pitch = shortest spring) get the grid-tile order, others Morton
         double h = INFINITY;
@@ -751,6 +752,7 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
             cells.clear();
             titan::morton_order(m->pos, n, sim->caller_of_dev);
             titan::component_order(n, s, sp->ends, sim->caller_of_dev);
+            titan::degree_order(n, s, sp->ends, sim->caller_of_dev, rank);
         }
     } else {
         sim->caller_of_dev.resize(n);
@@ -830,7 +832,7 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
 
     if (sim->accumulate == TITAN_ACCUM_CSR) {
         if (!titan::build_sell(nd, s, sp->ends, m->pos, sim->dev_of_caller, sim->sell,
-                               sim->grid_order ? cells.data() : nullptr))
+                               sim->grid_order ? cells.data() : nullptr, rank.empty() ? nullptr : rank.data()))
             return bail(fail(sim, TITAN_E_UNSUPPORTED, "padded incidence exceeds 2^32 entries"));
         const int want = p->kernel_variant;
         sim->csr_kernel = want == 0 ? (sim->grid_order ? 6 : 4) : want;
