@@ -242,8 +242,10 @@ k_batch_rollout(const BatchCta *__restrict__ ctas, const MassState *__restrict__
 // that read it (the lists of build_batch), so one cluster barrier ends a step
 // and no halo is fetched at its start.  Rows are summed in the same order as in
 // k_batch_rollout with one thread per mass: the same bits.
-// Measured, 64 voxel robots x 1000 steps 3.47 -> 2.03 ms, 1,024 robots of 27 to
-// 1,728 masses x 200 steps 6.16 -> 5.16 ms (both with reset and centroids).
+// Measured, 64 voxel robots x 1000 steps 3.47 -> 1.99 ms, 1,024 robots of 27 to
+// 1,728 masses x 200 steps 6.16 -> 4.98 ms (both with reset and centroids).  Entries
+// side by side, 4, 7, 8, 9, 10 and 13: robots 5.16, 4.93, 4.98, 4.84, 4.87 and 4.85 ms,
+// voxel robots 2.02, 2.11, 1.99, 2.07, 2.12 and 2.12.
 template <bool ACT, bool GROUND>
 __global__ void __launch_bounds__(titan::kRowSlots)
 k_batch_rows(const BatchCta *__restrict__ ctas, const MassState *__restrict__ state_in,
@@ -252,7 +254,7 @@ k_batch_rows(const BatchCta *__restrict__ ctas, const MassState *__restrict__ st
              const uint32_t *__restrict__ halo, const uint2 *__restrict__ push,
              const uint32_t *__restrict__ push_more, titan::StepConst c, long long step0, uint32_t n_steps,
              uint32_t cluster_size) {
-    constexpr int W = (int)titan::kRowWidth, G = 4;         // entries per row, evaluated side by side
+    constexpr int W = (int)titan::kRowWidth, G = 8;         // entries per row, evaluated side by side
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ float2 s_sc[2];                              // as in k_batch_rollout
     const BatchCta d = ctas[blockIdx.x];
