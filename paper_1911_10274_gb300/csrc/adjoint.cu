@@ -218,13 +218,19 @@ __global__ void k_adj_force0(const MassState *__restrict__ X, const float4 *__re
 // kAdjTrajectory between calls (the default pool gives every byte back at each
 // synchronisation, and mapping them again took as long as dozens of steps).
 // adjoint_trim gives the memory back (titan_destroy).
+// Kept while the device's context lives (a cudaDeviceReset destroys it).
+struct Pool {
+    unsigned long long ctx_id = 0;
+    cudaMemPool_t pool = nullptr;
+};
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[64] = {};
+Pool g_pool[64];
 
 cudaError_t adjoint_pool(int dev, cudaMemPool_t *out) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (!g_pool[dev]) {
+    const unsigned long long id = titan::current_context_id();
+    if (!g_pool[dev].pool || g_pool[dev].ctx_id != id) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -238,9 +244,9 @@ cudaError_t adjoint_pool(int dev, cudaMemPool_t *out) {
             cudaMemPoolDestroy(p);
             return e;
         }
-        g_pool[dev] = p;
+        g_pool[dev] = {id, p};
     }
-    *out = g_pool[dev];
+    *out = g_pool[dev].pool;
     return cudaSuccess;
 }
 
@@ -263,7 +269,8 @@ titan_status afail(titan_sim *sim, titan_status st, const std::string &msg) {
 
 void titan::adjoint_trim(int dev) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (dev >= 0 && dev < 64 && g_pool[dev]) cudaMemPoolTrimTo(g_pool[dev], 0);
+    if (dev >= 0 && dev < 64 && g_pool[dev].pool && g_pool[dev].ctx_id == titan::current_context_id())
+        cudaMemPoolTrimTo(g_pool[dev].pool, 0);
 }
 
 extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t every,

@@ -397,7 +397,8 @@ k_wgrad(const __grid_constant__ WgradArgs w, int hid, uint32_t spin_limit, int *
 // acc_full[b] in each CTA (multicast commits), acc_empty[b] in the leader (one
 // arrival per epilogue warp of both CTAs).  Every wait is bounded; after one
 // expires a CTA records it, stops, and meets the pair's last barrier.
-// 8192^3: 818 -> 704 us (1,344 -> 1,562 TFLOP/s), the same bits.
+// 8192^3: 818 us with one-CTA tiles, 704 (1,562 TFLOP/s) with pairs issued by one lane,
+// 587 (1,874) issued from whole warps (see gemm_tile); the same bits.
 constexpr int kPairStages = 6, kPairTile = 256, kPairThreads = 256;
 constexpr uint32_t kPairHalf = 128 * BK * 2;             // bytes of one CTA's half of A or B per stage
 constexpr size_t kPairSmem = (size_t)kPairStages * 2 * kPairHalf + 1024;

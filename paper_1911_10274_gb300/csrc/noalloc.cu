@@ -42,6 +42,37 @@ namespace titan {
 void set_thread_error(const std::string &msg);   // defined in runtime.cu
 }
 
+// The driver's context queries, reached through the runtime (no link against
+// libcuda): the id of the context current on this thread, 0 if none.
+namespace {
+using CtxGetCurrentFn = CUresult (*)(CUcontext *);
+using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long *);
+CtxGetCurrentFn g_ctx_get_current = nullptr;
+CtxGetIdFn g_ctx_get_id = nullptr;
+std::once_flag g_ctx_fns_once;
+
+}  // namespace
+
+unsigned long long titan::current_context_id() {
+    std::call_once(g_ctx_fns_once, [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            g_ctx_get_current = reinterpret_cast<CtxGetCurrentFn>(f);
+        f = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            g_ctx_get_id = reinterpret_cast<CtxGetIdFn>(f);
+    });
+    if (!g_ctx_get_current || !g_ctx_get_id) return 0;
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    if (g_ctx_get_current(&ctx) != CUDA_SUCCESS || !ctx) return 0;
+    if (g_ctx_get_id(ctx, &id) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
 namespace {
 
 using titan::MassState;
@@ -81,41 +112,13 @@ HostPage g_bad_host[kMappedDevices];
 std::mutex g_addr_mu;
 ScratchAddr g_addr[64];
 
-// The driver's context queries, reached through the runtime (no link against
-// libcuda): the id of the context current on this thread, 0 if none.
-using CtxGetCurrentFn = CUresult (*)(CUcontext *);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long *);
-CtxGetCurrentFn g_ctx_get_current = nullptr;
-CtxGetIdFn g_ctx_get_id = nullptr;
-std::once_flag g_ctx_fns_once;
-
-unsigned long long current_context_id() {
-    std::call_once(g_ctx_fns_once, [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_ctx_get_current = reinterpret_cast<CtxGetCurrentFn>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_ctx_get_id = reinterpret_cast<CtxGetIdFn>(f);
-    });
-    if (!g_ctx_get_current || !g_ctx_get_id) return 0;
-    CUcontext ctx = nullptr;
-    unsigned long long id = 0;
-    if (g_ctx_get_current(&ctx) != CUDA_SUCCESS || !ctx) return 0;
-    if (g_ctx_get_id(ctx, &id) != CUDA_SUCCESS) return 0;
-    return id;
-}
-
 cudaError_t scratch_address(ScratchAddr *out, int *dev_out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_addr_mu);
-    const unsigned long long id = current_context_id();
+    const unsigned long long id = titan::current_context_id();
     *dev_out = dev;
     if (id != 0 && g_addr[dev].ctx_id == id && g_addr[dev].ptr) {
         *out = g_addr[dev];
@@ -125,7 +128,7 @@ cudaError_t scratch_address(ScratchAddr *out, int *dev_out) {
     e = cudaGetSymbolAddress(&p, g_noalloc_force);     // also makes the primary context current
     if (e != cudaSuccess) return e;
     g_addr[dev].ptr = static_cast<float4 *>(p);
-    g_addr[dev].ctx_id = current_context_id();          // 0 (no id): looked up again next call
+    g_addr[dev].ctx_id = titan::current_context_id();          // 0 (no id): looked up again next call
     g_addr[dev].bad_dev = nullptr;
     if (dev < kMappedDevices) {
         void *h = const_cast<unsigned int *>(&g_bad_host[dev].bad), *d = nullptr;

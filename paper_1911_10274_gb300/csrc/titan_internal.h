@@ -206,4 +206,7 @@ cudaError_t launch_patch_words(uint32_t *base, const uint32_t *idx, const uint32
 cudaError_t launch_unpermute(const MassState *state, const uint32_t *dev_of_caller, uint32_t n,
                              float *pos, float *vel, cudaStream_t stream);
 
+// The id of the context current on this thread, 0 if the driver gives none (noalloc.cu).
+unsigned long long current_context_id();
+
 }  // namespace titan
