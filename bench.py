@@ -435,7 +435,7 @@ def mlp_leg(device, batch=4096, n_in=1024, hidden=512, reps=20, big=True):
         torch.cuda.synchronize()
         t0 = time.perf_counter()
         for _ in range(n):
-            net.train_step(x, t, 1e-3)          # enqueued back to back (one captured graph each)
+            net.train_step(x, t, 1e-3)          # enqueued back to back
         net.sync()
         return (time.perf_counter() - t0) / n
 
