@@ -111,9 +111,9 @@ __device__ __forceinline__ float adj_half_edge(const float4 &p, const float4 &v,
 // the force adjoint of the step before (Fout; the neighbours' is read from Fin).
 // (xb, vb) are this mass's alone and updated in place.
 //
-// Bound by the gathers (48 bytes an entry, 45 % of them from L1: the masses of
-// 2,500 threads and their neighbours just fill it) and the row stream (20 bytes
-// an entry from L2).  Two entries are reversed per iteration, with the next
+// Bound by the latency of the row stream (20 bytes an entry from L2) and of the
+// gathers (48 bytes an entry; L1 serves 60 % of all sectors, the masses of 2,500
+// threads and their neighbours just filling it).  Two entries are reversed per iteration, with the next
 // two's constants already requested; 128-thread blocks, six per SM.  The row
 // stream through an asynchronous ring in shared memory measured 9 % slower (it
 // takes L1 from the gathers), adding to the sums by load and store 6 %.  The sine
