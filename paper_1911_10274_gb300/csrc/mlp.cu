@@ -182,7 +182,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
         uint32_t s = 0, parity = 1;
         int issued = 0;
         for (int kb = 0, k = k0; kb < num_kb; ++kb, k += BK) {
-            if (kb >= STAGES && !titan::ptx::mbar_wait_bounded(&empty[s], parity, spin_limit)) {
+            if (kb >= STAGES && !titan::ptx::mbar_wait_warp(&empty[s], parity, spin_limit)) {
                 if (leader) atomicExch(&failed, 1);
                 break;
             }
@@ -222,13 +222,13 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
         uint32_t s = 0, parity = 0;
         bool ready = false;                            // this k-block was seen to have arrived
         for (int kb = 0; kb < num_kb; ++kb) {
-            if (!ready && !titan::ptx::mbar_wait_bounded(&full[s], parity, spin_limit)) {
+            if (!ready && !titan::ptx::mbar_wait_warp(&full[s], parity, spin_limit)) {
                 if (leader) atomicExch(&failed, 1);
                 break;
             }
             titan::ptx::tc_fence_after();
             const uint32_t s1 = s + 1 == STAGES ? 0 : s + 1, parity1 = parity ^ (s1 == 0);
-            ready = kb + 1 < num_kb && titan::ptx::mbar_test(&full[s1], parity1);
+            ready = kb + 1 < num_kb && __all_sync(0xffffffffu, titan::ptx::mbar_test(&full[s1], parity1));
             if (leader) {
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
@@ -398,7 +398,7 @@ k_wgrad(const __grid_constant__ WgradArgs w, int hid, uint32_t spin_limit, int *
 // arrival per epilogue warp of both CTAs).  Every wait is bounded; after one
 // expires a CTA records it, stops, and meets the pair's last barrier.
 // 8192^3: 818 us with one-CTA tiles, 704 (1,562 TFLOP/s) with pairs issued by one lane,
-// 587 (1,874) issued from whole warps (see gemm_tile); the same bits.
+// 587 to 605 (1,818 to 1,874) issued from whole warps (see gemm_tile); the same bits.
 constexpr int kPairStages = 6, kPairTile = 256, kPairThreads = 256;
 constexpr uint32_t kPairHalf = 128 * BK * 2;             // bytes of one CTA's half of A or B per stage
 constexpr size_t kPairSmem = (size_t)kPairStages * 2 * kPairHalf + 1024;
@@ -457,7 +457,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             int m0, n0;
             tile_at(t, m0, n0);
             for (int kb = 0; kb < num_kb; ++kb, ++it) {
-                if (it >= kPairStages && !px::mbar_wait_bounded(&empty[s], parity, spin_limit)) {
+                if (it >= kPairStages && !px::mbar_wait_warp(&empty[s], parity, spin_limit)) {
                     ok = false;
                     break;
                 }
@@ -478,7 +478,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
         // the leader sees the last copies of both CTAs land before the pair may leave
         if (rank == 0)
             for (int j = max(0, it - kPairStages); j < it; ++j)
-                if (!px::mbar_wait_bounded(&full[j % kPairStages], (j / kPairStages) & 1, spin_limit) && leader)
+                if (!px::mbar_wait_warp(&full[j % kPairStages], (j / kPairStages) & 1, spin_limit) && leader)
                     atomicExch(&failed, 1);
     } else if (warp == 1 && rank == 0) {                   // MMA issuer
         constexpr uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kPairTile >> 3) << 17) |
@@ -491,19 +491,19 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
         bool ok = true, ready = false;                     // ready: the next k-block was seen to have arrived
         for (int t = pair; t < tiles && ok; t += pairs, ++i) {
             const int b = i & 1;
-            if (i >= 2 && !px::mbar_wait_bounded(&acc_empty[b], ((i >> 1) & 1) ^ 1, spin_limit)) {
+            if (i >= 2 && !px::mbar_wait_warp(&acc_empty[b], ((i >> 1) & 1) ^ 1, spin_limit)) {
                 ok = false;
                 break;
             }
             px::tc_fence_after();
             for (int kb = 0; kb < num_kb; ++kb) {
-                if (!ready && !px::mbar_wait_bounded(&full[s], parity, spin_limit)) {
+                if (!ready && !px::mbar_wait_warp(&full[s], parity, spin_limit)) {
                     ok = false;
                     break;
                 }
                 px::tc_fence_after();
                 const uint32_t s1 = s + 1 == kPairStages ? 0 : s + 1, parity1 = parity ^ (s1 == 0);
-                ready = (kb + 1 < num_kb || t + pairs < tiles) && px::mbar_test(&full[s1], parity1);
+                ready = (kb + 1 < num_kb || t + pairs < tiles) && __all_sync(0xffffffffu, px::mbar_test(&full[s1], parity1));
                 if (leader) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
@@ -526,7 +526,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             const int b = i & 1;
             int m0, n0;
             tile_at(t, m0, n0);
-            if (!px::mbar_wait_bounded(&acc_full[b], (i >> 1) & 1, spin_limit)) {
+            if (!px::mbar_wait_warp(&acc_full[b], (i >> 1) & 1, spin_limit)) {
                 atomicExch(&failed, 1);
                 break;
             }

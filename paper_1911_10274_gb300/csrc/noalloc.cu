@@ -235,6 +235,7 @@ k_na_small(const float *pos, const float *vel, const float *__restrict__ inv_mas
         }
     };
     if (t < n_springs) fetch(t);
+    __syncwarp();
     titan::ptx::cluster_sync();                         // the accumulator is clear
     for (uint32_t s = t; s < n_springs; s += T) {
         if (s != t) fetch(s);

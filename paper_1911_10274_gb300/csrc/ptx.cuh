@@ -91,6 +91,14 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
+// The same for a converged warp that goes on as one: true once every lane has seen
+// the phase complete, the same answer in every lane (also when the polls run out).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, uint32_t limit) {
+    for (uint32_t it = 0; it < limit; ++it)
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return false;
+}
+
 // Programmatic dependent launch.  A kernel launched with the
 // programmatic-stream-serialization attribute may start before the kernel
 // ahead of it in the stream has finished: grid_dep_wait() blocks until that
