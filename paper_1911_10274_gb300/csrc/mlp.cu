@@ -21,7 +21,8 @@
 //                    its bias-gradient column sums.
 // Every mbarrier wait is bounded (spin_limit polls); on expiry the kernel sets
 // *err, waits (bounded) for its own copies and products in flight, skips the
-// epilogue, frees its TMEM and returns.
+// epilogue, frees its TMEM and returns.  No CTA leaves, after an expired wait or
+// not, before every copy and every commit that targets it has landed (gemm_ring.h).
 //
 // Training step: nine launches on one stream, each a programmatic dependent of
 // the one before: a copy of the batch, three forward products, the head (output
@@ -40,6 +41,7 @@
 #include <string>
 #include <vector>
 
+#include "gemm_ring.h"
 #include "ptx.cuh"
 #include "titan.h"
 
@@ -66,6 +68,9 @@ template <int BN_> constexpr uint32_t stage_b() { return (uint32_t)BN_ * BK * 2;
 template <int BN_> constexpr int stages() { return BN_ == 128 ? 3 : 4; }
 template <int BN_> constexpr int resident() { return BN_ == 256 ? 1 : 2; }
 template <int BN_> constexpr size_t gemm_smem() { return (size_t)stages<BN_>() * (kStageA + stage_b<BN_>()) + 1024; }
+
+// Polls of a wait for what is already under way and completes by itself.
+constexpr uint32_t kDrainPolls = 1u << 22;
 
 enum Epi { EPI_F32 = 0, EPI_BIAS_GELU = 1, EPI_GELU_GRAD = 2 };
 
@@ -139,7 +144,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
     __shared__ uint64_t full[STAGES], empty[STAGES], accf;
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
-    __shared__ int n_issued;                          // k blocks whose TMA loads were issued
+    __shared__ int n_issued, n_mma;                   // k-blocks whose loads, whose products were issued
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // known to be the same in every lane
     titan::ptx::grid_dep_launch();                    // the next kernel's prologue may overlap this one
@@ -161,7 +166,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
         titan::ptx::mbar_init(&accf, 1);
         titan::ptx::fence_mbar_init();
         failed = 0;
-        n_issued = 0;
+        n_issued = n_mma = 0;
     }
     titan::ptx::tc_fence_before();
     __syncthreads();
@@ -220,8 +225,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
                          : titan::ptx::smem_desc_sw128(titan::ptx::smem_u32(tileB(0)));
         constexpr uint32_t kStep = (kStageA + kStageB) >> 4, kStepA = (AMN ? 2048 : 32) >> 4, kStepB = (BMN ? 2048 : 32) >> 4;
         uint32_t s = 0, parity = 0;
+        int kb = 0;
         bool ready = false;                            // this k-block was seen to have arrived
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (; kb < num_kb; ++kb) {
             if (!ready && !titan::ptx::mbar_wait_warp(&full[s], parity, spin_limit)) {
                 if (leader) atomicExch(&failed, 1);
                 break;
@@ -241,7 +247,10 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
             s = s1;
             parity = parity1;
         }
-        if (leader) titan::ptx::tc_commit(&accf);      // fires when every issued MMA is done
+        if (leader) {
+            titan::ptx::tc_commit(&accf);              // fires when every issued MMA is done
+            n_mma = kb;
+        }
     }
     __syncwarp();
     // epilogue: every thread owns one output row (its TMEM lane); what its first
@@ -282,12 +291,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
             // a plain store: the flag may live in pinned host memory
             *reinterpret_cast<volatile int *>(err) = 1;
             __threadfence_system();
-            for (int st = 0; st < STAGES; ++st) {
-                int last = -1;
-                for (int kb = st; kb < n_issued; kb += STAGES) last = kb;
-                if (last >= 0) titan::ptx::mbar_wait_bounded(&full[st], (uint32_t)(last / STAGES) & 1u, spin_limit);
-            }
-            if (!acc_ok) titan::ptx::mbar_wait_bounded(&accf, 0, spin_limit);
+            for (int j = titan::ring_tail(n_issued, STAGES); j < n_issued; ++j)
+                titan::ptx::mbar_wait_bounded(&full[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES), kDrainPolls);
+            if (!acc_ok) titan::ptx::mbar_wait_bounded(&accf, 0, kDrainPolls);
         }
         __syncthreads();
     } else {
@@ -349,7 +355,12 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
     }
     titan::ptx::tc_fence_before();
     __syncthreads();
-    if (warp == 0) titan::ptx::tmem_dealloc(taddr, kTmemCols);
+    if (warp == 0) {
+        // the last releases of the ring, which no producer waited for
+        for (int j = titan::ring_tail(n_mma, STAGES); j < n_mma; ++j)
+            titan::ptx::mbar_wait_warp(&empty[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES), kDrainPolls);
+        titan::ptx::tmem_dealloc(taddr, kTmemCols);
+    }
 }
 
 // split K (gridDim.z slices): slice z multiplies k-columns [z K, (z + 1) K) of A
@@ -396,7 +407,9 @@ k_wgrad(const __grid_constant__ WgradArgs w, int hid, uint32_t spin_limit, int *
 // Barriers: full[s] lives in the leader (both CTAs' bytes), empty[s] and
 // acc_full[b] in each CTA (multicast commits), acc_empty[b] in the leader (one
 // arrival per epilogue warp of both CTAs).  Every wait is bounded; after one
-// expires a CTA records it, stops, and meets the pair's last barrier.
+// expires a CTA records it and stops.  Then the CTAs tell each other how far they
+// came and wait, bounded, for whatever of that is still to land (the commits in both
+// CTAs; after a failure also the copies, whose barriers the leader settles).
 // 8192^3: 818 us with one-CTA tiles, 704 (1,562 TFLOP/s) with pairs issued by one lane,
 // 587 to 605 (1,818 to 1,874) issued from whole warps (see gemm_tile); the same bits.
 constexpr int kPairStages = 6, kPairTile = 256, kPairThreads = 256;
@@ -408,9 +421,12 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             int tiles_n, int ldc, float *__restrict__ C, uint32_t spin_limit, int *__restrict__ err) {
     namespace px = titan::ptx;
     extern __shared__ uint8_t gsm_raw[];
-    __shared__ uint64_t full[kPairStages], empty[kPairStages], acc_full[2], acc_empty[2];
+    __shared__ uint64_t full[kPairStages], empty[kPairStages], acc_full[2], acc_empty[2], done;
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
+    // k-blocks whose copies this CTA issued; in the leader, k-blocks and tiles whose products were
+    // issued; the same, and `failed`, of the other CTA (written by it at the end)
+    __shared__ int n_issued, n_mma, n_acc, peer[4];
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // known to be the same in every lane
     const uint32_t rank = px::cluster_ctarank();
@@ -438,8 +454,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             px::mbar_init(&acc_full[b], 1);
             px::mbar_init(&acc_empty[b], 8);
         }
+        px::mbar_init(&done, 1);
         px::fence_mbar_init();
-        failed = 0;
+        failed = n_issued = n_mma = n_acc = 0;
     }
     px::tc_fence_before();
     __syncthreads();
@@ -475,11 +492,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             }
         }
         if (!ok && leader) atomicExch(&failed, 1);
-        // the leader sees the last copies of both CTAs land before the pair may leave
-        if (rank == 0)
-            for (int j = max(0, it - kPairStages); j < it; ++j)
-                if (!px::mbar_wait_warp(&full[j % kPairStages], (j / kPairStages) & 1, spin_limit) && leader)
-                    atomicExch(&failed, 1);
+        if (leader) n_issued = it;
     } else if (warp == 1 && rank == 0) {                   // MMA issuer
         constexpr uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kPairTile >> 3) << 17) |
                                     ((uint32_t)(kPairTile >> 4) << 24);
@@ -487,7 +500,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
         uint64_t da = px::smem_desc_sw128(px::smem_u32(tileA(0))), db = px::smem_desc_sw128(px::smem_u32(tileB(0)));
         constexpr int64_t kStep = 2 * kPairHalf >> 4;
         uint32_t s = 0, parity = 0;
-        int i = 0;
+        int i = 0, mma = 0;
         bool ok = true, ready = false;                     // ready: the next k-block was seen to have arrived
         for (int t = pair; t < tiles && ok; t += pairs, ++i) {
             const int b = i & 1;
@@ -496,7 +509,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
                 break;
             }
             px::tc_fence_after();
-            for (int kb = 0; kb < num_kb; ++kb) {
+            for (int kb = 0; kb < num_kb; ++kb, ++mma) {
                 if (!ready && !px::mbar_wait_warp(&full[s], parity, spin_limit)) {
                     ok = false;
                     break;
@@ -518,7 +531,12 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
             }
             if (leader) px::tc_commit_pair(&acc_full[b]);
         }
-        if (!ok && leader) atomicExch(&failed, 1);
+        if (leader) {
+            px::tc_commit_pair(&done);                     // fires when every issued MMA is done
+            n_mma = mma;
+            n_acc = i;
+            if (!ok) atomicExch(&failed, 1);
+        }
     } else if (warp >= 4) {                                // epilogue
         const uint32_t q = warp & 3;
         int i = 0;
@@ -556,7 +574,32 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ C
         *reinterpret_cast<volatile int *>(err) = 1;        // may live in pinned host memory
         __threadfence_system();
     }
-    px::cluster_sync();                                    // nothing of the pair's is in flight
+    if (tid < 4)
+        px::st_cluster(px::cluster_smem(&peer[tid], rank ^ 1), tid == 0 ? failed : tid == 1 ? n_issued : tid == 2 ? n_mma : n_acc);
+    px::cluster_sync();                                    // neither CTA issues anything any more
+    const bool bad = failed || peer[0];
+    if (warp == 0) {
+        const int mma = rank ? peer[2] : n_mma, acc = rank ? peer[3] : n_acc;
+        px::mbar_wait_warp(&done, 0, kDrainPolls);
+        // the last releases of the ring, which no producer waited for
+        for (int j = titan::ring_tail(mma, kPairStages); j < mma; ++j)
+            px::mbar_wait_warp(&empty[titan::ring_slot(j, kPairStages)], titan::ring_parity(j, kPairStages), kDrainPolls);
+        if (bad) {                                         // and what an epilogue or the issuer did not
+            for (int j = titan::ring_tail(acc, 2); j < acc; ++j)
+                px::mbar_wait_warp(&acc_full[titan::ring_slot(j, 2)], titan::ring_parity(j, 2), kDrainPolls);
+            if (rank == 0)
+                for (int j = mma; j < max(n_issued, peer[1]); ++j) {
+                    uint64_t *bar = &full[titan::ring_slot(j, kPairStages)];
+                    const titan::PairSettle fix = titan::pair_settle(j, n_issued, peer[1], 2 * kPairHalf);
+                    if (lane == 0 && fix.expect) px::mbar_arrive_expect_tx(bar, fix.expect);
+                    if (lane == 0 && fix.cancel) px::mbar_complete_tx(bar, fix.cancel);
+                    __syncwarp();
+                    px::mbar_wait_warp(bar, titan::ring_parity(j, kPairStages), kDrainPolls);
+                }
+        }
+    }
+    __syncwarp();
+    if (bad) px::cluster_sync();                           // the other CTA's copies report to the leader
     px::tc_fence_after();
     if (warp == 0) px::tmem_dealloc_pair(taddr, 512);
 }
