@@ -274,9 +274,18 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
         }
     };
     request(n0 + group * (BN_ / 4));
-    // one warp polls; the others sleep at the barrier
+    // one warp polls; the others sleep at the barrier.  Beside it the producer waits for the
+    // last releases of its ring, which land with the accumulator
     bool acc_ok = true;
-    if (warp == 1) {
+    if (warp == 0) {
+        if (n_issued == num_kb)
+            for (int j = titan::ring_tail(num_kb, STAGES); j < num_kb; ++j)
+                if (!titan::ptx::mbar_wait_warp(&empty[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES),
+                                                spin_limit)) {
+                    atomicExch(&failed, 1);
+                    break;
+                }
+    } else if (warp == 1) {
         acc_ok = titan::ptx::mbar_wait_bounded(&accf, 0, spin_limit);
         if (!acc_ok) atomicExch(&failed, 1);
     }
@@ -294,6 +303,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
             for (int j = titan::ring_tail(n_issued, STAGES); j < n_issued; ++j)
                 titan::ptx::mbar_wait_bounded(&full[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES), kDrainPolls);
             if (!acc_ok) titan::ptx::mbar_wait_bounded(&accf, 0, kDrainPolls);
+            for (int j = titan::ring_tail(n_mma, STAGES); j < n_mma; ++j)
+                titan::ptx::mbar_wait_bounded(&empty[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES), kDrainPolls);
         }
         __syncthreads();
     } else {
@@ -355,12 +366,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tma_a, const CUtens
     }
     titan::ptx::tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
-        // the last releases of the ring, which no producer waited for
-        for (int j = titan::ring_tail(n_mma, STAGES); j < n_mma; ++j)
-            titan::ptx::mbar_wait_warp(&empty[titan::ring_slot(j, STAGES)], titan::ring_parity(j, STAGES), kDrainPolls);
-        titan::ptx::tmem_dealloc(taddr, kTmemCols);
-    }
+    if (warp == 0) titan::ptx::tmem_dealloc(taddr, kTmemCols);
 }
 
 // split K (gridDim.z slices): slice z multiplies k-columns [z K, (z + 1) K) of A
