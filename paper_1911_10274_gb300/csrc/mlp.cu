@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "gemm_ring.h"
+#include "mlp_layout.h"
 #include "ptx.cuh"
 #include "titan.h"
 
@@ -773,13 +774,12 @@ __device__ __forceinline__ float2 loss_sum(const float *diff, uint32_t B, float2
 // partial products of each layer; vectors (b1, b2, b3, w4): sums by column of 32 rows
 // each; loss and b4: the head's y - t.
 struct GradArgs {
+    titan::MlpLayout at;
     const float *part[3];                 // [splits][hid][in_l]
-    uint32_t off[3], n[3];                // parameter offset and count of W_l^T
     uint32_t splits[3], hid;
     const float *vpart[4];
-    uint32_t voff[4];
     const float *diff;
-    uint32_t off_b4, B;
+    uint32_t B;
     float *loss;                          // may be null
 };
 struct AdamArgs {
@@ -816,14 +816,15 @@ __device__ __forceinline__ void for_gradients(const GradArgs &g, S &&state, W &&
         blk -= 4 * per + 1;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            const uint32_t blocks = g.n[l] >> 10;             // n is a multiple of 128 x 128
+            const uint32_t blocks = titan::grad_blocks(g.at.n_w[l]);
             if (blk < blocks) {
-                const uint32_t i = 1024 * blk + 4 * tid, splits = g.splits[l];     // at most 8
+                const size_t i = titan::grad_index(blk, tid);
+                const uint32_t splits = g.splits[l];          // at most 8
                 const auto st = state(l, i);
                 float4 r[8];
 #pragma unroll
                 for (uint32_t z = 0; z < 8; ++z)
-                    if (z < splits) r[z] = __ldcg(reinterpret_cast<const float4 *>(g.part[l] + (size_t)z * g.n[l] + i));
+                    if (z < splits) r[z] = __ldcg(reinterpret_cast<const float4 *>(g.part[l] + z * g.at.n_w[l] + i));
                 float4 q = r[0];
 #pragma unroll
                 for (uint32_t z = 1; z < 8; ++z)              // slices in order
@@ -843,7 +844,7 @@ __device__ __forceinline__ void for_gradients(const GradArgs &g, S &&state, W &&
     if (blk < 4 * per) {
         const uint32_t k = blk / per, c0 = 32 * (blk - k * per);
         const float *part = k == 0 ? g.vpart[0] : k == 1 ? g.vpart[1] : k == 2 ? g.vpart[2] : g.vpart[3];
-        const uint32_t off = k == 0 ? g.voff[0] : k == 1 ? g.voff[1] : k == 2 ? g.voff[2] : g.voff[3];
+        const size_t off = k == 0 ? g.at.b[0] : k == 1 ? g.at.b[1] : k == 2 ? g.at.b[2] : g.at.w4;
         const float v = column_sum(part, (int)(g.B / 32), (int)g.hid, (int)c0, s.col);
         if (tid < 32) scalar(off + c0 + tid, v);
         return;
@@ -851,7 +852,7 @@ __device__ __forceinline__ void for_gradients(const GradArgs &g, S &&state, W &&
     const float2 v = loss_sum(g.diff, g.B, s.loss);
     if (tid == 0) {
         if (g.loss) *g.loss = v.x / (float)g.B;
-        scalar(g.off_b4, v.y);
+        scalar(g.at.b4, v.y);
     }
 }
 
@@ -873,13 +874,13 @@ __global__ void __launch_bounds__(256) k_adam(GradArgs g, AdamArgs a) {
     };
     for_gradients(
         g,
-        [&](int l, uint32_t i) {
-            const size_t o = (size_t)g.off[l] + i;
+        [&](int l, size_t i) {
+            const size_t o = g.at.w[l] + i;
             return AdamState{__ldcg(reinterpret_cast<float4 *>(a.p + o)), __ldcg(reinterpret_cast<float4 *>(a.m + o)),
                              __ldcg(reinterpret_cast<float4 *>(a.v + o))};
         },
-        [&](int l, uint32_t i, const AdamState &st, float4 q) {
-            const size_t o = (size_t)g.off[l] + i;
+        [&](int l, size_t i, const AdamState &st, float4 q) {
+            const size_t o = g.at.w[l] + i;
             float4 p = st.p, m = st.m, v = st.v;
             float c1, c2;
             corrections(c1, c2);
@@ -908,8 +909,8 @@ __global__ void __launch_bounds__(256) k_form_gradient(GradArgs g, float *__rest
     titan::ptx::grid_dep_launch();
     titan::ptx::grid_dep_wait();
     for_gradients(
-        g, [](int, uint32_t) { return 0; },
-        [&](int l, uint32_t i, int, float4 q) { *reinterpret_cast<float4 *>(out + g.off[l] + i) = q; },
+        g, [](int, size_t) { return 0; },
+        [&](int l, size_t i, int, float4 q) { *reinterpret_cast<float4 *>(out + g.at.w[l] + i) = q; },
         [&](size_t i, float q) { out[i] = q; });
 }
 
@@ -1056,9 +1057,7 @@ struct titan_mlp {
     bool own_stream = false;
     uint32_t in = 0, hid = 0;
     uint32_t spin_limit = 1u << 22;
-    size_t n_params = 0;
-    // parameters: [W1t (hid x in), b1, W2t (hid x hid), b2, W3t, b3, w4 (hid), b4 (1)]
-    size_t off_w[3] = {0, 0, 0}, off_b[3] = {0, 0, 0}, off_w4 = 0, off_b4 = 0;
+    titan::MlpLayout at;                                   // of the parameters in p, g, m, v
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     // BF16 W^T [hid][in_l]: B operand of the forward product and, read with hid as
     // its K, of the input gradient
@@ -1129,7 +1128,7 @@ int wgrad_splits(uint32_t hid, uint32_t in, uint32_t B) {
 cudaError_t refresh_bf16(titan_mlp *m) {
     for (int l = 0; l < 3; ++l) {
         const size_t n = (size_t)m->hid * layer_in(m, l);
-        k_f32_to_bf16<<<nblk(n, 256), 256, 0, m->stream>>>(m->p + m->off_w[l], m->wt[l], n);
+        k_f32_to_bf16<<<nblk(n, 256), 256, 0, m->stream>>>(m->p + m->at.w[l], m->wt[l], n);
     }
     return cudaGetLastError();
 }
@@ -1165,7 +1164,7 @@ cudaError_t hidden_layers(titan_mlp *m, const __nv_bfloat16 *x, uint32_t B, bool
     cudaError_t e;
     const __nv_bfloat16 *a = x;
     for (int l = 0; l < 3; ++l) {
-        EpiArgs ep{EPI_BIAS_GELU, (int)m->hid, m->p + m->off_b[l], keep ? m->Z[l] : nullptr, m->H[l], nullptr};
+        EpiArgs ep{EPI_BIAS_GELU, (int)m->hid, m->p + m->at.b[l], keep ? m->Z[l] : nullptr, m->H[l], nullptr};
         if ((e = gemm_tn(a, m->wt[l], (int)B, (int)m->hid, (int)layer_in(m, l), ep, m->stream, m->spin_limit, m->err)) != cudaSuccess)
             return e;
         a = m->H[l];
@@ -1183,7 +1182,7 @@ cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, 
     if ((e = ensure_slices(m, B)) != cudaSuccess) return e;
     if ((e = hidden_layers(m, x, B, true)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_head, dim3(B / kHeadRows), kHeadThreads, 0, m->stream, m->H[2], m->Z[2], t,
-                              m->p + m->off_w4, m->p + m->off_b4, (int)B, hid, m->dZ[2], m->part, m->partb[2], m->diff,
+                              m->p + m->at.w4, m->p + m->at.b4, (int)B, hid, m->dZ[2], m->part, m->partb[2], m->diff,
                               train ? m->d_step : nullptr)) != cudaSuccess)
         return e;
     for (int l = 2; l > 0; --l) {
@@ -1209,17 +1208,13 @@ cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, 
         blocks += splits * w.tiles[l];
         at += (size_t)splits * m->hid * in;
         g->part[l] = w.out[l];
-        g->off[l] = (uint32_t)m->off_w[l];
-        g->n[l] = m->hid * in;
         g->splits[l] = (uint32_t)splits;
         g->vpart[l] = m->partb[l];
-        g->voff[l] = (uint32_t)m->off_b[l];
     }
+    g->at = m->at;
     g->hid = m->hid;
     g->vpart[3] = m->part;
-    g->voff[3] = (uint32_t)m->off_w4;
     g->diff = m->diff;
-    g->off_b4 = (uint32_t)m->off_b4;
     g->B = B;
     g->loss = loss;
     return wgrad_launch(w, blocks, hid, m->stream, m->spin_limit, m->err);
@@ -1227,7 +1222,9 @@ cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, 
 
 // The grid of k_adam and k_form_gradient (see for_gradients).
 unsigned gradient_blocks(const GradArgs &g) {
-    return (g.n[0] >> 10) + (g.n[1] >> 10) + (g.n[2] >> 10) + 4 * (g.hid >> 5) + 1;
+    unsigned blocks = 4 * (g.hid >> 5) + 1;
+    for (size_t n : g.at.n_w) blocks += titan::grad_blocks(n);
+    return blocks;
 }
 
 titan_status check_err(titan_mlp *m) {
@@ -1317,18 +1314,8 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     m->device = device;
     m->in = in;
     m->hid = hidden;
-    size_t o = 0;
-    for (int l = 0; l < 3; ++l) {
-        m->off_w[l] = o;
-        o += (size_t)hidden * (l == 0 ? in : hidden);
-        m->off_b[l] = o;
-        o += hidden;
-    }
-    m->off_w4 = o;
-    o += hidden;
-    m->off_b4 = o;
-    o += 1;
-    m->n_params = o;
+    m->at = titan::mlp_layout(in, hidden);
+    const size_t o = m->at.total;
     auto bail = [&](titan_status st) {
         titan::set_thread_error(m->error);
         for (void *p : m->allocs) cudaFree(p);
@@ -1370,12 +1357,12 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     for (int l = 0; l < 3; ++l) {
         const float a = std::sqrt(6.0f / (float)layer_in(m, l));
         std::uniform_real_distribution<float> U(-a, a);
-        for (size_t k = 0; k < (size_t)hidden * layer_in(m, l); ++k) h[m->off_w[l] + k] = U(rng);
+        for (size_t k = 0; k < (size_t)hidden * layer_in(m, l); ++k) h[m->at.w[l] + k] = U(rng);
     }
     {
         const float a = std::sqrt(3.0f / (float)hidden);
         std::uniform_real_distribution<float> U(-a, a);
-        for (uint32_t k = 0; k < hidden; ++k) h[m->off_w4 + k] = U(rng);
+        for (uint32_t k = 0; k < hidden; ++k) h[m->at.w4 + k] = U(rng);
     }
     C_CK(cudaMemcpy(m->p, h.data(), o * 4, cudaMemcpyHostToDevice));
     C_CK(cudaMemset(m->m, 0, o * 4));
@@ -1388,19 +1375,19 @@ titan_status titan_mlp_create(uint32_t in, uint32_t hidden, uint64_t seed, int32
     return TITAN_OK;
 }
 
-uint64_t titan_mlp_param_count(const titan_mlp *m) { return m ? m->n_params : 0; }
+uint64_t titan_mlp_param_count(const titan_mlp *m) { return m ? m->at.total : 0; }
 
 titan_status titan_mlp_get_params(titan_mlp *m, float *host) {
     if (!m || !host) return TITAN_E_INVALID;
     MLP_CK(m, cudaStreamSynchronize(m->stream));
-    MLP_CK(m, cudaMemcpy(host, m->p, m->n_params * 4, cudaMemcpyDeviceToHost));
+    MLP_CK(m, cudaMemcpy(host, m->p, m->at.total * 4, cudaMemcpyDeviceToHost));
     return TITAN_OK;
 }
 
 titan_status titan_mlp_set_params(titan_mlp *m, const float *host) {
     if (!m || !host) return TITAN_E_INVALID;
     MLP_CK(m, cudaStreamSynchronize(m->stream));
-    MLP_CK(m, cudaMemcpy(m->p, host, m->n_params * 4, cudaMemcpyHostToDevice));
+    MLP_CK(m, cudaMemcpy(m->p, host, m->at.total * 4, cudaMemcpyHostToDevice));
     MLP_CK(m, refresh_bf16(m));
     return check_err(m);
 }
@@ -1411,8 +1398,8 @@ titan_status titan_mlp_forward(titan_mlp *m, const uint16_t *x_dev, uint32_t bat
     MLP_CK(m, cudaSetDevice(m->device));
     MLP_CK(m, ensure_batch(m, batch));
     MLP_CK(m, hidden_layers(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), batch, false));
-    MLP_CK(m, launch_dependent(k_out_layer, dim3(nblk(batch, 8)), 256, 0, m->stream, m->H[2], m->p + m->off_w4,
-                               m->p + m->off_b4, y_dev, (int)batch, (int)m->hid));
+    MLP_CK(m, launch_dependent(k_out_layer, dim3(nblk(batch, 8)), 256, 0, m->stream, m->H[2], m->p + m->at.w4,
+                               m->p + m->at.b4, y_dev, (int)batch, (int)m->hid));
     return check_err(m);
 }
 
@@ -1425,7 +1412,7 @@ titan_status titan_mlp_gradient(titan_mlp *m, const uint16_t *x_dev, const float
     GradArgs g;
     MLP_CK(m, backward_pass(m, reinterpret_cast<const __nv_bfloat16 *>(x_dev), t_dev, batch, loss_dev, &g, false));
     MLP_CK(m, launch_dependent(k_form_gradient, dim3(gradient_blocks(g)), 256, 0, m->stream, g, m->g));
-    if (grad_dev) MLP_CK(m, cudaMemcpyAsync(grad_dev, m->g, m->n_params * 4, cudaMemcpyDeviceToDevice, m->stream));
+    if (grad_dev) MLP_CK(m, cudaMemcpyAsync(grad_dev, m->g, m->at.total * 4, cudaMemcpyDeviceToDevice, m->stream));
     return check_err(m);
 }
 
