@@ -775,7 +775,7 @@ __device__ __forceinline__ float2 loss_sum(const float *diff, uint32_t B, float2
 // each; loss and b4: the head's y - t.
 struct GradArgs {
     titan::MlpLayout at;
-    const float *part[3];                 // [splits][hid][in_l]
+    const float *part[3];                 // [splits][hid][in_l] (one slice: in the gradient array)
     uint32_t splits[3], hid;
     const float *vpart[4];
     const float *diff;
@@ -904,8 +904,8 @@ __global__ void __launch_bounds__(256) k_adam(GradArgs g, AdamArgs a) {
         });
 }
 
-// The same gradients into the flat array out.
-__global__ void __launch_bounds__(256) k_form_gradient(GradArgs g, float *__restrict__ out) {
+// The same gradients into the flat array out (a layer of one slice is there already).
+__global__ void __launch_bounds__(256) k_form_gradient(GradArgs g, float *out) {
     titan::ptx::grid_dep_launch();
     titan::ptx::grid_dep_wait();
     for_gradients(
@@ -1069,7 +1069,7 @@ struct titan_mlp {
     float *part = nullptr;                                 // dw4: sums of 32 rows [B / 32][hidden]
     float *partb[3] = {nullptr, nullptr, nullptr};         // the same for db_l
     float *diff = nullptr;                                 // y - t
-    float *wsk = nullptr;                                  // K slices of the weight gradients
+    float *wsk = nullptr;                                  // K slices of the weight gradients (layers of several)
     size_t wsk_cap = 0;                                    // floats
     volatile int *err_host = nullptr;                      // bounded-wait flag: pinned, mapped
     int *err = nullptr;
@@ -1148,11 +1148,14 @@ cudaError_t ensure_batch(titan_mlp *m, uint32_t B) {
     return cudaSuccess;
 }
 
-// The slices of the weight gradients (their number depends on the batch).
+// The slices of the weight gradients (their number depends on the batch).  A layer of
+// one slice needs none: its product goes straight to the gradient array.
 cudaError_t ensure_slices(titan_mlp *m, uint32_t B) {
     size_t ws = 0;
-    for (int l = 0; l < 3; ++l)
-        ws += (size_t)wgrad_splits(m->hid, layer_in(m, l), B) * m->hid * layer_in(m, l);
+    for (int l = 0; l < 3; ++l) {
+        const int splits = wgrad_splits(m->hid, layer_in(m, l), B);
+        if (splits > 1) ws += splits * m->at.n_w[l];
+    }
     if (ws <= m->wsk_cap) return cudaSuccess;
     cudaError_t e = malloc_t(m, &m->wsk, ws);
     if (e == cudaSuccess) m->wsk_cap = ws;
@@ -1199,14 +1202,14 @@ cudaError_t backward_pass(titan_mlp *m, const __nv_bfloat16 *x, const float *t, 
         const int splits = wgrad_splits(m->hid, in, B);
         if (!make_map(&w.a[l], m->dZ[l], B, m->hid, 64) || !make_map(&w.b[l], l ? m->H[l - 1] : x, B, in, 64))
             return cudaErrorInvalidValue;
-        w.out[l] = m->wsk + at;
+        w.out[l] = splits > 1 ? m->wsk + at : m->g + m->at.w[l];
         w.first[l] = blocks;
         w.tiles_n[l] = (int)(in / BN);
         w.tiles[l] = (int)(m->hid / BM) * w.tiles_n[l];
         w.ld[l] = (int)in;
         w.kslice[l] = (int)B / splits;
         blocks += splits * w.tiles[l];
-        at += (size_t)splits * m->hid * in;
+        if (splits > 1) at += splits * m->at.n_w[l];
         g->part[l] = w.out[l];
         g->splits[l] = (uint32_t)splits;
         g->vpart[l] = m->partb[l];
