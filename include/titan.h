@@ -285,9 +285,9 @@ titan_status titan_set_step(titan_sim *sim, uint64_t step);
  * robots; the paper's Sec. III-F shape and actuation optimisation done with
  * gradients).  From the current state and step, runs n_steps ordinary steps
  * (the simulation advances as titan_step would), keeping every state if they
- * take at most 1 GiB, else the state every `every` steps (0: 50) and
- * recomputing each segment but the last from its checkpoint, and reverses them,
- * accumulating
+ * take at most 1 GiB and the device has room for them, else the state every
+ * `every` steps (0: 50) and recomputing each segment but the last from its
+ * checkpoint, and reverses them, accumulating
  *   grad_amp_dev[s]   = dJ / dA_s,    grad_phase_dev[s] = dJ / dphi_s
  * for J = sum_i seed_pos[i] . x_T[i] + seed_vel[i] . v_T[i] (x_T, v_T: the
  * state after the rollout).  All arrays are DEVICE float arrays in caller

@@ -261,6 +261,7 @@ titan_status afail(titan_sim *sim, titan_status st, const std::string &msg) {
         if (e_ != cudaSuccess) {                                                                   \
             st_ = afail(sim, e_ == cudaErrorMemoryAllocation ? TITAN_E_OOM : TITAN_E_CUDA,         \
                         std::string(#call) + ": " + cudaGetErrorString(e_));                        \
+            cudaGetLastError();                                                                    \
             goto done;                                                                             \
         }                                                                                          \
     } while (0)
@@ -320,20 +321,37 @@ extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t
             sim->d_adj_nbr = static_cast<uint32_t *>(p1);
             sim->d_adj_owner = static_cast<uint32_t *>(p2);
         }
-        const bool whole = n_steps < kAdjTrajectory / state_bytes;
-        const uint64_t len_max = whole ? n_steps : every;
-        n_seg = whole ? (n_steps ? 1 : 0) : (n_steps + every - 1) / every;
         const unsigned gm = (nd + kT - 1) / kT, ga = (nd + kAdjT - 1) / kAdjT;
         ADJ_CK(adjoint_pool(sim->device, &pool));
         auto take = [&](auto **p, size_t bytes) { return cudaMallocFromPoolAsync((void **)p, bytes, pool, s); };
-        if (n_seg > 1) ADJ_CK(take(&ckpt, state_bytes * (n_seg - 1)));
-        ADJ_CK(take(&seg, state_bytes * (len_max + 1)));
         ADJ_CK(take(&xb, vec_bytes));
         ADJ_CK(take(&vb, vec_bytes));
         for (int b = 0; b < 2; ++b) ADJ_CK(take(&Fb[b], vec_bytes));
-        ADJ_CK(take(&seg_steps, sizeof(long long) * (len_max + 1)));
         ADJ_CK(take(&gacc, std::max<size_t>(E, 1) * sizeof(float2)));
         ADJ_CK(take(&row, std::max<size_t>(E, 1) * sizeof(float4)));
+        // the states: all of them in one segment, or, if that is too much or the device has no
+        // room for it, segments of `every` steps
+        uint64_t len_max = 0;
+        auto keep = [&](bool whole) {
+            len_max = whole ? n_steps : std::min<uint64_t>(every, n_steps);
+            n_seg = n_steps ? (n_steps + len_max - 1) / len_max : 0;
+            cudaError_t e = n_seg > 1 ? take(&ckpt, state_bytes * (n_seg - 1)) : cudaSuccess;
+            if (e == cudaSuccess) e = take(&seg, state_bytes * (len_max + 1));
+            if (e == cudaSuccess) e = take(&seg_steps, sizeof(long long) * (len_max + 1));
+            return e;
+        };
+        bool whole = n_steps < kAdjTrajectory / state_bytes;
+        if (whole) {
+            const cudaError_t room = keep(true);
+            whole = !(room == cudaErrorMemoryAllocation && n_steps > every);
+            if (whole) ADJ_CK(room);
+        }
+        if (!whole) {
+            cudaGetLastError();
+            if (seg) cudaFreeAsync(seg, s);           // taken for the whole trajectory before the room ran out
+            seg = nullptr;
+            ADJ_CK(keep(false));
+        }
         ADJ_CK(cudaMemsetAsync(gacc, 0, std::max<size_t>(E, 1) * sizeof(float2), s));
         if (E) {
             k_adj_rows<<<(E + kT - 1) / kT, kT, 0, s>>>(sim->d_kl, sim->d_act, E, row);
