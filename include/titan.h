@@ -285,9 +285,9 @@ titan_status titan_set_step(titan_sim *sim, uint64_t step);
  * robots; the paper's Sec. III-F shape and actuation optimisation done with
  * gradients).  From the current state and step, runs n_steps ordinary steps
  * (the simulation advances as titan_step would), keeping every state if they
- * take at most 1 GiB and the device has room for them, else the state every
- * `every` steps (0: 50) and recomputing each segment but the last from its
- * checkpoint, and reverses them, accumulating
+ * take at most 1 GiB (titan_adjoint_limit) and the device has room for them,
+ * else the state every `every` steps (0: 50) and recomputing each segment but
+ * the last from its checkpoint, and reverses them, accumulating
  *   grad_amp_dev[s]   = dJ / dA_s,    grad_phase_dev[s] = dJ / dphi_s
  * for J = sum_i seed_pos[i] . x_T[i] + seed_vel[i] . v_T[i] (x_T, v_T: the
  * state after the rollout).  All arrays are DEVICE float arrays in caller
@@ -296,10 +296,20 @@ titan_status titan_set_step(titan_sim *sim, uint64_t step);
  * actuation set with titan_set_actuation or titan_set_actuation_dev.  At the
  * kinks of contact and friction the derivative of the branch the forward step
  * took is used.
+ * The workspaces come from a memory pool of the library's own, one per device,
+ * which keeps up to 2 GiB of them for the next call; the driver takes that
+ * memory for any allocation that needs it, and titan_destroy of a simulation
+ * that called titan_adjoint gives it back.
  * Enqueued on the simulation stream.  Errors: TITAN_E_INVALID,
  * TITAN_E_UNSUPPORTED (atomic accumulation), TITAN_E_OOM, TITAN_E_CUDA. */
 titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t every, const float *seed_pos_dev,
                            const float *seed_vel_dev, float *grad_amp_dev, float *grad_phase_dev);
+
+/* Sets the most device memory the later titan_adjoint calls on this handle
+ * take to keep every state of a rollout, 32 bytes per mass slot and step
+ * (default 1 GiB; 0: checkpoints at every `every` steps always).  The gradients
+ * are the same bits either way.  Errors: TITAN_E_INVALID, TITAN_E_BUSY. */
+titan_status titan_adjoint_limit(titan_sim *sim, uint64_t bytes);
 
 /* Blocks until every enqueued step and copy has finished (the paper's
  * waitForEvent, Sec. III-D).  Errors: TITAN_E_CUDA, TITAN_E_TIMEOUT. */

@@ -3,7 +3,7 @@
 //
 // Forward: the ordinary step (Titan Sec. III-B, Eq. 1; Sec. III-A contact,
 // friction and constraints) with L = L0 (1 + A sin(2 pi f t + phi)).  The
-// rollout runs forward once, keeping every state if they fit (kAdjTrajectory),
+// rollout runs forward once, keeping every state if they fit (titan_adjoint_limit),
 // else the state every `every` steps (checkpoints) and the states of the last
 // segment; earlier segments are recomputed from their checkpoints.  Then, from
 // the last step back, k_adj_step reverses one step per launch, per mass:
@@ -31,9 +31,6 @@ namespace {
 constexpr int kT = 256;
 constexpr uint32_t kOwner = 0x80000000u;
 constexpr int kAdjT = 128;
-// The whole trajectory of a rollout is kept when it takes at most this (1/280 of
-// the memory), so that no step runs twice; longer ones are checkpointed.
-constexpr size_t kAdjTrajectory = (size_t)1 << 30;
 
 // The adjoint a force on a mass carries, from (x_b, v_b) of the state after the step:
 // v' = v + (F / m + ...) dt and x' = x + v' dt.
@@ -214,10 +211,12 @@ __global__ void k_adj_force0(const MassState *__restrict__ X, const float4 *__re
 }
 
 // The workspaces of titan_adjoint come from a pool of the library's own per
-// device, stream-ordered like the default pool but keeping up to twice
-// kAdjTrajectory between calls (the default pool gives every byte back at each
+// device, stream-ordered like the default pool but keeping up to kAdjKeep
+// between calls (the default pool gives every byte back at each
 // synchronisation, and mapping them again took as long as dozens of steps).
-// adjoint_trim gives the memory back (titan_destroy).
+// adjoint_trim gives the memory back (titan_destroy); before that the driver takes
+// it for any allocation that needs it.
+constexpr uint64_t kAdjKeep = 2ull << 30;
 // Kept while the device's context lives (a cudaDeviceReset destroys it).
 struct Pool {
     unsigned long long ctx_id = 0;
@@ -238,7 +237,7 @@ cudaError_t adjoint_pool(int dev, cudaMemPool_t *out) {
         cudaMemPool_t p = nullptr;
         cudaError_t e = cudaMemPoolCreate(&p, &props);
         if (e != cudaSuccess) return e;
-        uint64_t keep = 2 * kAdjTrajectory;
+        uint64_t keep = kAdjKeep;
         e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
         if (e != cudaSuccess) {
             cudaMemPoolDestroy(p);
@@ -272,6 +271,14 @@ void titan::adjoint_trim(int dev) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     if (dev >= 0 && dev < 64 && g_pool[dev].pool && g_pool[dev].ctx_id == titan::current_context_id())
         cudaMemPoolTrimTo(g_pool[dev].pool, 0);
+}
+
+extern "C" titan_status titan_adjoint_limit(titan_sim *sim, uint64_t bytes) {
+    if (!sim) return TITAN_E_INVALID;
+    if (sim->busy.exchange(true)) return afail(sim, TITAN_E_BUSY, "another call on this handle is in progress");
+    sim->adj_limit = bytes;
+    sim->busy.store(false);
+    return TITAN_OK;
 }
 
 extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t every,
@@ -340,7 +347,7 @@ extern "C" titan_status titan_adjoint(titan_sim *sim, uint64_t n_steps, uint32_t
             if (e == cudaSuccess) e = take(&seg_steps, sizeof(long long) * (len_max + 1));
             return e;
         };
-        bool whole = n_steps < kAdjTrajectory / state_bytes;
+        bool whole = n_steps < sim->adj_limit / state_bytes;       // n_steps + 1 states
         if (whole) {
             const cudaError_t room = keep(true);
             whole = !(room == cudaErrorMemoryAllocation && n_steps > every);

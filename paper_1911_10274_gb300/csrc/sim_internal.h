@@ -142,6 +142,7 @@ struct SimCore {
 struct titan_sim : SimCore {
     std::string error;
     std::atomic<bool> busy{false};
+    uint64_t adj_limit = 1ull << 30;      // most bytes of states titan_adjoint keeps at once to avoid checkpoints
 };
 
 namespace titan {

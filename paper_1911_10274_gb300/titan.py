@@ -99,6 +99,7 @@ def load(path: Optional[str] = None):
                 "titan_add_masses": (S, [_P, u32, _P, _P, _P, _P, C.POINTER(u32)]),
                 "titan_set_fixed": (S, [_P, u32, _P, _P]),
                 "titan_adjoint": (S, [_P, u64, u32, _P, _P, _P, _P]),
+                "titan_adjoint_limit": (S, [_P, u64]),
                 "titan_gemm_bf16_tn": (S, [u32, u32, u32, _P, _P, _P, _P]),
                 "titan_gemm_check": (S, []),
                 "titan_mlp_create": (S, [u32, u32, u64, C.c_int32, _P, C.POINTER(_P)]),
@@ -295,6 +296,12 @@ def titan_adjoint(sim: int, n_steps: int, every: int, seed_pos_dev, seed_vel_dev
                   grad_phase_dev) -> None:
     _check(load().titan_adjoint(sim, n_steps, every, _ptr(seed_pos_dev), _ptr(seed_vel_dev),
                                 _ptr(grad_amp_dev), _ptr(grad_phase_dev)), sim)
+
+
+def titan_adjoint_limit(sim: int, n_bytes: int) -> None:
+    """The most device memory later titan_adjoint calls take to keep every state of a
+    rollout (default 1 GiB; 0: always checkpoints every ``every`` steps)."""
+    _check(load().titan_adjoint_limit(sim, n_bytes), sim)
 
 
 def titan_sync(sim: int) -> None:
@@ -631,7 +638,8 @@ class CentroidRollout:
 
     ``__call__(amp, phase)`` takes CUDA float32 tensors and returns a tensor
     of per-robot displacements; gradients flow back through the library's
-    adjoint (titan_adjoint) with checkpoints every ``every`` steps."""
+    adjoint (titan_adjoint), which keeps every state of the rollout if they take
+    at most 1 GiB (titan_adjoint_limit), else one every ``every`` steps."""
 
     def __init__(self, robots, n_steps: int, every: int = 50, device: int = 0, order: int = ORDER_MORTON):
         import torch
