@@ -23,6 +23,7 @@
 #include <string>
 #include <vector>
 
+#include "context_id.h"
 #include "physics.cuh"
 #include "sim_internal.h"
 
@@ -217,7 +218,8 @@ __global__ void k_adj_force0(const MassState *__restrict__ X, const float4 *__re
 // adjoint_trim gives the memory back (titan_destroy); before that the driver takes
 // it for any allocation that needs it.
 constexpr uint64_t kAdjKeep = 2ull << 30;
-// Kept while the device's context lives (a cudaDeviceReset destroys it).
+// Kept while the device's context lives (a cudaDeviceReset destroys it); the device's
+// default pool serves where that cannot be told.
 struct Pool {
     unsigned long long ctx_id = 0;
     cudaMemPool_t pool = nullptr;
@@ -229,7 +231,8 @@ cudaError_t adjoint_pool(int dev, cudaMemPool_t *out) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_pool_mu);
     const unsigned long long id = titan::current_context_id();
-    if (!g_pool[dev].pool || g_pool[dev].ctx_id != id) {
+    if (id == 0) return cudaDeviceGetDefaultMemPool(out, dev);
+    if (!g_pool[dev].pool || !titan::same_context(g_pool[dev].ctx_id, id)) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -269,7 +272,7 @@ titan_status afail(titan_sim *sim, titan_status st, const std::string &msg) {
 
 void titan::adjoint_trim(int dev) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (dev >= 0 && dev < 64 && g_pool[dev].pool && g_pool[dev].ctx_id == titan::current_context_id())
+    if (dev >= 0 && dev < 64 && g_pool[dev].pool && same_context(g_pool[dev].ctx_id, current_context_id()))
         cudaMemPoolTrimTo(g_pool[dev].pool, 0);
 }
 

@@ -33,6 +33,7 @@
 #include <mutex>
 #include <string>
 
+#include "context_id.h"
 #include "physics.cuh"
 #include "ptx.cuh"
 #include "titan.h"
@@ -120,7 +121,7 @@ cudaError_t scratch_address(ScratchAddr *out, int *dev_out) {
     std::lock_guard<std::mutex> lk(g_addr_mu);
     const unsigned long long id = titan::current_context_id();
     *dev_out = dev;
-    if (id != 0 && g_addr[dev].ctx_id == id && g_addr[dev].ptr) {
+    if (titan::same_context(g_addr[dev].ctx_id, id) && g_addr[dev].ptr) {
         *out = g_addr[dev];
         return cudaSuccess;
     }
