@@ -34,8 +34,10 @@ constexpr uint32_t kOwner = 0x80000000u;
 constexpr int kAdjT = 128;
 
 // The adjoint a force on a mass carries, from (x_b, v_b) of the state after the step:
-// v' = v + (F / m + ...) dt and x' = x + v' dt.
+// v' = v + (F / m + ...) dt and x' = x + v' dt.  None on a fixed mass, whatever its own
+// adjoint is (its neighbours must not take an infinity or NaN times 0 from it).
 __device__ __forceinline__ float4 force_adjoint(float4 xo, float4 vo, float im, float dt) {
+    if (im == 0.f) return make_float4(0.f, 0.f, 0.f, 0.f);
     const float vtx = vo.x + dt * xo.x, vty = vo.y + dt * xo.y, vtz = vo.z + dt * xo.z;
     return make_float4(dt * vtx * im, dt * vty * im, dt * vtz * im, 0.f);
 }
