@@ -18,16 +18,15 @@
 // Spring records: one {i, j, k, L0} record per spring, sorted by (lower,
 // higher) device index, for the atomic scatter.
 #include "layout.h"
+#include "threads.h"
 
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <climits>
-#include <new>
 #include <numeric>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <utility>
 
@@ -470,26 +469,7 @@ bool build_halo(uint32_t n, const SellHost &sell, uint32_t max_slots, bool grid_
         my.groups = groups;
         my.wavefronts = wavefronts;
     };
-    std::atomic<bool> no_memory{false};
-    auto guarded = [&](uint32_t part) {
-        try {
-            build(part);
-        } catch (const std::bad_alloc &) {
-            no_memory.store(true);
-        }
-    };
-    std::vector<std::thread> pool;
-    pool.reserve(nt);
-    for (uint32_t t = 1; t < nt; ++t) {
-        try {
-            pool.emplace_back(guarded, t);
-        } catch (const std::system_error &) {
-            guarded(t);                       // no thread to be had: on this one
-        }
-    }
-    guarded(0);
-    for (auto &th : pool) th.join();
-    if (no_memory.load()) throw std::bad_alloc();
+    run_parts(nt, build);
     if (!fits.load()) return false;
     uint64_t groups = 0, wavefronts = 0;
     uint32_t b = 0;

@@ -21,6 +21,7 @@
 #include "group_mean.cuh"
 #include "layout.h"
 #include "sim_internal.h"
+#include "threads.h"
 #include "titan.h"
 #include "titan_internal.h"
 
@@ -274,14 +275,7 @@ bool fill_state_parallel(const titan_sim *sim, const double *pos, const double *
             out[d] = m;
         }
     };
-    if (nt == 1) {
-        work(0);
-    } else {
-        std::vector<std::thread> pool;
-        for (unsigned t = 1; t < nt; ++t) pool.emplace_back(work, t);
-        work(0);
-        for (auto &th : pool) th.join();
-    }
+    titan::run_parts(nt, work);
     return ok.load();
 }
 
