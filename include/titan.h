@@ -332,6 +332,20 @@ int32_t titan_exec_mode(const titan_sim *sim);
  * layout rebuild. */
 int32_t titan_csr_kernel(const titan_sim *sim);
 
+/* Forms that some kernels come in, chosen by size and options; every form of a
+ * kernel gives the same bits (batches: with one thread per mass). */
+enum {
+    TITAN_FORM_PLAIN = 0, /* the general form                                       */
+    TITAN_FORM_ROWS = 1,  /* persistent and batch kernels: a thread per mass, whose
+                             row (at most 26 entries) stays in its registers        */
+    TITAN_FORM_DEEP = 2   /* step kernels 4 and 6: four columns of the row stream at
+                             a time, on grids of at most two CTAs per SM            */
+};
+
+/* The form in which titan_step runs this system now (TITAN_FORM_*), -1 for a
+ * NULL handle. */
+int32_t titan_step_form(const titan_sim *sim);
+
 /* Text of the last error on this handle, or of the last failed titan_create
  * on this thread when sim is NULL.  Owned by the library; never NULL. */
 const char *titan_last_error(const titan_sim *sim);
@@ -451,12 +465,17 @@ titan_status titan_batch_read(titan_batch *b, uint32_t system, float *pos, float
  * enqueued work.  Waits. */
 titan_status titan_batch_centroids(titan_batch *b, float *out);
 
-/* Number of launch groups and, per group, its cluster size, the looped form's
- * threads per CTA and most threads per mass, and its CTA count (outputs may be
- * NULL). */
+/* Number of launch groups and, per group, its cluster size, the general (looped)
+ * form's threads per CTA and most threads per mass, and its CTA count (outputs
+ * may be NULL). */
 uint32_t titan_batch_groups(const titan_batch *b);
 titan_status titan_batch_info(const titan_batch *b, uint32_t group, uint32_t *cluster,
                               uint32_t *threads, uint32_t *threads_per_mass, uint32_t *ctas);
+
+/* The form in which a launch group runs: TITAN_FORM_ROWS (one thread per mass)
+ * or TITAN_FORM_PLAIN (the shape of titan_batch_info), and the threads per CTA it
+ * is launched with (may be NULL).  -1 for a null batch or a group out of range. */
+int32_t titan_batch_form(const titan_batch *b, uint32_t group, uint32_t *threads);
 
 /* The launch group (0 .. titan_batch_groups - 1) whose launches advance
  * system `system`.  TITAN_E_INVALID for a null batch or output, or a system

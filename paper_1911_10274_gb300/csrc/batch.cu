@@ -885,6 +885,13 @@ titan_status titan_batch_info(const titan_batch *b, uint32_t group, uint32_t *cl
     return TITAN_OK;
 }
 
+int32_t titan_batch_form(const titan_batch *b, uint32_t group, uint32_t *threads) {
+    if (!b || group >= b->groups.size()) return -1;
+    const Group &g = b->groups[group];
+    if (threads) *threads = g.rows ? g.row_threads : g.threads;
+    return g.rows ? TITAN_FORM_ROWS : TITAN_FORM_PLAIN;
+}
+
 titan_status titan_batch_configure(titan_batch *b, uint32_t group, uint32_t threads, uint32_t threads_per_mass) {
     if (!b || group >= b->groups.size()) return bfail(b, TITAN_E_INVALID, "batch is null or group out of range");
     if (threads < 32 || threads > 1024 || threads % 32 ||

@@ -1299,6 +1299,14 @@ int32_t titan_csr_kernel(const titan_sim *sim) {
     return sim->accumulate == TITAN_ACCUM_CSR ? sim->csr_kernel : 0;
 }
 
+int32_t titan_step_form(const titan_sim *sim) {
+    if (!sim) return -1;
+    if (sim->persistent) return sim->persist_rows ? TITAN_FORM_ROWS : TITAN_FORM_PLAIN;
+    if (sim->accumulate != TITAN_ACCUM_CSR || (sim->csr_kernel != 4 && sim->csr_kernel != 6)) return TITAN_FORM_PLAIN;
+    DeviceGuard dg(sim->device);
+    return titan::step_is_deep(sim->n_dev) ? TITAN_FORM_DEEP : TITAN_FORM_PLAIN;
+}
+
 const char *titan_last_error(const titan_sim *sim) {
     return sim ? sim->error.c_str() : g_thread_error.c_str();
 }

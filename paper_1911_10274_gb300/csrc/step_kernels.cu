@@ -1199,6 +1199,8 @@ static bool deep_grid(unsigned blocks) {
     return cudaGetDevice(&dev) == cudaSuccess &&
            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && blocks <= 2u * (unsigned)sms;
 }
+static unsigned halo_grid(uint32_t n) { return n ? (n + kHaloThreads - 1) / kHaloThreads : 1; }
+bool step_is_deep(uint32_t n) { return deep_grid(halo_grid(n)); }
 
 // The launch attributes of a step kernel: the L2 window (optional) and
 // programmatic stream serialization (overlap).
@@ -1222,7 +1224,7 @@ cudaError_t launch_step_halo(const MassState *in, MassState *out, uint32_t n, co
                              long long *step_out, cudaStream_t stream, const cudaAccessPolicyWindow *l2win,
                              bool overlap) {
     const bool hc = v.c != nullptr, ha = v.act != nullptr, gr = c.ground != 0;
-    const unsigned g = n ? (n + kHaloThreads - 1) / kHaloThreads : 1;
+    const unsigned g = halo_grid(n);
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
     const bool deep = deep_grid(g);
     const int act = ha ? (c.act_mode == 2 ? kActWorm : kActSinusoid) : kActNone;
@@ -1272,7 +1274,7 @@ cudaError_t launch_step_box(const MassState *in, MassState *out, uint32_t n, con
                             const StepConst &c, const long long *step_in, long long *step_out,
                             cudaStream_t stream, const cudaAccessPolicyWindow *l2win, bool overlap) {
     const bool hc = v.c != nullptr, ha = v.act != nullptr, gr = c.ground != 0;
-    const unsigned g = n ? (n + kHaloThreads - 1) / kHaloThreads : 1;
+    const unsigned g = halo_grid(n);
     const size_t bytes = (size_t)h.table_slots * (sizeof(float4) + sizeof(float2));
     if (reinterpret_cast<uintptr_t>(h.col_off) & 3) return cudaErrorInvalidValue;
     const bool deep = deep_grid(g);

@@ -186,6 +186,9 @@ struct PersistArgs {
     uint32_t halo_off[9];
 };
 
+// Whether the halo and box step kernels take their deep form for n masses on the current device.
+bool step_is_deep(uint32_t n);
+
 // n_steps steps in one launch: reads `in`, writes `out` once at the end;
 // step_out = step_in + n_steps.
 // push, push_more: the copy lists of invert_halos, by device mass (null: the

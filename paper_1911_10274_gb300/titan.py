@@ -22,6 +22,7 @@ TITAN_OK, TITAN_E_INVALID, TITAN_E_CUDA, TITAN_E_OOM, TITAN_E_TIMEOUT, TITAN_E_B
 ACCUM_CSR, ACCUM_ATOMIC = 0, 1
 ORDER_INPUT, ORDER_MORTON = 0, 1
 EXEC_AUTO, EXEC_LAUNCH, EXEC_PERSISTENT = 0, 1, 2
+FORM_PLAIN, FORM_ROWS, FORM_DEEP = 0, 1, 2
 _STATUS = {0: "TITAN_OK", 1: "TITAN_E_INVALID", 2: "TITAN_E_CUDA", 3: "TITAN_E_OOM",
            4: "TITAN_E_TIMEOUT", 5: "TITAN_E_BUSY", 6: "TITAN_E_UNSUPPORTED"}
 
@@ -86,6 +87,8 @@ def load(path: Optional[str] = None):
                 "titan_steps": (u64, [_P]),
                 "titan_csr_kernel": (C.c_int32, [_P]),
                 "titan_exec_mode": (C.c_int32, [_P]),
+                "titan_step_form": (C.c_int32, [_P]),
+                "titan_batch_form": (C.c_int32, [_P, u32, C.POINTER(u32)]),
                 "titan_last_error": (C.c_char_p, [_P]),
                 "titan_destroy": (S, [_P]),
                 "titan_step_atomic_noalloc": (S, [u32, _P, _P, _P, u32, _P, _P, _P, f32,
@@ -482,13 +485,18 @@ class Batch:
         _bcheck(load().titan_batch_configure(self.handle, group, threads, threads_per_mass), self.handle)
 
     def groups(self):
+        """Per launch group: cluster size, CTAs, the looped form's threads per CTA and per mass, and what
+        is launched: its form (FORM_ROWS: one thread per mass, or FORM_PLAIN) and threads per CTA."""
         lib = load()
         res = []
         for g in range(lib.titan_batch_groups(self.handle)):
             cl, th, tm, ct = C.c_uint32(), C.c_uint32(), C.c_uint32(), C.c_uint32()
             _bcheck(lib.titan_batch_info(self.handle, g, C.byref(cl), C.byref(th), C.byref(tm), C.byref(ct)),
                     self.handle)
-            res.append(dict(cluster=cl.value, threads=th.value, threads_per_mass=tm.value, ctas=ct.value))
+            lt = C.c_uint32()
+            form = lib.titan_batch_form(self.handle, g, C.byref(lt))
+            res.append(dict(cluster=cl.value, threads=th.value, threads_per_mass=tm.value, ctas=ct.value, form=form,
+                            launch_threads=lt.value))
         return res
 
     def close(self) -> None:
@@ -587,6 +595,11 @@ class Sim:
     def exec_mode(self) -> int:
         """EXEC_PERSISTENT or EXEC_LAUNCH: how titan_step runs this system."""
         return int(load().titan_exec_mode(self.handle))
+
+    @property
+    def step_form(self) -> int:
+        """FORM_PLAIN, FORM_ROWS or FORM_DEEP: the form of the kernel that titan_step runs."""
+        return int(load().titan_step_form(self.handle))
 
     @property
     def csr_kernel(self) -> int:
