@@ -1,28 +1,29 @@
 """Checkpointed gradients of small robots (the limit on kept states set so that the whole trajectory is not
-kept): the bits of the whole trajectory's, whatever the interval, within 1e-3 of the FP64 oracle, and the
-simulation left where plain steps leave it."""
+kept): the bits of the whole trajectory's, whatever the interval, and the simulation left where it leaves it;
+and, on the robots that test_gpu_adjoint holds the whole trajectory to, the FP64 oracle's gradients."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_1911_10274_gb300 import inputs
 from paper_1911_10274_gb300 import titan as T
-from test_gpu_adjoint import _close
+from test_gpu_adjoint import _close, _robot
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 STEPS = 120
 
 
-def _run(sy, every, limit):
+def _run(sy, every, limit, seed=None, steps=STEPS):
     with T.Sim(sy) as sim:
         if limit is not None:
             T.titan_adjoint_limit(sim.handle, limit)
-        s = torch.as_tensor(oracle.centroid_x_seed(sy.n_masses), dtype=torch.float32, device="cuda")
+        seed = oracle.centroid_x_seed(sy.n_masses) if seed is None else seed
+        s = torch.as_tensor(seed, dtype=torch.float32, device="cuda")
         ga = torch.full((sy.n_springs,), float("nan"), device="cuda")
         gp = torch.full_like(ga, float("nan"))
         torch.cuda.synchronize()
-        T.titan_adjoint(sim.handle, STEPS, every, s, None, ga, gp)
+        T.titan_adjoint(sim.handle, steps, every, s, None, ga, gp)
         sim.step(3)
         x, v, t = sim.snapshot()
     return ga.cpu().numpy(), gp.cpu().numpy(), x.copy(), v.copy(), t
@@ -36,9 +37,18 @@ def test_checkpoints_give_the_bits_of_the_whole_trajectory(every):
         got = _run(sy, every, limit)
         for a, b in zip(whole, got):
             assert np.array_equal(a, b)
-    ra, rp, _, _ = oracle.adjoint(sy, STEPS, oracle.centroid_x_seed(sy.n_masses))
-    _close(whole[0].astype(np.float64), ra)
-    _close(whole[1].astype(np.float64), rp)
+
+
+@pytest.mark.parametrize("every", [7, 50])
+@pytest.mark.parametrize("ground", [False, True], ids=["floating", "on-ground"])
+def test_checkpointed_gradient_matches_the_oracle(ground, every):
+    sy, steps = _robot(ground=ground, all_actuated=not ground), 200
+    rng = np.random.default_rng(0)
+    seed = oracle.centroid_x_seed(sy.n_masses) if ground else rng.standard_normal((sy.n_masses, 3))
+    ga, gp = _run(sy, every, 0, seed, steps)[:2]
+    ra, rp, _, _ = oracle.adjoint(sy, steps, seed)
+    _close(ga.astype(np.float64), ra)
+    _close(gp.astype(np.float64), rp)
 
 
 def test_a_limit_below_the_trajectory_bounds_the_memory():
