@@ -29,10 +29,18 @@ void component_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<u
 // mass now at d had before.  A SELL slice is as wide as its longest row, so
 // slices of similar rows hold less padding; a block keeps its masses, hence
 // its table.  build_sell takes the rank to leave every row's order as it was.
-// Per step: mesh of 500,000 points 18.5 -> 17.0 us, 100 worms 4.9 -> 4.3 (of a graph of
-// 20), 400 worms 17.9 -> 15.6, 256 and 512 robots in one system 13.3 -> 12.1, 22.9 -> 18.9.
+// Per step: mesh of 500,000 points 18.5 -> 17.0 us, of 2,000,000 80.5 -> 72.4, 100 worms
+// 4.9 -> 4.3 (of a graph of 20), 400 worms 17.9 -> 15.6, 256 and 512 robots in one system
+// 13.3 -> 12.1, 22.9 -> 18.9.
 void degree_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<uint32_t> &caller_of_dev,
                   std::vector<uint32_t> &rank);
+// Not for the atomic scatter, which has no rows (meshes 1 to 4 % slower), nor for the
+// staged stream (kernel_variant 2), whose gathers it spreads: meshes of 100,000 to
+// 300,000 points 25 % slower, of 2,000,000 146 -> 155 us.  The other kernels gain (2,000,000
+// points: 95 -> 86 us direct, 87 -> 81 prefetched, 81 -> 72 from tables).
+constexpr bool degree_order_helps(int accumulate, int kernel_variant) {
+    return accumulate == TITAN_ACCUM_CSR && kernel_variant != 2;
+}
 
 // Grid-tile order for masses that sit on a cubic grid of pitch h (every
 // coordinate within 1e-3 h of lo + integer x h, at most one mass per cell):

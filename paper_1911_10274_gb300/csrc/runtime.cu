@@ -746,7 +746,8 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
             cells.clear();
             titan::morton_order(m->pos, n, sim->caller_of_dev);
             titan::component_order(n, s, sp->ends, sim->caller_of_dev);
-            titan::degree_order(n, s, sp->ends, sim->caller_of_dev, rank);
+            if (titan::degree_order_helps(p->accumulate, p->kernel_variant))
+                titan::degree_order(n, s, sp->ends, sim->caller_of_dev, rank);
         }
     } else {
         sim->caller_of_dev.resize(n);
