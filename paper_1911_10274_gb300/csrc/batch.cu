@@ -245,9 +245,12 @@ k_batch_rollout(const BatchCta *__restrict__ ctas, const MassState *__restrict__
 // Measured, 64 voxel robots x 1000 steps 3.47 -> 1.99 ms, 1,024 robots of 27 to
 // 1,728 masses x 200 steps 6.16 -> 4.98 ms (both with reset and centroids).  Entries
 // side by side, 4, 7, 8, 9, 10 and 13: robots 5.16, 4.93, 4.98, 4.84, 4.87 and 4.85 ms,
-// voxel robots 2.02, 2.11, 1.99, 2.07, 2.12 and 2.12.
+// voxel robots 2.02, 2.11, 1.99, 2.07, 2.12 and 2.12 (eight: no other was as fast on both).
+// Unactuated, 1,024 robots of 27 to 1,728 masses x 200 steps: looped 4.56 ms, planned
+// for 384 threads an SM 4.50, for the 512 that its registers allow 3.72; of 27 to 216
+// masses 1.03, 1.08 and 0.93.
 template <bool ACT, bool GROUND>
-__global__ void __launch_bounds__(titan::kRowSlots)
+__global__ void __launch_bounds__(titan::row_slots(ACT))
 k_batch_rows(const BatchCta *__restrict__ ctas, const MassState *__restrict__ state_in,
              MassState *__restrict__ state_out, const uint32_t *__restrict__ slice_rel,
              const float2 *__restrict__ kl, const float4 *__restrict__ kla, const uint16_t *__restrict__ nbr,

@@ -860,7 +860,7 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
         uint32_t C = 0;
         if (plan.rows && *std::max_element(deg.begin(), deg.end()) <= kRowWidth)
             for (uint32_t c : {1u, 2u, 3u, 4u, 5u, 6u, 8u})
-                if (smem_on(c, kRowSlots) <= kBatchSmemLimit) {
+                if (smem_on(c, row_slots(any_act)) <= kBatchSmemLimit) {
                     C = c;
                     rows_of[r] = 1;
                     break;
@@ -989,7 +989,7 @@ bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_spr
         if (rows_of[r]) {           // by the CTAs whose threads an SM's registers hold
             uint32_t cls = 0;
             for (uint32_t k = 0; k < sizeof(kPerSm) / sizeof(kPerSm[0]); ++k)
-                if (per_sys[r][0].d.slot_count * kPerSm[k] <= kRowSlots) cls = k;
+                if (per_sys[r][0].d.slot_count * kPerSm[k] <= row_slots(any_act)) cls = k;
             return cls;
         }
         size_t worst = 0;

@@ -235,9 +235,10 @@ bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const s
 // A thread keeps a mass's whole row in its registers when no row is wider than
 // kRowWidth (the neighbours of a lattice site).  4.5 registers per actuated
 // entry x 26 and the arithmetic need 168 registers a thread, so an SM holds 384
-// threads of that form (kRowSlots); without actuation 128, and 512.
+// threads of that form (kRowSlots); without actuation 128, and 512 (row_slots).
 constexpr uint32_t kRowWidth = 26;
 constexpr uint32_t kRowSlots = 384;
+constexpr uint32_t row_slots(bool actuated) { return actuated ? kRowSlots : 512; }
 constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
 
 // The halo lists of a cluster the other way round: where each mass is copied
@@ -323,7 +324,7 @@ struct BatchGroup {
 };
 
 // The systems of a batch that qualify for the row-register form: rows at most
-// kRowWidth wide, masses on at most 8 CTAs of kRowSlots.
+// kRowWidth wide, masses on at most 8 CTAs of row_slots.
 struct BatchPlan {
     bool rows = false;                   // plan them for it
 };
@@ -354,7 +355,7 @@ struct BatchHost {
 // null: system r is not actuated).  False, with the reason in *why, if a
 // system fits no cluster of kBatchMaxCluster CTAs.  With plan.rows, systems that
 // qualify for the row-register form get the smallest cluster of 1, 2, 3, 4,
-// 5, 6 or 8 CTAs of at most kRowSlots masses and launch groups of their own, split
+// 5, 6 or 8 CTAs of at most row_slots masses and launch groups of their own, split
 // by how many of their CTAs an SM's registers hold.
 bool build_batch(uint32_t n_systems, const titan_masses *masses, const titan_springs *springs,
                  const titan_actuation *act, BatchHost &out, std::string *why, const BatchPlan &plan = BatchPlan());

@@ -153,7 +153,7 @@ k_step_persist(const MassState *__restrict__ in, MassState *__restrict__ out, ui
 constexpr int kRowGroup = 6;
 
 template <bool HAS_ACT, bool GROUND>
-__global__ void __launch_bounds__(HAS_ACT ? 384 : 512)
+__global__ void __launch_bounds__(row_slots(HAS_ACT))
 k_step_persist_rows(const MassState *__restrict__ in, MassState *__restrict__ out, uint32_t n, PersistArgs pa,
                     const uint32_t *__restrict__ slice_off, const uint16_t *__restrict__ slot,
                     const uint32_t *__restrict__ halo, const uint2 *__restrict__ push,
@@ -294,7 +294,7 @@ k_step_persist_rows(const MassState *__restrict__ in, MassState *__restrict__ ou
 // would not fit the registers), a thread per mass within the form's block
 // size, and rows of at most kRowWidth entries.
 bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, bool has_c, bool has_act) {
-    if (has_c || plan.per_cta > (has_act ? kRowSlots : 512u)) return false;
+    if (has_c || plan.per_cta > row_slots(has_act)) return false;
     for (size_t s = 0; s + 1 < slice_off.size(); ++s)
         if (slice_off[s + 1] - slice_off[s] > 32 * kRowWidth) return false;
     return true;

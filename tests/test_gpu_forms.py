@@ -30,7 +30,8 @@ def _ring(n):
 @pytest.mark.parametrize("name", list(CASES))
 def test_batches_of_short_rows_start_in_the_row_form(name, act):
     with T.Batch(CASES[name](act)) as b:
-        assert b.groups() and all(g["form"] == T.FORM_ROWS and g["launch_threads"] <= 384 for g in b.groups())
+        most = 384 if act else 512
+        assert b.groups() and all(g["form"] == T.FORM_ROWS and g["launch_threads"] <= most for g in b.groups())
         for g in range(len(b.groups())):
             b.configure(g, 512, 1)
         assert all(g["form"] == T.FORM_PLAIN and g["launch_threads"] == 512 for g in b.groups())
