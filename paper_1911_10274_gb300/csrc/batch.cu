@@ -470,9 +470,12 @@ struct titan_batch {
     std::vector<void *> allocs;
     std::string error;
     std::atomic<bool> busy{false};
-    cudaGraphExec_t graph = nullptr;
-    uint64_t graph_steps = 0;
-    int graph_cur = -1;
+    // per state buffer that a rollout starts from: the graph of a rollout of `steps` steps
+    // (with actuation: from step 0), captured when that count comes a second time
+    struct {
+        cudaGraphExec_t exec = nullptr;
+        uint64_t steps = 0;
+    } graphs[2];
 };
 
 namespace {
@@ -511,8 +514,16 @@ cudaError_t balloc(titan_batch *b, T **p, size_t count) {
     return cudaSuccess;
 }
 
+void drop_graphs(titan_batch *b) {
+    for (auto &g : b->graphs) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
+        g.steps = 0;
+    }
+}
+
 void release(titan_batch *b) {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    drop_graphs(b);
     for (void *p : b->allocs) cudaFree(p);
     for (auto s : b->group_streams) cudaStreamDestroy(s);
     for (auto e : b->group_events) cudaEventDestroy(e);
@@ -749,29 +760,33 @@ titan_status titan_batch_rollout(titan_batch *b, uint64_t n_steps) {
     int prev = -1;
     cudaGetDevice(&prev);
     BATCH_CK(b, cudaSetDevice(b->device));
-    // one captured graph per (step count, parity): the fork/join of all groups
-    if (!b->graph || b->graph_steps != n_steps || b->graph_cur != b->cur) {
-        if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
+    // Every rollout swaps the state buffers, so each buffer keeps a graph of its own: with one
+    // for both, every rollout captured it again (10 us a launch group).
+    auto &gr = b->graphs[b->cur];
+    const bool from_zero = !b->has_act || b->steps == 0;      // where a graph's actuation clock starts
+    if (from_zero && gr.steps == n_steps && !gr.exec) {
         cudaStream_t cap;
         BATCH_CK(b, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         cudaError_t le = e == cudaSuccess ? enqueue_rollout(b, cap, 0, (uint32_t)n_steps) : e;
-        cudaGraph_t gr = nullptr;
-        e = cudaStreamEndCapture(cap, &gr);
+        cudaGraph_t graph = nullptr;
+        e = cudaStreamEndCapture(cap, &graph);
         cudaStreamDestroy(cap);
-        if (le != cudaSuccess) { if (gr) cudaGraphDestroy(gr); return bfail_cuda(b, le, "capture rollout"); }
+        if (le != cudaSuccess) { if (graph) cudaGraphDestroy(graph); return bfail_cuda(b, le, "capture rollout"); }
         if (e != cudaSuccess) return bfail_cuda(b, e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&b->graph, gr, 0);
-        cudaGraphDestroy(gr);
+        e = cudaGraphInstantiate(&gr.exec, graph, 0);
+        cudaGraphDestroy(graph);
         if (e != cudaSuccess) return bfail_cuda(b, e, "cudaGraphInstantiate");
-        b->graph_steps = n_steps;
-        b->graph_cur = b->cur;
     }
-    if (b->has_act && b->steps != 0) {
-        // the captured graph starts its actuation clock at step 0: later rollouts launch directly
-        BATCH_CK(b, enqueue_rollout(b, b->stream, (long long)b->steps, (uint32_t)n_steps));
+    if (from_zero && gr.steps == n_steps) {
+        BATCH_CK(b, cudaGraphLaunch(gr.exec, b->stream));
     } else {
-        BATCH_CK(b, cudaGraphLaunch(b->graph, b->stream));
+        BATCH_CK(b, enqueue_rollout(b, b->stream, (long long)b->steps, (uint32_t)n_steps));
+        if (from_zero) {
+            if (gr.exec) cudaGraphExecDestroy(gr.exec);
+            gr.exec = nullptr;
+            gr.steps = n_steps;
+        }
     }
     b->cur ^= 1;
     b->steps += n_steps;
@@ -873,7 +888,7 @@ titan_status titan_batch_autotune(titan_batch *b, uint32_t probe_steps) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
+    drop_graphs(b);
     // the probes wrote into the other state buffer only; the current state is unchanged
     return TITAN_OK;
 }
@@ -903,7 +918,7 @@ titan_status titan_batch_configure(titan_batch *b, uint32_t group, uint32_t thre
     b->groups[group].rows = false;
     b->groups[group].threads = threads;
     b->groups[group].tpm = threads_per_mass;
-    if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
+    drop_graphs(b);
     return TITAN_OK;
 }
 
