@@ -410,14 +410,15 @@ k_batch_rows(const BatchCta *__restrict__ ctas, const MassState *__restrict__ st
     }
 }
 
-// Per-robot centroid x, y, z.  A block per robot; see group_mean.
+// Per-robot centroid x, y, z; see group_means.
+template <int LANES>
 __global__ void __launch_bounds__(titan::kMeanThreads)
-k_batch_centroid(const uint32_t *__restrict__ mass_off, const uint32_t *__restrict__ mass_cnt,
+k_batch_centroid(const uint32_t *__restrict__ mass_off, const uint32_t *__restrict__ mass_cnt, uint32_t n_robots,
                  const MassState *__restrict__ state, float *__restrict__ out) {
-    const uint32_t r = blockIdx.x, o = mass_off[r];
-    double m[3];
-    titan::group_mean(mass_cnt[r], [&](uint32_t i) { return state[o + i].p; }, m);
-    if (threadIdx.x < 3) out[3 * (size_t)r + threadIdx.x] = (float)m[threadIdx.x];
+    titan::group_means<LANES>(
+        n_robots, [&](uint32_t r) { return mass_cnt[r]; },
+        [&](uint32_t r, uint32_t i) { return state[mass_off[r] + i].p; },
+        [&](uint32_t r, uint32_t axis, double m) { out[3 * (size_t)r + axis] = (float)m; });
 }
 
 struct Group {
@@ -837,8 +838,14 @@ titan_status titan_batch_read(titan_batch *b, uint32_t system, float *pos, float
 titan_status titan_batch_centroids(titan_batch *b, float *out) {
     if (!b || !out) return bfail(b, TITAN_E_INVALID, "batch or out is null");
     if (!b->n_robots) return TITAN_OK;
-    k_batch_centroid<<<b->n_robots, titan::kMeanThreads, 0, b->stream>>>(b->d_moff, b->d_mcnt, b->d_state[b->cur],
-                                                                          b->d_centroid);
+    uint64_t masses = 0;
+    for (uint32_t c : b->mass_cnt) masses += c;
+    const uint32_t lanes = titan::mean_lanes(masses, b->n_robots);
+    const auto kern = lanes == 1                 ? k_batch_centroid<1>
+                      : lanes == titan::kMeanFew ? k_batch_centroid<titan::kMeanFew>
+                                                 : k_batch_centroid<titan::kMeanThreads>;
+    kern<<<titan::mean_blocks(masses, b->n_robots), titan::kMeanThreads, 0, b->stream>>>(
+        b->d_moff, b->d_mcnt, b->n_robots, b->d_state[b->cur], b->d_centroid);
     BATCH_CK(b, cudaGetLastError());
     titan_status st = titan_batch_sync(b);
     if (st != TITAN_OK) return st;

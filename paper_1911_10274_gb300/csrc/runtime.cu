@@ -286,18 +286,20 @@ bool uses_cube(const titan_sim *sim) { return sim->csr_kernel == 8; }
 // Uploads the per-entry actuation arrays of the current layout.
 // Mean position of each group of masses (caller indices first[g] ..
 // first[g+1] - 1, clamped to n), minus the group's origin if given (an empty
-// group: 0).  A block per group; see group_mean.
+// group: 0); see group_means.
+template <int LANES>
 __global__ void __launch_bounds__(titan::kMeanThreads)
 k_group_centroid(const MassState *__restrict__ state, const uint32_t *__restrict__ dev_of_caller, uint32_t n,
-                 const uint32_t *__restrict__ first, const float *__restrict__ origin, float *__restrict__ out) {
-    const uint32_t g = blockIdx.x;
-    const uint32_t i0 = min(first[g], n), i1 = max(i0, min(first[g + 1], n));
-    double m[3];
-    titan::group_mean(i1 - i0, [&](uint32_t i) { return state[dev_of_caller[i0 + i]].p; }, m);
-    if (threadIdx.x < 3) {
-        const float o = origin && i1 > i0 ? origin[3 * (size_t)g + threadIdx.x] : 0.f;
-        out[3 * (size_t)g + threadIdx.x] = (float)(m[threadIdx.x] - (double)o);
-    }
+                 const uint32_t *__restrict__ first, uint32_t n_groups, const float *__restrict__ origin,
+                 float *__restrict__ out) {
+    auto begin = [&](uint32_t g) { return min(first[g], n); };
+    auto count = [&](uint32_t g) { return max(begin(g), min(first[g + 1], n)) - begin(g); };
+    titan::group_means<LANES>(
+        n_groups, count, [&](uint32_t g, uint32_t i) { return state[dev_of_caller[begin(g) + i]].p; },
+        [&](uint32_t g, uint32_t axis, double m) {
+            const float o = origin && count(g) ? origin[3 * (size_t)g + axis] : 0.f;
+            out[3 * (size_t)g + axis] = (float)(m - (double)o);
+        });
 }
 
 // seed[i][axis] = w[g] / |group g| for the masses of group g; a warp per group.
@@ -1239,8 +1241,12 @@ titan_status titan_group_centroids(titan_sim *sim, uint32_t n_groups, const uint
         titan_status es_ = titan::ensure_layout(sim);
         if (es_ != TITAN_OK) return es_;
     }
-    k_group_centroid<<<n_groups, titan::kMeanThreads, 0, sim->stream>>>(sim->state[sim->cur], sim->d_dev_of_caller,
-                                                                         sim->n, first_dev, origin_dev, out_dev);
+    const uint32_t lanes = titan::mean_lanes(sim->n, n_groups);
+    const auto kern = lanes == 1                 ? k_group_centroid<1>
+                      : lanes == titan::kMeanFew ? k_group_centroid<titan::kMeanFew>
+                                                 : k_group_centroid<titan::kMeanThreads>;
+    kern<<<titan::mean_blocks(sim->n, n_groups), titan::kMeanThreads, 0, sim->stream>>>(
+        sim->state[sim->cur], sim->d_dev_of_caller, sim->n, first_dev, n_groups, origin_dev, out_dev);
     TITAN_CK(sim, cudaGetLastError());
     return TITAN_OK;
 }
