@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "gemm_ring.h"
+#include "gemm_rule.h"
 #include "mlp_layout.h"
 #include "ptx.cuh"
 #include "titan.h"
@@ -1021,13 +1022,12 @@ cudaError_t gemm_tn(const void *A, const void *B, int M, int N, int K, const Epi
     const bool narrow = !wide && tiles128 <= 152;
     CUtensorMap ma, mb;
     if (!make_map(&ma, A, M, K)) return cudaErrorInvalidValue;
-    // CTA pairs once every pair of SMs has a tile of its own; the epilogue
-    // writes whole 32-byte sectors
+    // the pairs' epilogue writes whole 32-byte sectors
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!BMN && ep.mode == EPI_F32 && M % kPairTile == 0 && N % kPairTile == 0 &&
-        (int64_t)(M / kPairTile) * (N / kPairTile) >= sms / 2 && !(reinterpret_cast<uintptr_t>(ep.out_f32) & 31)) {
+    if (!BMN && ep.mode == EPI_F32 && titan::gemm_takes_pairs(M, N, K, sms) &&
+        !(reinterpret_cast<uintptr_t>(ep.out_f32) & 31)) {
         if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
         return gemm_pair_launch(ma, mb, M, N, K, ep, st, spin_limit, err, sms);
     }
