@@ -22,4 +22,16 @@ constexpr bool gemm_takes_pairs(int64_t M, int64_t N, int64_t K, int sms) {
             (K >= 8192 && tiles >= pairs));
 }
 
+// Tile width of the one-CTA kernel (128 rows): 64 columns when 128-wide tiles would not
+// fill one wave of 152 SMs; 256 once there are at least two waves of such tiles - but with a
+// GELU in the epilogue (gelu), which two CTAs of 128-wide tiles an SM hide better, only from
+// K = 4096 on.  128 -> 256 wide, us: forward pass of a hidden layer of 512 at a batch of 32,768
+// 161 -> 177, of 2,048 at 16,384 378 -> 384, of 4,096 at 16,384 1,073 -> 1,008, of 8,192 at 4,096
+// 995 -> 915.
+constexpr int gemm_tile_width(int64_t M, int64_t N, int64_t K, bool gelu) {
+    return N % 256 == 0 && (N / 256) * (M / 128) >= 2 * 152 && (!gelu || K >= 4096) ? 256
+           : (N / 128) * (M / 128) <= 152                                            ? 64
+                                                                                     : 128;
+}
+
 }  // namespace titan

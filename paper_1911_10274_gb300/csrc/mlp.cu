@@ -1013,13 +1013,7 @@ cudaError_t gemm_tn(const void *A, const void *B, int M, int N, int K, const Epi
                     uint32_t spin_limit, int *err) {
     if (M % BM || N % BN || K % BK || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return cudaErrorInvalidValue;
-    // 64-wide tiles when 128-wide ones would not fill one wave of 152 SMs; 256-wide
-    // ones for plain products once there are at least two waves of them (with a GELU in
-    // the epilogue, 128-wide tiles at two CTAs per SM hide it: hidden layer of 512 at a
-    // batch of 32,768, K = 512: 57 -> 46 us)
-    const int64_t tiles128 = (int64_t)(N / 128) * (M / BM);
-    const bool wide = ep.mode == EPI_F32 && N % 256 == 0 && (int64_t)(N / 256) * (M / BM) >= 2 * 152;
-    const bool narrow = !wide && tiles128 <= 152;
+    const int width = titan::gemm_tile_width(M, N, K, ep.mode != EPI_F32);
     CUtensorMap ma, mb;
     if (!make_map(&ma, A, M, K)) return cudaErrorInvalidValue;
     // the pairs' epilogue writes whole 32-byte sectors
@@ -1031,10 +1025,10 @@ cudaError_t gemm_tn(const void *A, const void *B, int M, int N, int K, const Epi
         if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
         return gemm_pair_launch(ma, mb, M, N, K, ep, st, spin_limit, err, sms);
     }
-    if (!(BMN ? make_map(&mb, B, K, N, 64) : make_map(&mb, B, N, K, wide ? 256 : (narrow ? 64 : 128))))
+    if (!(BMN ? make_map(&mb, B, K, N, 64) : make_map(&mb, B, N, K, (uint32_t)width)))
         return cudaErrorInvalidValue;
-    if (wide) return gemm_tn_launch<256, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
-    if (narrow) return gemm_tn_launch<64, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
+    if (width == 256) return gemm_tn_launch<256, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
+    if (width == 64) return gemm_tn_launch<64, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
     return gemm_tn_launch<128, BMN>(ma, mb, M, N, K, ep, st, spin_limit, err);
 }
 
