@@ -517,7 +517,8 @@ cudaError_t resolve_exec(titan_sim *sim) {
     if ((e = upload(sim->d_pslot, slot, sim->stream)) != cudaSuccess) return e;
     if ((e = upload(sim->d_phalo, halo, sim->stream)) != cudaSuccess) return e;
     std::vector<uint32_t> push, more;
-    sim->persist_rows = titan::persist_rows_fit(plan, sim->sell.slice_off, sim->has_c, sim->has_act);
+    sim->persist_rows = titan::persist_rows_fit(plan, sim->sell.slice_off, sim->n, sim->has_c, sim->has_act,
+                                                sim->c.act_mode != 2);
     if (sim->persist_rows) {
         std::vector<std::pair<const uint32_t *, uint32_t>> lists;
         for (uint32_t r = 0; r < plan.cluster; ++r)

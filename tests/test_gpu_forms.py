@@ -51,14 +51,16 @@ def test_the_autotuner_reports_the_form_it_keeps():
 
 
 @pytest.mark.parametrize("sy,act,per_spring,form", [
-    (lambda: SYSTEMS["row_26"](), True, False, T.FORM_ROWS), (lambda: SYSTEMS["row_28"](), True, False, T.FORM_PLAIN),
+    (lambda: SYSTEMS["row_26"](), False, False, T.FORM_ROWS), (lambda: SYSTEMS["row_28"](), False, False, T.FORM_PLAIN),
     (lambda: _star(27, 9), False, False, T.FORM_PLAIN), (lambda: SYSTEMS["cube"](), False, False, T.FORM_ROWS),
     (lambda: SYSTEMS["cube"](), False, True, T.FORM_PLAIN),
-    # masses a CTA: 384 with actuation, 512 without
+    # with the sinusoid from 160 masses on; masses a CTA: 384 with actuation, 512 without
+    (lambda: _ring(159), True, False, T.FORM_PLAIN), (lambda: _ring(160), True, False, T.FORM_ROWS),
+    (lambda: _ring(159), False, False, T.FORM_ROWS),
     (lambda: _ring(384), True, False, T.FORM_ROWS), (lambda: _ring(385), True, False, T.FORM_PLAIN),
     (lambda: _ring(512), False, False, T.FORM_ROWS), (lambda: _ring(4096), False, False, T.FORM_ROWS),
     (lambda: _ring(4097), False, False, T.FORM_PLAIN)],
-    ids=["row_26", "row_28", "row_27", "cube", "per_spring", "384", "385", "512", "4096", "4097"])
+    ids=["row_26", "row_28", "row_27", "cube", "per_spring", "159", "160", "159_plain", "384", "385", "512", "4096", "4097"])
 def test_persistent_form(sy, act, per_spring, form):
     sy = sy()
     if not act:
@@ -70,6 +72,21 @@ def test_persistent_form(sy, act, per_spring, form):
         sim.step(3)
         x, _, _ = sim.snapshot()
     assert np.isfinite(x).all()
+
+
+def test_small_bodies_with_the_worm_take_rows():
+    sy = _ring(100)
+    amp, sy.act_amp = sy.act_amp, None
+    with T.Sim(sy, exec_mode=T.EXEC_PERSISTENT) as sim, T.Sim(sy, exec_mode=T.EXEC_LAUNCH, kernel_variant=1) as ref:
+        for s in (sim, ref):
+            T.titan_set_worm_actuation(s.handle, np.arange(sy.n_springs), amp, np.linspace(0.0, 0.9, sy.n_springs), 20.0, 0.01)
+            s.step(9)
+        assert sim.step_form == T.FORM_ROWS
+        for s in (sim, ref):                          # and give them up for the sinusoid
+            T.titan_set_actuation(s.handle, np.arange(sy.n_springs), amp, np.linspace(0, 6, sy.n_springs), 2.0)
+            s.step(9)
+        x, y = sim.snapshot(), ref.snapshot()
+        assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
 
 
 def test_actuation_set_later_changes_the_form_with_the_entries():
