@@ -713,7 +713,7 @@ void invert_halos(const std::vector<std::pair<const uint32_t *, uint32_t>> &halo
 
 bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const std::vector<uint32_t> &nbr,
                      bool has_c, bool has_act, size_t smem_limit, PersistPlan &plan,
-                     std::vector<uint16_t> &slot, std::vector<uint32_t> &halo) {
+                     std::vector<uint16_t> &slot, std::vector<uint32_t> &halo, uint32_t aim) {
     if (n == 0 || slice_off.size() != (size_t)(n + 31) / 32 + 1 || nbr.size() != slice_off.back()) return false;
     // per cluster size: masses per CTA, each CTA's entries and halo (the
     // distinct masses of other CTAs its rows touch, in first-use order)
@@ -762,13 +762,13 @@ bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const s
         t.bytes = persistent_smem_bytes(t.per, t.max_h, t.max_e, has_c, has_act);
         return t.bytes <= smem_limit;
     };
-    // the smallest cluster that fits and gives each thread one mass (512 per
-    // CTA); failing that, the smallest that fits at all
+    // the smallest cluster that fits with at most `aim` masses per CTA; failing that,
+    // with a thread per mass (512); failing that, the smallest that fits at all
     Try t;
     uint32_t cl = 0;
-    for (int pass = 0; pass < 2 && !cl; ++pass)
+    for (uint32_t most : {aim, 512u, UINT32_MAX})
         for (uint32_t c2 = 1; c2 <= 8 && !cl; c2 *= 2) {
-            if (pass == 0 && (((n + c2 - 1) / c2 + 31) & ~31u) > 512) continue;
+            if ((((n + c2 - 1) / c2 + 31) & ~31u) > most) continue;
             t = Try();
             if (build(c2, t)) cl = c2;
         }

@@ -221,14 +221,14 @@ struct PersistPlan {
 
 size_t persistent_smem_bytes(uint32_t per_cta, uint32_t max_halo, uint32_t max_entries, bool has_c, bool has_act);
 
-// Picks the smallest cluster whose CTAs fit smem_limit (preferring one mass
-// per thread, 512 per CTA) and writes, per SELL entry, the neighbour's slot in
+// Picks the smallest cluster whose CTAs fit smem_limit (preferring at most `aim`
+// masses per CTA, then one mass per thread, 512) and writes, per SELL entry, the neighbour's slot in
 // its CTA's local table (own masses first, then the halo), and the halo list
 // (rank << 16 | local slot in the owning CTA).  False if the system does not
 // fit one cluster of 8.
 bool plan_persistent(uint32_t n, const std::vector<uint32_t> &slice_off, const std::vector<uint32_t> &nbr,
                      bool has_c, bool has_act, size_t smem_limit, PersistPlan &plan,
-                     std::vector<uint16_t> &slot, std::vector<uint32_t> &halo);
+                     std::vector<uint16_t> &slot, std::vector<uint32_t> &halo, uint32_t aim = 512);
 
 // ---- row-register forms (k_batch_rows, k_step_persist_rows)
 //
@@ -240,6 +240,20 @@ constexpr uint32_t kRowWidth = 26;
 constexpr uint32_t kRowSlots = 384;
 constexpr uint32_t row_slots(bool actuated) { return actuated ? kRowSlots : 512; }
 constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
+
+// Whether a persistent system should run in the row-register form: not with per-spring
+// damping (its array would not fit the registers), nor a small body with the sinusoid,
+// whose few warps each run the sine of 26 entries written out one after another and wait
+// for instructions (200 steps, looped -> rows: 27 masses 758 -> 818 us, 64 682 -> 734, 125
+// 709 -> 732, a mesh of 200 512 -> 535, 343 886 -> 765; with the worm or without actuation
+// rows gain).  Its CTAs are then planned for the masses that form can hold
+// (persist_aim): 441 actuated masses on one CTA of the looped form 979 us, on two 799.
+constexpr bool persist_rows_wanted(uint32_t masses, bool has_c, bool has_act, bool sine) {
+    return !has_c && !(has_act && sine && masses < 256);
+}
+constexpr uint32_t persist_aim(uint32_t masses, bool has_c, bool has_act, bool sine) {
+    return persist_rows_wanted(masses, has_c, has_act, sine) ? row_slots(has_act) : 512;
+}
 
 // The halo lists of a cluster the other way round: where each mass is copied
 // to.  halo[q] lists CTA q's halo entries (owner rank << 16 | slot in the owner);

@@ -290,16 +290,10 @@ k_step_persist_rows(const MassState *__restrict__ in, MassState *__restrict__ ou
 
 }  // namespace
 
-// Whether a plan runs in the row-register form: no per-spring damping (its array
-// would not fit the registers), a thread per mass within the form's block
-// size, and rows of at most kRowWidth entries.  Small bodies with the sinusoid stay in
-// the looped form: their few warps each run the sine of 26 entries written out one after
-// another, and wait for instructions (200 steps, looped -> rows: 27 masses 758 -> 818 us, 64
-// 682 -> 734, 125 709 -> 732, 216 761 -> 715, 343 886 -> 765; with the worm or without
-// actuation rows gain at every size).
-bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, uint32_t masses, bool has_c,
-                      bool has_act, bool sine) {
-    if (has_c || plan.per_cta > row_slots(has_act) || (has_act && sine && masses < 160)) return false;
+// Whether a plan runs in the row-register form: wanted (persist_rows_wanted), a thread per
+// mass within the form's block size, and rows of at most kRowWidth entries.
+bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, bool wanted, bool has_act) {
+    if (!wanted || plan.per_cta > row_slots(has_act)) return false;
     for (size_t s = 0; s + 1 < slice_off.size(); ++s)
         if (slice_off[s + 1] - slice_off[s] > 32 * kRowWidth) return false;
     return true;

@@ -504,8 +504,10 @@ cudaError_t resolve_exec(titan_sim *sim) {
     titan::PersistPlan plan;
     std::vector<uint16_t> slot;
     std::vector<uint32_t> halo;
+    const bool sine = sim->c.act_mode != 2;
     if (!titan::plan_persistent(sim->n_dev, sim->sell.slice_off, sim->sell.nbr, sim->has_c, sim->has_act,
-                                kPersistSmemLimit, plan, slot, halo))
+                                kPersistSmemLimit, plan, slot, halo,
+                                titan::persist_aim(sim->n, sim->has_c, sim->has_act, sine)))
         return cudaSuccess;
     if (sim->exec_req == TITAN_EXEC_AUTO && plan.per_cta > kPersistAutoMaxPerCta) return cudaSuccess;
     cudaError_t e;
@@ -517,8 +519,9 @@ cudaError_t resolve_exec(titan_sim *sim) {
     if ((e = upload(sim->d_pslot, slot, sim->stream)) != cudaSuccess) return e;
     if ((e = upload(sim->d_phalo, halo, sim->stream)) != cudaSuccess) return e;
     std::vector<uint32_t> push, more;
-    sim->persist_rows = titan::persist_rows_fit(plan, sim->sell.slice_off, sim->n, sim->has_c, sim->has_act,
-                                                sim->c.act_mode != 2);
+    sim->persist_rows = titan::persist_rows_fit(plan, sim->sell.slice_off,
+                                                titan::persist_rows_wanted(sim->n, sim->has_c, sim->has_act, sine),
+                                                sim->has_act);
     if (sim->persist_rows) {
         std::vector<std::pair<const uint32_t *, uint32_t>> lists;
         for (uint32_t r = 0; r < plan.cluster; ++r)

@@ -194,8 +194,7 @@ bool step_is_deep(uint32_t n);
 // push, push_more: the copy lists of invert_halos, by device mass (null: the
 // looped form).
 struct PersistPlan;
-bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, uint32_t masses, bool has_c,
-                      bool has_act, bool sine);
+bool persist_rows_fit(const PersistPlan &plan, const std::vector<uint32_t> &slice_off, bool wanted, bool has_act);
 cudaError_t launch_step_persistent(const MassState *in, MassState *out, uint32_t n, const PersistPlan &plan,
                                    const uint32_t *slice_off, const uint16_t *slot, const uint32_t *halo,
                                    const uint2 *push, const uint32_t *push_more, const float2 *kl, const float *cc, const float2 *act, const StepConst &c,

@@ -54,13 +54,14 @@ def test_the_autotuner_reports_the_form_it_keeps():
     (lambda: SYSTEMS["row_26"](), False, False, T.FORM_ROWS), (lambda: SYSTEMS["row_28"](), False, False, T.FORM_PLAIN),
     (lambda: _star(27, 9), False, False, T.FORM_PLAIN), (lambda: SYSTEMS["cube"](), False, False, T.FORM_ROWS),
     (lambda: SYSTEMS["cube"](), False, True, T.FORM_PLAIN),
-    # with the sinusoid from 160 masses on; masses a CTA: 384 with actuation, 512 without
-    (lambda: _ring(159), True, False, T.FORM_PLAIN), (lambda: _ring(160), True, False, T.FORM_ROWS),
-    (lambda: _ring(159), False, False, T.FORM_ROWS),
-    (lambda: _ring(384), True, False, T.FORM_ROWS), (lambda: _ring(385), True, False, T.FORM_PLAIN),
+    # with the sinusoid from 256 masses on; masses a CTA of at most eight: 384 with actuation, 512 without
+    (lambda: _ring(255), True, False, T.FORM_PLAIN), (lambda: _ring(256), True, False, T.FORM_ROWS),
+    (lambda: _ring(255), False, False, T.FORM_ROWS),
+    (lambda: _ring(384), True, False, T.FORM_ROWS), (lambda: _ring(385), True, False, T.FORM_ROWS),
+    (lambda: _ring(3072), True, False, T.FORM_ROWS), (lambda: _ring(3073), True, False, T.FORM_PLAIN),
     (lambda: _ring(512), False, False, T.FORM_ROWS), (lambda: _ring(4096), False, False, T.FORM_ROWS),
     (lambda: _ring(4097), False, False, T.FORM_PLAIN)],
-    ids=["row_26", "row_28", "row_27", "cube", "per_spring", "159", "160", "159_plain", "384", "385", "512", "4096", "4097"])
+    ids=["row_26", "row_28", "row_27", "cube", "per_spring", "255", "256", "255_plain", "384", "385", "3072", "3073", "512", "4096", "4097"])
 def test_persistent_form(sy, act, per_spring, form):
     sy = sy()
     if not act:
@@ -90,7 +91,7 @@ def test_small_bodies_with_the_worm_take_rows():
 
 
 def test_actuation_set_later_changes_the_form_with_the_entries():
-    sy = _ring(512)
+    sy = _ring(3100)                                  # 388 masses a CTA of eight
     amp, phase, sy.act_amp = sy.act_amp, sy.act_phase, None
     with T.Sim(sy, exec_mode=T.EXEC_PERSISTENT) as sim, T.Sim(sy, exec_mode=T.EXEC_LAUNCH, kernel_variant=1) as ref:
         assert (sim.step_form, ref.step_form) == (T.FORM_ROWS, T.FORM_PLAIN)
