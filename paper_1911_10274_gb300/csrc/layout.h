@@ -37,9 +37,17 @@ void degree_order(uint32_t n, uint32_t s, const uint32_t *ends, std::vector<uint
 // Not for the atomic scatter, which has no rows (meshes 1 to 4 % slower), nor for the
 // staged stream (kernel_variant 2), whose gathers it spreads: meshes of 100,000 to
 // 300,000 points 25 % slower, of 2,000,000 146 -> 155 us.  The other kernels gain (2,000,000
-// points: 95 -> 86 us direct, 87 -> 81 prefetched, 81 -> 72 from tables).
-constexpr bool degree_order_helps(int accumulate, int kernel_variant) {
-    return accumulate == TITAN_ACCUM_CSR && kernel_variant != 2;
+// points: 95 -> 86 us direct, 87 -> 81 prefetched, 81 -> 72 from tables).  Nor for systems
+// with per-spring damping that may run in the looped form of the persistent kernel
+// (looped), whose CTAs then share their blocks unevenly: 200 steps of 11^3 masses off the
+// grid 794 -> 871 us (with actuation 1,048 -> 1,233), of 16^3 880 -> 965.
+constexpr bool degree_order_helps(int accumulate, int kernel_variant, bool looped) {
+    return accumulate == TITAN_ACCUM_CSR && kernel_variant != 2 && !looped;
+}
+// Whether a system of n masses may run in that form: if launches are not asked for, and up
+// to a thread per mass of the largest cluster.
+constexpr bool may_run_looped(uint32_t n, int exec, bool per_spring_damping) {
+    return per_spring_damping && exec != TITAN_EXEC_LAUNCH && n <= 8 * 512;
 }
 
 // Grid-tile order for masses that sit on a cubic grid of pitch h (every

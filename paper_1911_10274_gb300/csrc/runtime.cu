@@ -732,6 +732,9 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
 
     // ---- host-side layout
     const uint32_t n = m->n, s = sp->n;
+    bool uniform_c = true;                // one damping for all springs
+    if (sp->damping)
+        for (uint32_t q = 1; q < s; ++q) uniform_c = uniform_c && (float)sp->damping[q] == (float)sp->damping[0];
     std::vector<int32_t> cells;           // grid cell per device index (grid-tile order only)
     std::vector<uint32_t> rank;           // Morton position per device index (Morton order only)
     if (p->order == TITAN_ORDER_MORTON) {
@@ -752,7 +755,7 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
             cells.clear();
             titan::morton_order(m->pos, n, sim->caller_of_dev);
             titan::component_order(n, s, sp->ends, sim->caller_of_dev);
-            if (titan::degree_order_helps(p->accumulate, p->kernel_variant))
+            if (titan::degree_order_helps(p->accumulate, p->kernel_variant, titan::may_run_looped(n, p->exec, !uniform_c)))
                 titan::degree_order(n, s, sp->ends, sim->caller_of_dev, rank);
         }
     } else {
@@ -769,7 +772,6 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
     sim->k.resize(s);
     sim->rest.resize(s);
     sim->damp.resize(s);
-    bool uniform_c = true;
     for (uint32_t q = 0; q < s; ++q) {
         const uint32_t i = sp->ends[2 * (size_t)q], j = sp->ends[2 * (size_t)q + 1];
         sim->k[q] = (float)sp->k[q];
@@ -784,7 +786,6 @@ titan_status titan_create(const titan_masses *m, const titan_springs *sp, const 
         }
         sim->rest[q] = (float)L;
         sim->damp[q] = (float)(sp->damping ? sp->damping[q] : p->damping);
-        if (q && sim->damp[q] != sim->damp[0]) uniform_c = false;
     }
     sim->has_c = !uniform_c;
     if (uniform_c && s) sim->c.c_uniform = sim->damp[0];
