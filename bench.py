@@ -53,7 +53,7 @@ E2E_PASSES = 3
 # header and the build script with its flags).  Reported only while those are
 # unchanged.  Capture: profiles/k_step_box_lattice1m.md.
 NCU_TRAFFIC = {
-    ("lattice1m", "csr", "k_step_box", "544b3a1b8dc37538"): 251_609_856 + 12_306_432,
+    ("lattice1m", "csr", "k_step_box", "d37f9df17958fba5"): 251_609_344 + 12_481_280,
 }
 KERNEL_INPUTS = ("paper_1911_10274_gb300/csrc/step_kernels.cu", "paper_1911_10274_gb300/csrc/physics.cuh",
                  "paper_1911_10274_gb300/build.py")
@@ -386,7 +386,8 @@ def adjoint_leg(device, n_robots=4096, steps=200, every=50):
     return {"workload": f"{n_robots} robots ({f.system.n_springs} springs), {steps}-step rollout, "
                         f"checkpoint every {every}", "seconds": t,
             "gradient_entries": 2 * f.system.n_springs, "adjoint_steps_per_s": steps / t,
-            "note": "forward with checkpoints + per-segment recompute + two reverse kernels per step"}
+            "note": "forward (every state kept up to 1 GiB, else checkpoints and recomputed segments) + one reverse "
+                    "kernel per step"}
 
 
 def mlp_leg(device, batch=4096, n_in=1024, hidden=512, reps=20, big=True):
@@ -457,10 +458,10 @@ def mlp_leg(device, batch=4096, n_in=1024, hidden=512, reps=20, big=True):
             "gemm_8192_tflops": large_tflops, "gemm_8192_frac": large_tflops / peak[0],
             "roofline": {"bound": "tensor", "achieved": large_tflops, "peak": peak[0], "unit": "TFLOP/s",
                          "frac": large_tflops / peak[0], "peak_source": peak[1],
-                         "kernel": "k_gemm_tn", "shape": f"{L}x{L}x{L}",
+                         "kernel": "k_gemm_pair", "shape": f"{L}x{L}x{L}",
                          "note": "the kernel on a square product, 5 calls enqueued back to back and timed "
                                  "to the end of the last; at the MLP's own shapes (gemm_tflops) one call is a "
-                                 "256-CTA launch (128 x 64 tiles, two per SM) of 4.3 GFLOP"}}
+                                 "256-CTA launch of k_gemm_tn (128 x 64 tiles, two per SM) of 4.3 GFLOP"}}
 
 
 def bf16_peak():

@@ -255,7 +255,8 @@ constexpr uint32_t kNoPush = 0xffffffffu, kMorePush = 0x80000000u;
 // for instructions (200 steps, looped -> rows: 27 masses 758 -> 818 us, 64 682 -> 734, 125
 // 709 -> 732, a mesh of 200 512 -> 535, 343 886 -> 765; with the worm or without actuation
 // rows gain).  Its CTAs are then planned for the masses that form can hold
-// (persist_aim): 441 actuated masses on one CTA of the looped form 979 us, on two 799.
+// (persist_aim): 441 actuated masses on one CTA of the looped form 979 us, on two CTAs of
+// rows 879, 960 masses on two and four 1,111 and 814.
 constexpr bool persist_rows_wanted(uint32_t masses, bool has_c, bool has_act, bool sine) {
     return !has_c && !(has_act && sine && masses < 256);
 }
@@ -274,8 +275,9 @@ void invert_halos(const std::vector<std::pair<const uint32_t *, uint32_t>> &halo
 
 // ---- batches of independent systems (see batch.cu)
 //
-// Every system is owned by one thread-block cluster of C CTAs (C = 1, 2, 4 or
-// 8, the smallest whose CTAs fit kBatchSmemLimit).  CTA q of a system owns its
+// Every system is owned by one thread-block cluster of C CTAs, the smallest whose
+// CTAs fit kBatchSmemLimit (C = 1, 2, 4 or 8; in the row-register form also 3, 5
+// and 6, of at most row_slots masses).  CTA q of a system owns its
 // masses [q P, (q + 1) P) in caller order, P = ceil(n / C) rounded up to 32,
 // at global state slots mass_begin .. mass_begin + P (slots past the system's
 // last mass are padding: fixed, at rest).  The CTA's rows are SELL-32 over its

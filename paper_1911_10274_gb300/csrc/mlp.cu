@@ -12,7 +12,7 @@
 // dimension, which is how back-propagation multiplies by transposes).  One CTA
 // per 128 x BN output tile (BN = 64, 128 or 256), 512 threads:
 //   warp 0         - TMA producer: 2-D tiled loads (128-byte swizzle) of the
-//                    A and B K-blocks (64 wide) into a 4-stage ring;
+//                    A and B K-blocks (64 wide) into a ring of 3 or 4 stages;
 //   warp 1         - MMA issuer: tcgen05.mma.kind::f16 (M = 128, N = BN,
 //                    K = 16) into an FP32 accumulator in TMEM, releasing each
 //                    stage with tcgen05.commit;
@@ -28,7 +28,8 @@
 // the one before: a copy of the batch, three forward products, the head (output
 // layer, loss, first step back), two input gradients, the three weight gradients,
 // and Adam (which adds the K slices and column sums up itself).  The learning rate
-// and the Adam step counter live in device memory.
+// and the Adam step counter live in device memory.  Large products of a caller's own
+// (titan_gemm_bf16_tn) go to persistent CTA pairs, k_gemm_pair, where gemm_rule.h says.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>

@@ -3,20 +3,23 @@
 // For a system whose state and SELL rows fit in the shared memory of one
 // thread-block cluster (up to 8 CTAs), launching one kernel per step leaves
 // the GPU idle for most of each step (a step is a few hundred nanoseconds of
-// work against microseconds of launch and drain).  This kernel instead loads
-// the system once and runs a whole chunk of steps: CTA r of the cluster owns
-// device masses [r P, (r + 1) P); at launch it copies their state and SELL rows
-// (the simulation's own arrays, so parameter edits between launches are seen)
-// into shared memory, then for every step first copies the current state of
-// its halo - the masses of other CTAs its rows touch - out of their shared
-// memory (distributed shared memory, one coalesced pass) into a local halo
-// region, and evaluates each owned mass's row from local shared memory only,
-// exactly as the launch kernels do (same entries, same order, same helpers:
-// Sec. III-B, Eq. 1; Sec. III-A constraints; Eqs. 3-5 actuation); it writes
-// the new state into the other shared buffer and meets one hardware cluster
-// barrier.  The final state goes back to
-// global memory.  No spin-wait of its own: the cluster barrier is hardware and
-// all CTAs of a cluster are co-resident by construction.
+// work against microseconds of launch and drain).  These kernels instead load
+// the system once and run a whole chunk of steps: CTA r of the cluster owns
+// device masses [r P, (r + 1) P), whose state and SELL rows it reads at launch
+// (the simulation's own arrays, so parameter edits between launches are seen),
+// and evaluates each owned mass's row from local shared memory only, exactly as
+// the launch kernels do (same entries, same order, same helpers: Sec. III-B, Eq.
+// 1; Sec. III-A constraints; Eqs. 3-5 actuation); it writes the new state into
+// the other shared buffer and meets one hardware cluster barrier per step.
+//   k_step_persist_rows - a thread per mass, its row and state in registers; each
+//                         new state is written straight into the halo slots of the
+//                         CTAs that read it (persist_rows_fit says when);
+//   k_step_persist      - rows in shared memory; each step first copies the current
+//                         state of its halo - the masses of other CTAs its rows touch -
+//                         out of their shared memory (distributed shared memory, one
+//                         coalesced pass).
+// The final state goes back to global memory.  No spin-wait of their own: the cluster
+// barrier is hardware and all CTAs of a cluster are co-resident by construction.
 #include <cooperative_groups.h>
 
 #include <algorithm>
