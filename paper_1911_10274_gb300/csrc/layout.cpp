@@ -693,20 +693,27 @@ size_t persistent_smem_bytes(uint32_t per_cta, uint32_t max_halo, uint32_t max_e
 
 void invert_halos(const std::vector<std::pair<const uint32_t *, uint32_t>> &halo, uint32_t per, uint32_t *push,
                   std::vector<uint32_t> &more) {
-    std::vector<std::vector<uint32_t>> to(halo.size() * per);
+    // the copies of each mass side by side: [at[k], at[k + 1]) of to, in the order of the lists
+    const size_t n = halo.size() * per;
+    std::vector<uint32_t> at(n + 1, 0), to;
+    auto slot = [&](uint32_t code) { return (size_t)(code >> 16) * per + (code & 0xffffu); };
+    for (const auto &list : halo)
+        for (uint32_t h = 0; h < list.second; ++h) ++at[slot(list.first[h]) + 1];
+    for (size_t k = 0; k < n; ++k) at[k + 1] += at[k];
+    to.resize(at[n]);
     for (uint32_t q = 0; q < (uint32_t)halo.size(); ++q)
-        for (uint32_t h = 0; h < halo[q].second; ++h) {
-            const uint32_t code = halo[q].first[h];
-            to[(size_t)(code >> 16) * per + (code & 0xffffu)].push_back(q << 16 | h);
-        }
-    for (size_t k = 0; k < to.size(); ++k) {
+        for (uint32_t h = 0; h < halo[q].second; ++h) to[at[slot(halo[q].first[h])]++] = q << 16 | h;
+    for (size_t k = n; k; --k) at[k] = at[k - 1];           // the ends became the next ones' starts
+    at[0] = 0;
+    for (size_t k = 0; k < n; ++k) {
         uint32_t *pc = push + 2 * k;
-        pc[0] = to[k].size() > 0 ? to[k][0] : kNoPush;
-        pc[1] = to[k].size() == 2 ? to[k][1] : kNoPush;
-        if (to[k].size() > 2) {
+        const uint32_t first = at[k], count = at[k + 1] - first;
+        pc[0] = count > 0 ? to[first] : kNoPush;
+        pc[1] = count == 2 ? to[first + 1] : kNoPush;
+        if (count > 2) {
             pc[1] = kMorePush | (uint32_t)more.size();
-            more.push_back((uint32_t)to[k].size() - 1);
-            more.insert(more.end(), to[k].begin() + 1, to[k].end());
+            more.push_back(count - 1);
+            more.insert(more.end(), to.begin() + first + 1, to.begin() + first + count);
         }
     }
 }

@@ -498,13 +498,12 @@ bool choose_box_width(titan_sim *sim) {
 // each CTA's rows are short enough that a few SMs beat a whole-GPU launch per
 // step; else one launch per step.  Rewrites the neighbour codes if the plan
 // changed.
-cudaError_t resolve_exec(titan_sim *sim) {
+cudaError_t plan_exec(titan_sim *sim, bool sine) {
     sim->persistent = false;
     if (sim->accumulate != TITAN_ACCUM_CSR || sim->exec_req == TITAN_EXEC_LAUNCH) return cudaSuccess;
     titan::PersistPlan plan;
     std::vector<uint16_t> slot;
     std::vector<uint32_t> halo;
-    const bool sine = sim->c.act_mode != 2;
     if (!titan::plan_persistent(sim->n_dev, sim->sell.slice_off, sim->sell.nbr, sim->has_c, sim->has_act,
                                 kPersistSmemLimit, plan, slot, halo,
                                 titan::persist_aim(sim->n, sim->has_c, sim->has_act, sine)))
@@ -546,6 +545,18 @@ cudaError_t resolve_exec(titan_sim *sim) {
     sim->plan = plan;
     sim->persistent = true;
     return cudaSuccess;
+}
+
+cudaError_t resolve_exec(titan_sim *sim) {
+    // All that the plan depends on besides the layout, whose springs and masses stay where they
+    // are while it lives: setting other values of the same actuation changes nothing here.
+    const bool sine = sim->c.act_mode != 2;
+    const int plan_of = (sim->has_c ? 1 : 0) | (sim->has_act ? 2 : 0) | (sine ? 4 : 0);
+    if (sim->plan_of == plan_of) return cudaSuccess;
+    sim->plan_of = -1;
+    const cudaError_t e = plan_exec(sim, sine);
+    if (e == cudaSuccess) sim->plan_of = plan_of;
+    return e;
 }
 
 // After per-spring damping or actuation arrays appear (larger SELL entries).

@@ -56,6 +56,7 @@ struct SimCore {
     uint32_t *d_phalo = nullptr;          // persistent kernel: halo list
     size_t phalo_cap = 0;
     bool persist_rows = false;            // the plan runs in the row-register form
+    int plan_of = -1;                     // what this layout was last planned for (resolve_exec), -1: not yet
     uint2 *d_ppush = nullptr;             // its copy lists, two words per device mass
     uint32_t *d_ppush_more = nullptr;
     size_t ppush_cap = 0, ppush_more_cap = 0;

@@ -116,3 +116,25 @@ def test_step_form(shape, form):
             assert (sim.csr_kernel, sim.step_form) == (variant, form)
     with T.Sim(sy, exec_mode=T.EXEC_LAUNCH, kernel_variant=1) as sim:
         assert sim.step_form == T.FORM_PLAIN
+
+
+@pytest.mark.parametrize("n", [100, 600])
+def test_actuation_set_again_and_again(n):
+    """Every value set is stepped with, also where the plan of the launch stays as it is."""
+    sy = _ring(n)
+    sy.act_amp = None
+    ids, rng = np.arange(sy.n_springs), np.random.default_rng(n)
+    with T.Sim(sy, exec_mode=T.EXEC_PERSISTENT) as sim, T.Sim(sy, exec_mode=T.EXEC_LAUNCH, kernel_variant=1) as ref:
+        for k in range(6):
+            amp, phase = rng.uniform(0, 0.2, sy.n_springs), rng.uniform(0, 6, sy.n_springs)
+            for s in (sim, ref):
+                if k in (2, 3):
+                    T.titan_set_worm_actuation(s.handle, ids, amp, phase / 7, 20.0, 0.01)
+                else:
+                    T.titan_set_actuation(s.handle, ids, amp, phase, 2.0 + k)
+                if k == 4:
+                    T.titan_set_spring_params(s.handle, ids[:3], damping=np.array([0.5, 0.7, 1.3]))
+                s.step(7)
+            x, y = sim.snapshot(), ref.snapshot()
+            assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1]), k
+        assert sim.exec_mode == T.EXEC_PERSISTENT and sim.step_form == T.FORM_PLAIN        # per-spring damping now
